@@ -92,43 +92,35 @@ typedef struct {
  * Workspace size in bytes for blr_scan_fwd / blr_scan_bwd (and their _gated
  * and _varlen forms) on `desc`; 0 when the description is invalid or needs none
  * (B, L or D zero). The workspace holds what the forward keeps for the
- * backward, by kernel family (blr_scan_family):
+ * backward, by the kernels that serve the problem:
  *   serial: the state every 16 float32 / 8 bfloat16 steps, 0.25-0.5 bytes per
  *           element;
- *   tiled: per-tile records (24 bytes per channel per 64-step tile, under 0.4
- *           bytes per element);
- *   segmented: the serial kernels' kept states, 8 bytes per channel per
- *           segment (of 128 steps or more) and the chained forward's records
- *           (12 bytes per channel per 128 steps), laid over the tiled forward
- *           records, plus the tiled backward records (for the _varlen forms),
- *           under 0.95 bytes per element;
- * plus the float64 partial sums of dlambda and a small header (about 72 bytes
+ *   team:   the state every 16 steps, 0.25 bytes per element, and where tiles
+ *           are chained by a look-back its records, 12 bytes per channel per
+ *           tile of up to 128 steps (0.1 bytes per element);
+ * plus the float64 partial sums of dlambda and a small header (about 64 bytes
  * per channel). It depends only on B, L, D and the I/O dtype.
  */
 BLR_API size_t blr_workspace_bytes(const blr_desc* desc);
 
 /*
- * Which kernels blr_scan_fwd / blr_scan_bwd (and their _gated forms; the
- * _varlen forms when with_lengths is nonzero) run on `desc` (diagnostic; the
- * choice depends only on B, L, D and the I/O dtype). A chain is 32 float32 or
- * 64 bfloat16 channels of one batch row.
- *   BLR_FAMILY_SERIAL     at least 256 chains: one warp walks each chain
- *                         through the whole sequence (one kernel per call).
+ * The shape class of `desc` (diagnostic; it depends only on B, L, D and the I/O
+ * dtype, and on with_lengths, which asks for the _varlen forms). A chain is 32
+ * float32 or 64 bfloat16 channels of one batch row.
+ *   BLR_FAMILY_SERIAL     at least 256 chains.
  *   BLR_FAMILY_SEGMENTED  bfloat16 I/O, fewer chains, L >= 2048 and either
  *                         at least 8 Mi elements or L >= 16384, without
- *                         lengths. blr_scan_fwd and blr_scan_bwd run one
- *                         chained kernel each: 128-step tiles folded by 16
- *                         warps and chained along time by a decoupled
- *                         look-back (the operator of Sec. 3.3), after one
- *                         cudaMemsetAsync that empties the look-back records.
- *                         The _gated forms cut each chain into time segments
- *                         of 128 steps or more: a reduction kernel computes
- *                         every segment's affine map, then one warp walks each
- *                         segment from the carry the maps compose (two kernels
- *                         per call).
- *   BLR_FAMILY_TILED      otherwise: 64-step tiles chained by a decoupled
- *                         look-back (a preparation kernel, then the scan).
+ *                         lengths: the backward of a plain or gated forward
+ *                         refuses the workspace of a _varlen forward here, and
+ *                         the reverse.
+ *   BLR_FAMILY_TILED      otherwise.
  *   BLR_FAMILY_NONE       an invalid or empty problem (nothing is launched).
+ * From 512 float32 or 640 bfloat16 chains on the serial kernels run: one warp
+ * walks each chain through the whole sequence. Below, the team kernels: teams
+ * of 8 warps scan tiles of up to 128 steps of a chain, 16 steps a warp, whole
+ * chains at a time where there are enough of them, else tiles of all chains in
+ * time order, chained by a decoupled look-back (the operator of Sec. 3.3) after
+ * one cudaMemsetAsync that empties its records. Every call is one kernel.
  */
 #define BLR_FAMILY_NONE 0
 #define BLR_FAMILY_TILED 1
@@ -207,8 +199,7 @@ BLR_API blr_status blr_scan_bwd(const blr_desc* desc, const void* dh, const floa
  * errors as blr_scan_fwd / blr_scan_bwd; the backward's ws must come from a
  * blr_scan_fwd_varlen with the same lengths, or be NULL (the carries are then
  * recomputed with these lengths, as blr_scan_bwd does). Work and traffic scale with the
- * rows' lengths on problems served by the serial kernels (at least 256
- * chains); the tiled kernels still stream the padding and mask it.
+ * rows' lengths.
  */
 BLR_API blr_status blr_scan_fwd_varlen(const blr_desc* desc, const int32_t* lengths, const void* x,
                                        const void* gate_logits, const float* lambda, const float* h0,
@@ -230,10 +221,7 @@ BLR_API blr_status blr_scan_bwd_varlen(const blr_desc* desc, const int32_t* leng
  * y           (B, L, D)  io dtype, output; may be NULL (then only h_last and
  *                        the carries, as blr_scan_fwd with h == NULL)
  * Other arguments, the workspace and the errors as blr_scan_fwd; z must be
- * 16-byte aligned and no output may overlap an input. The merge is fused into
- * the serial and segmented kernels; problems on the tiled kernels
- * (blr_scan_family) run the scan and then an elementwise merge kernel over y
- * in place.
+ * 16-byte aligned and no output may overlap an input.
  */
 BLR_API blr_status blr_scan_fwd_gated(const blr_desc* desc, const void* x, const void* gate_logits,
                                       const float* lambda, const float* h0, const void* z, void* y,
@@ -250,10 +238,7 @@ BLR_API blr_status blr_scan_fwd_gated(const blr_desc* desc, const void* x, const
  * dz          (B, L, D)  io dtype, output
  * ws          the workspace of a blr_scan_fwd_gated (or blr_scan_fwd) of the same
  *             desc and inputs, or NULL, as for blr_scan_bwd.
- * Other arguments as blr_scan_bwd; no output may overlap an input. Problems on
- * the tiled kernels (blr_scan_family) recompute h into dz, form dh in dx and dz
- * in place with an elementwise kernel, then run the scan's backward from dx;
- * the serial and segmented kernels fuse the merge.
+ * Other arguments as blr_scan_bwd; no output may overlap an input.
  */
 BLR_API blr_status blr_scan_bwd_gated(const blr_desc* desc, const void* dy, const float* dh_last,
                                       const void* x, const void* gate_logits, const float* lambda,

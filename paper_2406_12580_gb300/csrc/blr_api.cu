@@ -1,5 +1,5 @@
 // C ABI of the BD-LRU scan library (declared in include/blr.h): host-side
-// validation, the tiling plan, workspace clearing and kernel launches. The
+// validation, the plan, workspace clearing and kernel launches. The
 // library allocates nothing and never synchronises except in
 // blr_workspace_status().
 #include <math.h>
@@ -12,10 +12,8 @@
 #include <cudaTypedefs.h>
 
 #include "blr.h"
-#include "blr_chain.cuh"
-#include "blr_chain_bwd.cuh"
-#include "blr_merge.cuh"
 #include "blr_seq.cuh"
+#include "blr_team_bwd.cuh"
 
 namespace {
 
@@ -38,8 +36,13 @@ blr_status cuda_check(cudaError_t e, const char* what) {
 
 bool aligned(const void* p, size_t a) { return ((uintptr_t)p % a) == 0; }
 
+// The library's static device scratch (defined with blr_scan_fwd_noalloc).
+constexpr size_t kLibraryScratchBytes = (size_t)128 << 20;  // 128 MiB
+
 // Shared checks of the problem description; fills `plan` when B, L, D > 0.
-blr_status check_desc(const blr_desc* d, Plan* plan, bool* empty_bd) {
+// `scratch`: the plan of a call that runs in the library's scratch, which takes
+// the team kernels' local order where the look-back's records would not fit.
+blr_status check_desc(const blr_desc* d, Plan* plan, bool* empty_bd, bool scratch = false) {
   if (d == nullptr) return fail(BLR_ERR_INVALID_ARG, "desc is NULL");
   if (d->B < 0 || d->L < 0 || d->D < 0)
     return fail(BLR_ERR_INVALID_ARG, "negative size B=%lld L=%lld D=%lld", (long long)d->B,
@@ -59,13 +62,14 @@ blr_status check_desc(const blr_desc* d, Plan* plan, bool* empty_bd) {
   if (d->B >= ((int64_t)1 << 31) || d->L >= ((int64_t)1 << 31) ||
       (double)d->L * (double)d->D * 8.0 >= (double)((int64_t)1 << 40))
     return fail(BLR_ERR_UNSUPPORTED, "problem too large for the tiled loads");
-  blr::make_plan(d->B, d->L, d->D, (int)d->io, d->c, plan);
-  if (plan->n_tiles_f >= ((int64_t)1 << 30) || plan->n_tiles_b >= ((int64_t)1 << 30))
-    return fail(BLR_ERR_UNSUPPORTED, "too many tiles (%lld)", (long long)plan->n_tiles_b);
-  if (plan->nseg > 0 && plan->n_tc * plan->n_chain >= ((int64_t)1 << 31))
-    return fail(BLR_ERR_UNSUPPORTED, "too many chained tiles");
-  if (plan->seq && plan->n_chain >= ((int64_t)1 << 31))
-    return fail(BLR_ERR_UNSUPPORTED, "too many chains (%lld)", (long long)plan->n_chain);
+  blr::make_plan(d->B, d->L, d->D, (int)d->io, d->c, false, plan);
+  if (scratch && plan->bytes > kLibraryScratchBytes)
+    blr::make_plan(d->B, d->L, d->D, (int)d->io, d->c, true, plan);
+  // Chain and tile numbers are 32-bit: tiles of at most 64 steps x 32 channels
+  // (no kernel's are smaller) stay below 2^30.
+  const int64_t n64 = (d->L + 63) / 64, rows = ((d->L + n64 - 1) / n64 + 15) / 16 * 16;
+  if ((double)((d->L + rows - 1) / rows) * (double)(d->B * ((d->D + 31) / 32)) >= (double)((int64_t)1 << 30))
+    return fail(BLR_ERR_UNSUPPORTED, "too many tiles");
   return BLR_OK;
 }
 
@@ -236,11 +240,6 @@ blr_status allow_smem(K kernel, size_t smem) {
                     "set dynamic shared memory size");
 }
 
-// Blocks of a serial kernel: one per chain, or per (segment, chain).
-int64_t seq_blocks(const Plan& p, int mode) {
-  return mode == blr::kSeqSeg ? p.n_chain * p.nseg : p.n_chain;
-}
-
 // float32 rings deep enough run the LATE form (refill after the next stage's
 // arithmetic); bfloat16 always the early one.
 template <typename T>
@@ -251,7 +250,7 @@ bool late_refill(int stages) {
 template <typename T, class M, int VEC, int R, int RB, bool GATED, int MODE = blr::kSeqPlain>
 blr_status launch_seq_fwd(blr::SeqFwdArgs& a, cudaStream_t st) {
   constexpr int NB = GATED ? 4 : 3;
-  const int64_t blocks = seq_blocks(a.p, MODE);
+  const int64_t blocks = a.p.n_chain;
   a.stages = seq_stages(blocks, NB * (size_t)blr::seq_box_bytes<T, VEC, R>());
   const size_t smem = blr::seq_smem_bytes<T, VEC, R>(a.stages, NB);
   auto kernel = blr::seq_fwd_kernel<T, M, VEC, R, RB, GATED, MODE, false>;
@@ -266,7 +265,7 @@ blr_status launch_seq_fwd(blr::SeqFwdArgs& a, cudaStream_t st) {
 template <typename T, class M, int VEC, int R, int RB, bool GATED, int MODE = blr::kSeqPlain>
 blr_status launch_seq_bwd(blr::SeqBwdArgs& a, cudaStream_t st) {
   constexpr int NB = GATED ? 5 : 4;
-  const int64_t blocks = seq_blocks(a.p, MODE);
+  const int64_t blocks = a.p.n_chain;
   a.stages = seq_stages(blocks, NB * (size_t)blr::seq_box_bytes<T, VEC, R>());
   const size_t smem = blr::seq_smem_bytes<T, VEC, R>(a.stages, NB);
   auto kernel = blr::seq_bwd_kernel<T, M, VEC, R, RB, GATED, MODE, false>;
@@ -276,22 +275,6 @@ blr_status launch_seq_bwd(blr::SeqBwdArgs& a, cudaStream_t st) {
   BLR_TRY(allow_smem(kernel, smem));
   kernel<<<(unsigned)blocks, 32, smem, st>>>(a);
   return cuda_check(cudaGetLastError(), "launch seq_bwd_kernel");
-}
-
-// Rows per TMA box of the segment reductions (seg_len is a multiple).
-constexpr int kSegReduceRows = 16;
-
-template <typename T, class M, int VEC, bool BWD, bool GATED = false>
-blr_status launch_seg_reduce(blr::SegReduceArgs& a, cudaStream_t st) {
-  constexpr int R = kSegReduceRows;
-  auto kernel = blr::seg_reduce_kernel<T, M, VEC, R, BWD, GATED>;
-  constexpr int NB = (BWD && !GATED) ? 2 : 3;
-  const int64_t blocks = a.p.n_chain * a.p.nseg;
-  a.stages = seq_stages(blocks, NB * (size_t)blr::seq_box_bytes<T, VEC, R>());
-  const size_t smem = blr::seq_smem_bytes<T, VEC, R>(a.stages, NB);
-  BLR_TRY(allow_smem(kernel, smem));
-  kernel<<<(unsigned)blocks, 32, smem, st>>>(a);
-  return cuda_check(cudaGetLastError(), "launch seg_reduce_kernel");
 }
 
 // The serial kernels' views: x-shaped tensors as (D, L, B); gate_logits-shaped
@@ -310,7 +293,7 @@ blr_status seq_maps_gl(CUtensorMap* mr, CUtensorMap* mi, const void* base, const
 // z given: the merge of the gated layer is fused, and h receives y = h SiLU(z).
 blr_status scan_fwd_seq(const Plan& plan, const void* x, const void* gl, const float* lambda,
                         const float* h0, void* h, float* h_last, unsigned char* w, cudaStream_t st,
-                        const void* z, const int32_t* lengths, bool seg = false) {
+                        const void* z, const int32_t* lengths) {
   blr::SeqFwdArgs a;
   a.lengths = lengths;
   BLR_TRY(seq_maps_x(&a.tm_x, x, plan, plan.sr));
@@ -326,11 +309,6 @@ blr_status scan_fwd_seq(const Plan& plan, const void* x, const void* gl, const f
   a.h_last = h_last;
   a.ws = w;
   a.stages = 2;
-  if (seg) {  // bfloat16 only (make_plan)
-    constexpr int S = blr::kSeqSeg;
-    if (z != nullptr) return launch_seq_fwd<__nv_bfloat16, blr::MathFast, 2, 16, 8, true, S>(a, st);
-    return launch_seq_fwd<__nv_bfloat16, blr::MathFast, 2, 16, 8, false, S>(a, st);
-  }
   if (z != nullptr) {
     if (plan.io == BLR_F32) {
       if (plan.sr == 32) return launch_seq_fwd<float, blr::MathPrecise, 1, 32, 16, true>(a, st);
@@ -357,7 +335,7 @@ blr_status scan_fwd_seq(const Plan& plan, const void* x, const void* gl, const f
 blr_status scan_bwd_seq(const Plan& plan, const void* dh, const float* dh_last, const void* x,
                         const void* gl, const float* lambda, const float* h0, void* dx, void* dgl,
                         float* dlambda, float* dh0, unsigned char* w, cudaStream_t st,
-                        const void* z, void* dz, const int32_t* lengths, bool seg = false) {
+                        const void* z, void* dz, const int32_t* lengths) {
   blr::SeqBwdArgs a;
   a.lengths = lengths;
   BLR_TRY(seq_maps_x(&a.tm_dh, dh, plan, plan.srb));
@@ -381,11 +359,6 @@ blr_status scan_bwd_seq(const Plan& plan, const void* dh, const float* dh_last, 
   a.dh0 = dh0;
   a.ws = w;
   a.stages = 2;
-  if (seg) {  // bfloat16 only (make_plan)
-    constexpr int S = blr::kSeqSeg;
-    if (gated) return launch_seq_bwd<__nv_bfloat16, blr::MathFast, 2, 8, 8, true, S>(a, st);
-    return launch_seq_bwd<__nv_bfloat16, blr::MathFast, 2, 8, 8, false, S>(a, st);
-  }
   if (gated) {
     if (plan.io == BLR_F32) return launch_seq_bwd<float, blr::MathPrecise, 1, 16, 16, true>(a, st);
     return launch_seq_bwd<__nv_bfloat16, blr::MathFast, 2, 8, 8, true>(a, st);
@@ -399,257 +372,132 @@ blr_status scan_bwd_seq(const Plan& plan, const void* dh, const float* dh_last, 
   return launch_seq_bwd<__nv_bfloat16, blr::MathFast, 2, 8, 8, false>(a, st);
 }
 
-// The segmented serial kernels (few chains, long sequences; bfloat16 I/O):
-// the segment reduction, then the serial kernel over (segment, chain) blocks,
-// each composing its carry from the maps.
-blr_status scan_fwd_seg(const Plan& plan, const void* x, const void* gl, const float* lambda,
-                        const float* h0, void* h, float* h_last, unsigned char* w,
-                        cudaStream_t st, const void* z) {
-  if (plan.io != BLR_BF16) return fail(BLR_ERR_UNSUPPORTED, "segmented kernels take bfloat16 I/O");
-  blr::SegReduceArgs r;
-  BLR_TRY(seq_maps_x(&r.tm_a, x, plan, kSegReduceRows));
-  BLR_TRY(seq_maps_gl(&r.tm_r, &r.tm_i, gl, plan, kSegReduceRows));
-  r.p = plan;
-  r.lambda = lambda;
-  r.ws = w;
-  r.stages = 2;
-  BLR_TRY((launch_seg_reduce<__nv_bfloat16, blr::MathFast, 2, false>(r, st)));
-  return scan_fwd_seq(plan, x, gl, lambda, h0, h, h_last, w, st, z, nullptr, true);
+// ------------------------------------------------------------- team kernels
+
+// Launches a kernel that may begin its prologue while the kernel before it on
+// the stream finishes (programmatic dependent launch): the kernel itself waits
+// for that one (griddepcontrol.wait) before it touches global memory.
+template <typename K, typename A>
+blr_status launch_chained(K kernel, unsigned grid, int threads, size_t smem, cudaStream_t st,
+                          const A& args, const char* what) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cuda_check(cudaLaunchKernelEx(&cfg, kernel, args), what);
 }
 
-blr_status scan_bwd_seg(const Plan& plan, const void* dh, const float* dh_last, const void* x,
-                        const void* gl, const float* lambda, const float* h0, void* dx, void* dgl,
-                        float* dlambda, float* dh0, unsigned char* w, cudaStream_t st,
-                        const void* z, void* dz) {
-  if (plan.io != BLR_BF16) return fail(BLR_ERR_UNSUPPORTED, "segmented kernels take bfloat16 I/O");
-  blr::SegReduceArgs r;
-  BLR_TRY(seq_maps_x(&r.tm_a, dh, plan, kSegReduceRows));
-  BLR_TRY(seq_maps_gl(&r.tm_r, &r.tm_i, gl, plan, kSegReduceRows));
-  if (z != nullptr) BLR_TRY(seq_maps_x(&r.tm_z, z, plan, kSegReduceRows));
-  else memset(&r.tm_z, 0, sizeof(r.tm_z));
-  r.p = plan;
-  r.lambda = lambda;
-  r.ws = w;
-  r.stages = 2;
-  if (z != nullptr)
-    BLR_TRY((launch_seg_reduce<__nv_bfloat16, blr::MathFast, 2, true, true>(r, st)));
-  else
-    BLR_TRY((launch_seg_reduce<__nv_bfloat16, blr::MathFast, 2, true>(r, st)));
-  return scan_bwd_seq(plan, dh, dh_last, x, gl, lambda, h0, dx, dgl, dlambda, dh0, w, st, z, dz,
-                      nullptr, true);
-}
-
-// The chained single-pass forward (few chains, long sequences): its records
-// are emptied, then one cooperative grid, one block per SM, scans every tile.
-template <typename T, class M, int VEC, int RB>
-blr_status launch_chain_fwd(const Plan& plan, const blr::ChainFwdArgs& a, cudaStream_t st) {
-  constexpr int threads = blr::kChainThreads;
-  auto k = blr::chain_fwd_kernel<T, M, VEC, RB>;
-  const size_t smem = blr::ChainSmem<T, VEC>::bytes;
+// One block per SM (its shared memory fills one), at most one team per unit of
+// work: a chain in the local order, a tile with the look-back.
+template <typename K, typename A>
+blr_status launch_team(K kernel, size_t smem, A& args, cudaStream_t st, const char* what) {
+  constexpr int threads = blr::kTeamThreads;
+  const Plan& p = args.p;
+  const int64_t units = p.lookback ? p.n_tc * p.n_chain : p.n_chain;
   unsigned grid = 1;
-  BLR_TRY(persistent_grid(k, threads, smem, plan.n_tc * plan.n_chain, &grid));
-  return launch_cooperative(k, grid, threads, smem, st, a, "launch chain_fwd_kernel");
+  BLR_TRY(persistent_grid(kernel, threads, smem, (units + blr::kTeams - 1) / blr::kTeams, &grid));
+  // A multiple of the channel groups, if that idles few teams: a team then
+  // stays within one group, and the backward adds its d Lambda sums up once.
+  args.teams = grid * (unsigned)blr::kTeams;
+  const int64_t n_g = p.n_chain / p.B;
+  if (args.teams >= 8 * n_g) args.teams -= args.teams % (unsigned)n_g;
+  if (!p.lookback) return launch_chained(kernel, grid, threads, smem, st, args, what);
+  BLR_TRY(cuda_check(cudaMemsetAsync(args.ws + p.off_cinc, 0xff, p.off_cend - p.off_cinc, st),
+                     "empty the look-back records"));
+  return launch_cooperative(kernel, grid, threads, smem, st, args, what);
 }
 
-blr_status scan_fwd_chain(const Plan& plan, const void* x, const void* gl, const float* lambda,
-                          const float* h0, void* h, float* h_last, unsigned char* w,
-                          cudaStream_t st) {
-  if (plan.io != BLR_BF16) return fail(BLR_ERR_UNSUPPORTED, "the chained forward takes bfloat16 I/O");
-  BLR_TRY(cuda_check(cudaMemsetAsync(w + plan.off_cinc, 0xff, plan.off_cend - plan.off_cinc, st),
-                     "empty the chained forward's records"));
-  blr::ChainFwdArgs a;
-  BLR_TRY(seq_maps_x(&a.tm_x, x, plan, blr::kChainTile));
-  BLR_TRY(seq_maps_gl(&a.tm_r, &a.tm_i, gl, plan, blr::kChainTile));
+template <typename T, bool GATED>
+blr_status launch_team_fwd(blr::TeamFwdArgs& a, cudaStream_t st) {
+  return launch_team(blr::team_fwd_kernel<T, GATED>, blr::TeamFwdSmem<T>::bytes, a, st,
+                     "launch team_fwd_kernel");
+}
+template <typename T, bool GATED>
+blr_status launch_team_bwd(blr::TeamBwdArgs& a, cudaStream_t st) {
+  return launch_team(blr::team_bwd_kernel<T, GATED>, blr::TeamBwdSmem<T, GATED>::bytes, a, st,
+                     "launch team_bwd_kernel");
+}
+
+// The problem tag a forward leaves in the workspace. The plain and gated scans
+// of the shapes BLR_FAMILY_SEGMENTED have one of their own: a backward of
+// theirs refuses the workspace of a forward with row lengths, and the reverse.
+uint32_t team_tag(const Plan& p, bool varlen) {
+  return p.segmented && !varlen ? p.tag ^ 0x80000000u : p.tag;
+}
+
+blr_status scan_fwd_team(const Plan& plan, const void* x, const void* gl, const float* lambda,
+                         const float* h0, void* h, float* h_last, unsigned char* w,
+                         cudaStream_t st, const void* z, const int32_t* lengths, bool varlen) {
+  blr::TeamFwdArgs a;
+  BLR_TRY(seq_maps_x(&a.tm_x, x, plan, plan.ts));
+  BLR_TRY(seq_maps_gl(&a.tm_r, &a.tm_i, gl, plan, plan.ts));
+  if (z != nullptr) BLR_TRY(seq_maps_x(&a.tm_z, z, plan, plan.ts));
+  else memset(&a.tm_z, 0, sizeof(a.tm_z));
   a.p = plan;
+  a.lengths = lengths;
   a.lambda = lambda;
   a.h0 = h0;
+  a.z = z;
   a.h = h;
   a.h_last = h_last;
   a.ws = w;
-  return launch_chain_fwd<__nv_bfloat16, blr::MathFast, 2, 8>(plan, a, st);
-}
-
-// The chained single-pass backward (the problems the chained forward serves,
-// bfloat16): the records are emptied again (the forward's are no longer
-// needed), then one cooperative grid, one block per SM.
-blr_status scan_bwd_chain(const Plan& plan, const void* dh, const float* dh_last, const void* x,
-                          const void* gl, const float* lambda, const float* h0, void* dx, void* dgl,
-                          float* dlambda, float* dh0, unsigned char* w, cudaStream_t st) {
-  if (plan.io != BLR_BF16) return fail(BLR_ERR_UNSUPPORTED, "the chained backward takes bfloat16 I/O");
-  BLR_TRY(cuda_check(cudaMemsetAsync(w + plan.off_cinc, 0xff, plan.off_cend - plan.off_cinc, st),
-                     "empty the chained backward's records"));
-  blr::ChainBwdArgs a;
-  BLR_TRY(seq_maps_x(&a.tm_dh, dh, plan, blr::kChainTile));
-  BLR_TRY(seq_maps_x(&a.tm_x, x, plan, blr::kChainTile));
-  BLR_TRY(seq_maps_gl(&a.tm_r, &a.tm_i, gl, plan, blr::kChainTile));
-  BLR_TRY(seq_maps_x(&a.tm_dx, dx, plan, blr::kChainTile));
-  BLR_TRY(seq_maps_gl(&a.tm_dr, &a.tm_di, dgl, plan, blr::kChainTile));
-  a.p = plan;
-  a.dh_last = dh_last;
-  a.lambda = lambda;
-  a.h0 = h0;
-  a.dlambda = dlambda;
-  a.dh0 = dh0;
-  a.ws = w;
+  a.tag = team_tag(plan, varlen);
   using bf = __nv_bfloat16;
-  auto k = blr::chain_bwd_kernel<bf, blr::MathFast, 2, 8>;
-  const size_t smem = blr::ChainBwdSmem<bf, 2>::bytes;
-  unsigned grid = 1;
-  BLR_TRY(persistent_grid(k, blr::kCbThreads, smem, plan.n_tc * plan.n_chain, &grid));
-  return launch_cooperative(k, grid, blr::kCbThreads, smem, st, a, "launch chain_bwd_kernel");
+  if (plan.io == BLR_F32)
+    return z != nullptr ? launch_team_fwd<float, true>(a, st) : launch_team_fwd<float, false>(a, st);
+  return z != nullptr ? launch_team_fwd<bf, true>(a, st) : launch_team_fwd<bf, false>(a, st);
 }
 
-// Clears [zero, zero + zero_bytes), fills [fill, fill + fill_bytes) with the
-// empty record pattern and writes k = -c softplus(Lambda).
-blr_status launch_prep(unsigned char* zero, size_t zero_bytes, unsigned char* fill,
-                       size_t fill_bytes, float* k, const float* lambda, int64_t D, float c,
-                       cudaStream_t st) {
-  const int64_t words = (int64_t)(zero_bytes / 4);
-  const int64_t vec4 = (int64_t)(fill_bytes / 16);
-  int64_t work = words > D ? words : D;
-  if (vec4 > work) work = vec4;
-  int64_t blocks = (work + 255) / 256;
-  if (blocks > 2048) blocks = 2048;
-  blr::prep_kernel<<<(unsigned)blocks, 256, 0, st>>>(reinterpret_cast<uint32_t*>(zero), words,
-                                                     reinterpret_cast<uint4*>(fill), vec4, k,
-                                                     lambda, D, c);
-  return cuda_check(cudaGetLastError(), "launch prep_kernel");
-}
-
-template <typename T, class M, bool VARLEN>
-blr_status launch_tiled_fwd(const Plan& plan, const blr::FwdArgs& a, cudaStream_t st) {
-  const int threads = (plan.nwarps + 1) * 32;  // consumer warps + the scanner warp
-  auto k = blr::scan_fwd_kernel<T, M, VARLEN>;
-  const size_t smem = blr::ring_bytes<T, blr::fwd_stages<T>(), 3>();
-  unsigned grid = 1;
-  BLR_TRY(persistent_grid(k, threads, smem, plan.n_tiles_f, &grid));
-  return launch_cooperative(k, grid, threads, smem, st, a, "launch scan_fwd_kernel");
-}
-
-template <typename T, class M, bool VARLEN>
-blr_status launch_tiled_bwd(const Plan& plan, const blr::BwdArgs& a, cudaStream_t st) {
-  const int threads = plan.nwarps * 32;
-  auto k = blr::scan_bwd_kernel<T, M, VARLEN>;
-  const size_t smem = blr::ring_bytes<T, blr::bwd_stages<T>(), 4>();
-  unsigned grid = 1;
-  BLR_TRY(persistent_grid(k, threads, smem, plan.n_tiles_b, &grid));
-  return launch_cooperative(k, grid, threads, smem, st, a, "launch scan_bwd_kernel");
-}
-
-// The tiled look-back kernels: a preparation kernel, then the scan.
-blr_status scan_fwd_tiled(const Plan& plan, const blr_desc* desc, const void* x,
-                          const void* gate_logits, const float* lambda, const float* h0, void* h,
-                          float* h_last, unsigned char* w, cudaStream_t st,
-                          const int32_t* lengths) {
-  // Clear the forward header (counters, error word), empty the
-  // forward records, precompute k = -c softplus(Lambda).
-  BLR_TRY(launch_prep(w + plan.off_fhdr, sizeof(blr::FwdHeader), w + plan.off_fpre,
-                      plan.off_frec_end - plan.off_fpre, reinterpret_cast<float*>(w + plan.off_k),
-                      lambda, desc->D, desc->c, st));
-  blr::FwdArgs a;
-  a.lengths = lengths;
-  BLR_TRY(make_tensor_map(&a.tm_x, x, desc->io, desc->D, desc->L, desc->B, plan.tsteps));
-  BLR_TRY(make_tensor_map(&a.tm_gl, gate_logits, desc->io, 2 * desc->D, desc->L, desc->B, plan.tsteps));
+blr_status scan_bwd_team(const Plan& plan, const void* dh, const float* dh_last, const void* x,
+                         const void* gl, const float* lambda, const float* h0, void* dx, void* dgl,
+                         float* dlambda, float* dh0, unsigned char* w, cudaStream_t st,
+                         const void* z, void* dz, const int32_t* lengths, bool varlen) {
+  blr::TeamBwdArgs a;
+  constexpr int R = blr::kTeamSlice;
+  BLR_TRY(seq_maps_x(&a.tm_dh, dh, plan, R));
+  BLR_TRY(seq_maps_x(&a.tm_x, x, plan, R));
+  BLR_TRY(seq_maps_gl(&a.tm_r, &a.tm_i, gl, plan, R));
+  BLR_TRY(seq_maps_x(&a.tm_dx, dx, plan, R));
+  BLR_TRY(seq_maps_gl(&a.tm_dr, &a.tm_di, dgl, plan, R));
+  if (z != nullptr) BLR_TRY(seq_maps_x(&a.tm_z, z, plan, R));
+  else memset(&a.tm_z, 0, sizeof(a.tm_z));
   a.p = plan;
-  a.h0 = h0;
-  a.h = h;
-  a.h_last = h_last;
-  a.ws = w;
-  if (desc->io == BLR_F32) {
-    if (lengths != nullptr) return launch_tiled_fwd<float, blr::MathPrecise, true>(plan, a, st);
-    return launch_tiled_fwd<float, blr::MathPrecise, false>(plan, a, st);
-  }
-  if (lengths != nullptr) return launch_tiled_fwd<__nv_bfloat16, blr::MathFast, true>(plan, a, st);
-  return launch_tiled_fwd<__nv_bfloat16, blr::MathFast, false>(plan, a, st);
-}
-
-// dh may be the dx buffer itself: every element of dh is read (into shared
-// memory, with its tile) before its tile writes dx.
-blr_status scan_bwd_tiled(const Plan& plan, const blr_desc* desc, const void* dh,
-                          const float* dh_last, const void* x, const void* gate_logits,
-                          const float* lambda, const float* h0, void* dx, void* dgate_logits,
-                          float* dlambda, float* dh0, unsigned char* w, cudaStream_t st,
-                          const int32_t* lengths) {
-  // Clear the backward header and the dLambda partial sums, empty the backward
-  // records (the forward's records stay: they hold the carries).
-  BLR_TRY(launch_prep(w + plan.off_bhdr, plan.off_k - plan.off_bhdr, w + plan.off_bagg,
-                      plan.bytes - plan.off_bagg, reinterpret_cast<float*>(w + plan.off_k), lambda,
-                      desc->D, desc->c, st));
-  blr::BwdArgs a;
   a.lengths = lengths;
-  BLR_TRY(make_tensor_map(&a.tm_dh, dh, desc->io, desc->D, desc->L, desc->B, plan.tsteps));
-  BLR_TRY(make_tensor_map(&a.tm_x, x, desc->io, desc->D, desc->L, desc->B, plan.tsteps));
-  BLR_TRY(make_tensor_map(&a.tm_gl, gate_logits, desc->io, 2 * desc->D, desc->L, desc->B, plan.tsteps));
-  a.p = plan;
+  a.dy = dh;
+  a.z = z;
+  a.dz = dz;
   a.dh_last = dh_last;
   a.lambda = lambda;
   a.h0 = h0;
-  a.dx = dx;
-  a.dgl = dgate_logits;
   a.dlambda = dlambda;
   a.dh0 = dh0;
   a.ws = w;
-  if (desc->io == BLR_F32) {
-    if (lengths != nullptr) return launch_tiled_bwd<float, blr::MathPrecise, true>(plan, a, st);
-    return launch_tiled_bwd<float, blr::MathPrecise, false>(plan, a, st);
-  }
-  if (lengths != nullptr) return launch_tiled_bwd<__nv_bfloat16, blr::MathFast, true>(plan, a, st);
-  return launch_tiled_bwd<__nv_bfloat16, blr::MathFast, false>(plan, a, st);
+  a.tag = team_tag(plan, varlen);
+  using bf = __nv_bfloat16;
+  if (plan.io == BLR_F32)
+    return z != nullptr ? launch_team_bwd<float, true>(a, st) : launch_team_bwd<float, false>(a, st);
+  return z != nullptr ? launch_team_bwd<bf, true>(a, st) : launch_team_bwd<bf, false>(a, st);
 }
 
-// Grid of the elementwise merge kernels: 16-byte vectors, 256 threads a block,
-// at most 8 blocks per SM (grid-stride beyond).
-unsigned merge_grid(int64_t n_vec) {
-  int64_t blocks = (n_vec + 255) / 256;
-  const int64_t cap = (int64_t)sm_count() * 8;
-  if (blocks > cap) blocks = cap;
-  return (unsigned)(blocks > 0 ? blocks : 1);
-}
-
-blr_status launch_merge_fwd(int io, void* y, const void* z, int64_t n, cudaStream_t st) {
-  if (io == BLR_F32) {
-    const int64_t nv = n / 4;
-    blr::merge_fwd_kernel<float><<<merge_grid(nv), 256, 0, st>>>(static_cast<float*>(y),
-                                                                 static_cast<const float*>(z), nv);
-  } else {
-    const int64_t nv = n / 8;
-    blr::merge_fwd_kernel<__nv_bfloat16><<<merge_grid(nv), 256, 0, st>>>(
-        static_cast<__nv_bfloat16*>(y), static_cast<const __nv_bfloat16*>(z), nv);
-  }
-  return cuda_check(cudaGetLastError(), "launch merge_fwd_kernel");
-}
-
-blr_status launch_merge_bwd(int io, const void* dy, const void* z, void* dh, void* hz, int64_t n,
-                            cudaStream_t st) {
-  if (io == BLR_F32) {
-    const int64_t nv = n / 4;
-    blr::merge_bwd_kernel<float><<<merge_grid(nv), 256, 0, st>>>(
-        static_cast<const float*>(dy), static_cast<const float*>(z), static_cast<float*>(dh),
-        static_cast<float*>(hz), nv);
-  } else {
-    const int64_t nv = n / 8;
-    using bf = __nv_bfloat16;
-    blr::merge_bwd_kernel<bf><<<merge_grid(nv), 256, 0, st>>>(
-        static_cast<const bf*>(dy), static_cast<const bf*>(z), static_cast<bf*>(dh),
-        static_cast<bf*>(hz), nv);
-  }
-  return cuda_check(cudaGetLastError(), "launch merge_bwd_kernel");
-}
-
-// The library's static device scratch (defined with blr_scan_fwd_noalloc):
-// its size, and its address on the current device after checking that the
-// problem's workspace fits (BLR_ERR_UNSUPPORTED, nothing enqueued, if not).
-constexpr size_t kLibraryScratchBytes = (size_t)128 << 20;  // 128 MiB
+// The address of the library's scratch on the current device, after checking
+// that the problem's workspace fits (BLR_ERR_UNSUPPORTED, nothing enqueued, if not).
 blr_status library_scratch(const Plan& plan, const char* who, void** out);
 
 // blr_scan_fwd (z == NULL) and blr_scan_fwd_gated (z given; h is then y).
 blr_status scan_fwd_entry(const blr_desc* desc, const void* x, const void* gate_logits,
                           const float* lambda, const float* h0, const void* z, void* h,
                           float* h_last, void* ws, size_t ws_bytes, blr_stream_t stream,
-                          bool gated, const int32_t* lengths = nullptr, bool varlen = false) {
+                          bool gated, const int32_t* lengths = nullptr, bool varlen = false,
+                          bool scratch = false) {
   Plan plan;
   bool empty = false;
-  BLR_TRY(check_desc(desc, &plan, &empty));
+  BLR_TRY(check_desc(desc, &plan, &empty, scratch));
   if (empty) return BLR_OK;
   BLR_TRY(need(lambda, "lambda", 16));
   BLR_TRY(optional(h0, "h0", 4));
@@ -671,21 +519,9 @@ blr_status scan_fwd_entry(const blr_desc* desc, const void* x, const void* gate_
   BLR_TRY(check_ws(plan, ws, ws_bytes));
 
   unsigned char* w = static_cast<unsigned char*>(ws);
-  if (plan.seq)  // serial kernels (the merge fused): no preparation
-    return scan_fwd_seq(plan, x, gate_logits, lambda, h0, h, h_last, w, st,
-                        h != nullptr ? z : nullptr, lengths);
-  // Few long chains: the chained single-pass forward, or with the gated
-  // layer's merge the segmented serial kernels (the merge fused); rows with
-  // lengths on these problems run the tiled kernels. Either forward leaves the
-  // kept states the segmented backward starts from.
-  if (plan.nseg > 0 && lengths == nullptr) {
-    if (z == nullptr || h == nullptr)
-      return scan_fwd_chain(plan, x, gate_logits, lambda, h0, h, h_last, w, st);
-    return scan_fwd_seg(plan, x, gate_logits, lambda, h0, h, h_last, w, st, z);
-  }
-  BLR_TRY(scan_fwd_tiled(plan, desc, x, gate_logits, lambda, h0, h, h_last, w, st, lengths));
-  if (z == nullptr || h == nullptr) return BLR_OK;
-  return launch_merge_fwd(desc->io, h, z, desc->B * desc->L * desc->D, st);
+  const void* merge = h != nullptr ? z : nullptr;
+  if (plan.seq) return scan_fwd_seq(plan, x, gate_logits, lambda, h0, h, h_last, w, st, merge, lengths);
+  return scan_fwd_team(plan, x, gate_logits, lambda, h0, h, h_last, w, st, merge, lengths, varlen);
 }
 
 // blr_scan_bwd (z == NULL; dh is the gradient of h) and blr_scan_bwd_gated
@@ -697,7 +533,7 @@ blr_status scan_bwd_entry(const blr_desc* desc, const void* dh, const float* dh_
                           const int32_t* lengths = nullptr, bool varlen = false) {
   Plan plan;
   bool empty = false;
-  BLR_TRY(check_desc(desc, &plan, &empty));
+  BLR_TRY(check_desc(desc, &plan, &empty, ws == nullptr));
   if (empty) return BLR_OK;
   BLR_TRY(need(lambda, "lambda", 16));
   BLR_TRY(need(dlambda, "dlambda", 4));
@@ -731,7 +567,7 @@ blr_status scan_bwd_entry(const blr_desc* desc, const void* dh, const float* dh_
     void* scratch = nullptr;
     BLR_TRY(library_scratch(plan, "a backward without a workspace", &scratch));
     BLR_TRY(scan_fwd_entry(desc, x, gate_logits, lambda, h0, nullptr, nullptr, nullptr, scratch,
-                           kLibraryScratchBytes, stream, false, lengths, varlen));
+                           kLibraryScratchBytes, stream, false, lengths, varlen, true));
     ws = scratch;
     ws_bytes = kLibraryScratchBytes;
   }
@@ -741,23 +577,8 @@ blr_status scan_bwd_entry(const blr_desc* desc, const void* dh, const float* dh_
   if (plan.seq)  // the forward cleared the counters and partial sums
     return scan_bwd_seq(plan, dh, dh_last, x, gate_logits, lambda, h0, dx, dgate_logits, dlambda,
                         dh0, w, st, z, dz, lengths);
-  if (plan.nseg > 0 && lengths == nullptr) {
-    if (z == nullptr)
-      return scan_bwd_chain(plan, dh, dh_last, x, gate_logits, lambda, h0, dx, dgate_logits,
-                            dlambda, dh0, w, st);
-    return scan_bwd_seg(plan, dh, dh_last, x, gate_logits, lambda, h0, dx, dgate_logits, dlambda,
-                        dh0, w, st, z, dz);
-  }
-  if (z == nullptr)
-    return scan_bwd_tiled(plan, desc, dh, dh_last, x, gate_logits, lambda, h0, dx, dgate_logits,
-                          dlambda, dh0, w, st, lengths);
-  // Gated, tiled: h recomputed into dz (a forward of the same problem, which
-  // also rewrites the same carries), then dh = dy SiLU(z) into dx and
-  // dz = dy h SiLU'(z), then the scan's backward from dh in dx.
-  BLR_TRY(scan_fwd_tiled(plan, desc, x, gate_logits, lambda, h0, dz, nullptr, w, st, nullptr));
-  BLR_TRY(launch_merge_bwd(desc->io, dh, z, dx, dz, desc->B * desc->L * desc->D, st));
-  return scan_bwd_tiled(plan, desc, dx, dh_last, x, gate_logits, lambda, h0, dx, dgate_logits,
-                        dlambda, dh0, w, st, nullptr);
+  return scan_bwd_team(plan, dh, dh_last, x, gate_logits, lambda, h0, dx, dgate_logits, dlambda,
+                       dh0, w, st, z, dz, lengths, varlen);
 }
 
 }  // namespace
@@ -775,8 +596,8 @@ int blr_scan_family(const blr_desc* desc, int with_lengths) {
   Plan plan;
   bool empty = false;
   if (check_desc(desc, &plan, &empty) != BLR_OK || empty || desc->L == 0) return BLR_FAMILY_NONE;
-  if (plan.seq) return BLR_FAMILY_SERIAL;
-  if (plan.nseg > 0 && !with_lengths) return BLR_FAMILY_SEGMENTED;
+  if (plan.n_chain >= blr::kManyChains) return BLR_FAMILY_SERIAL;
+  if (plan.segmented && !with_lengths) return BLR_FAMILY_SEGMENTED;
   return BLR_FAMILY_TILED;
 }
 
@@ -916,7 +737,7 @@ blr_status blr_workspace_status(const blr_desc* desc, const void* ws, size_t ws_
                                 blr_stream_t stream) {
   Plan plan;
   bool empty = false;
-  BLR_TRY(check_desc(desc, &plan, &empty));
+  BLR_TRY(check_desc(desc, &plan, &empty, ws == nullptr));
   if (empty || desc->L == 0) return BLR_OK;
   if (ws == nullptr) {  // the scratch of a backward called without a workspace
     void* scratch = nullptr;
@@ -1051,11 +872,11 @@ extern "C" blr_status blr_scan_fwd_noalloc(const blr_desc* desc, const void* x,
                                            blr_stream_t stream) {
   Plan plan;
   bool empty = false;
-  BLR_TRY(check_desc(desc, &plan, &empty));
+  BLR_TRY(check_desc(desc, &plan, &empty, true));
   if (empty || desc->L == 0)  // nothing that needs scratch: the ordinary path does it
     return blr_scan_fwd(desc, x, gate_logits, lambda, h0, h, h_last, nullptr, 0, stream);
   void* scratch = nullptr;
   BLR_TRY(library_scratch(plan, "blr_scan_fwd_noalloc", &scratch));
-  return blr_scan_fwd(desc, x, gate_logits, lambda, h0, h, h_last, scratch, kLibraryScratchBytes,
-                      stream);
+  return scan_fwd_entry(desc, x, gate_logits, lambda, h0, nullptr, h, h_last, scratch,
+                        kLibraryScratchBytes, stream, false, nullptr, false, true);
 }

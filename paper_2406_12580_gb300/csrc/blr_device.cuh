@@ -493,6 +493,13 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const void* tmap, uint64_
       : "memory");
 }
 
+// Requests the box at (c0, c1, c2) of the tensor map into L2.
+__device__ __forceinline__ void tma_prefetch_3d(const void* tmap, int c0, int c1, int c2) {
+  asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(tmap),
+               "r"(c0), "r"(c1), "r"(c2)
+               : "memory");
+}
+
 // One 3-D tile store: shared memory into the box at (c0, c1, c2) of the tensor
 // map; elements outside the tensor are not written. The writes of the box in
 // shared memory must be fenced to the async proxy first.
