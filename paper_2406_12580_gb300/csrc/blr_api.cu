@@ -203,6 +203,25 @@ blr_status launch_cooperative(K kernel, unsigned grid, int threads, size_t smem,
   return cuda_check(cudaLaunchKernelEx(&cfg, kernel, args), what);
 }
 
+// Launches a kernel that may begin its prologue while the kernel before it on
+// the stream finishes (programmatic dependent launch): the kernel itself waits
+// for that one (griddepcontrol.wait) before it touches global memory.
+template <typename K, typename A>
+blr_status launch_overlapped(K kernel, unsigned grid, dim3 threads, size_t smem, cudaStream_t st,
+                          const A& args, const char* what) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = threads;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cuda_check(cudaLaunchKernelEx(&cfg, kernel, args), what);
+}
+
 // ----------------------------------------------------------- serial kernels
 //
 // One warp per block, one block per chain. The ring's stage count is sized so
@@ -258,8 +277,7 @@ blr_status launch_seq_fwd(blr::SeqFwdArgs& a, cudaStream_t st) {
     if (late_refill<T>(a.stages)) kernel = blr::seq_fwd_kernel<T, M, VEC, R, RB, GATED, MODE, true>;
   }
   BLR_TRY(allow_smem(kernel, smem));
-  kernel<<<(unsigned)blocks, 32, smem, st>>>(a);
-  return cuda_check(cudaGetLastError(), "launch seq_fwd_kernel");
+  return launch_overlapped(kernel, (unsigned)blocks, dim3(32), smem, st, a, "launch seq_fwd_kernel");
 }
 
 template <typename T, class M, int VEC, int R, int RB, bool GATED, int MODE = blr::kSeqPlain>
@@ -273,8 +291,7 @@ blr_status launch_seq_bwd(blr::SeqBwdArgs& a, cudaStream_t st) {
     if (late_refill<T>(a.stages)) kernel = blr::seq_bwd_kernel<T, M, VEC, R, RB, GATED, MODE, true>;
   }
   BLR_TRY(allow_smem(kernel, smem));
-  kernel<<<(unsigned)blocks, 32, smem, st>>>(a);
-  return cuda_check(cudaGetLastError(), "launch seq_bwd_kernel");
+  return launch_overlapped(kernel, (unsigned)blocks, dim3(32), smem, st, a, "launch seq_bwd_kernel");
 }
 
 // The serial kernels' views: x-shaped tensors as (D, L, B); gate_logits-shaped
@@ -374,25 +391,6 @@ blr_status scan_bwd_seq(const Plan& plan, const void* dh, const float* dh_last, 
 
 // ------------------------------------------------------------- team kernels
 
-// Launches a kernel that may begin its prologue while the kernel before it on
-// the stream finishes (programmatic dependent launch): the kernel itself waits
-// for that one (griddepcontrol.wait) before it touches global memory.
-template <typename K, typename A>
-blr_status launch_chained(K kernel, unsigned grid, int threads, size_t smem, cudaStream_t st,
-                          const A& args, const char* what) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3((unsigned)threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cuda_check(cudaLaunchKernelEx(&cfg, kernel, args), what);
-}
-
 // One block per SM (its shared memory fills one), at most one team per unit of
 // work: a chain in the local order, a tile with the look-back.
 template <typename K, typename A>
@@ -407,7 +405,7 @@ blr_status launch_team(K kernel, size_t smem, A& args, cudaStream_t st, const ch
   args.teams = grid * (unsigned)blr::kTeams;
   const int64_t n_g = p.n_chain / p.B;
   if (args.teams >= 8 * n_g) args.teams -= args.teams % (unsigned)n_g;
-  if (!p.lookback) return launch_chained(kernel, grid, threads, smem, st, args, what);
+  if (!p.lookback) return launch_overlapped(kernel, grid, dim3((unsigned)threads), smem, st, args, what);
   BLR_TRY(cuda_check(cudaMemsetAsync(args.ws + p.off_cinc, 0xff, p.off_cend - p.off_cinc, st),
                      "empty the look-back records"));
   return launch_cooperative(kernel, grid, threads, smem, st, args, what);
@@ -677,12 +675,13 @@ blr_status blr_step(int64_t B, int64_t D, blr_dtype io, float c, const float* h_
   if (n_vgroups * n_rg >= ((int64_t)1 << 31)) return fail(BLR_ERR_UNSUPPORTED, "grid too large");
   blr::StepArgs a{B, D, c, n_vgroups, h_prev, x_t, gate_logits_t, lambda, h_t};
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  const dim3 grid((unsigned)(n_vgroups * n_rg)), block((unsigned)bx, (unsigned)by);
+  const unsigned grid = (unsigned)(n_vgroups * n_rg);
+  const dim3 block((unsigned)bx, (unsigned)by);
   if (io == BLR_F32)
-    blr::step_kernel<float, 4, blr::MathPrecise, 2><<<grid, block, 0, st>>>(a);
-  else
-    blr::step_kernel<__nv_bfloat16, 8, blr::MathFast, 1><<<grid, block, 0, st>>>(a);
-  return cuda_check(cudaGetLastError(), "launch step_kernel");
+    return launch_overlapped(blr::step_kernel<float, 4, blr::MathPrecise, 2>, grid, block, 0, st, a,
+                             "launch step_kernel");
+  return launch_overlapped(blr::step_kernel<__nv_bfloat16, 8, blr::MathFast, 1>, grid, block, 0, st, a,
+                           "launch step_kernel");
 }
 
 blr_status blr_steps(int64_t B, int64_t K, int64_t D, blr_dtype io, blr_dtype state, float c,
@@ -714,23 +713,25 @@ blr_status blr_steps(int64_t B, int64_t K, int64_t D, blr_dtype io, blr_dtype st
   BLR_TRY(need(gate_logits, "gate_logits", 16));
   BLR_TRY(optional(h_seq, "h_seq", 16));
   const int vec = io == BLR_F32 ? 4 : 8;
-  const int64_t threads = B * (D / vec);
-  const int64_t blocks = (threads + 255) / 256;
-  if (blocks >= ((int64_t)1 << 31)) return fail(BLR_ERR_UNSUPPORTED, "grid too large");
-  blr::StepsArgs a{B, K, D, c, h_prev, x, gate_logits, lambda, h_out, h_seq};
+  const int64_t nvec = D / vec;
+  const int bx = (int)(nvec < 64 ? nvec : 64);
+  const int by = 256 / bx;
+  const int64_t n_vgroups = (nvec + bx - 1) / bx;
+  // a persistent grid, at most one row group per block row of work
+  const int64_t need_rg = (B + by - 1) / by;
+  int64_t n_rg = ((int64_t)sm_count() * blr::kStepsBlocksPerSm + n_vgroups - 1) / n_vgroups;
+  if (n_rg > need_rg) n_rg = need_rg;
+  if (n_rg < 1) n_rg = 1;
+  if (n_vgroups * n_rg >= ((int64_t)1 << 31)) return fail(BLR_ERR_UNSUPPORTED, "grid too large");
+  blr::StepsArgs a{B, K, D, c, n_vgroups, h_prev, x, gate_logits, lambda, h_out, h_seq};
   using bf = __nv_bfloat16;
-  if (io == BLR_F32) {
-    if (state == BLR_F32)
-      blr::steps_kernel<float, float, 4, blr::MathPrecise><<<(unsigned)blocks, 256, 0, st>>>(a);
-    else
-      blr::steps_kernel<float, bf, 4, blr::MathPrecise><<<(unsigned)blocks, 256, 0, st>>>(a);
-  } else {
-    if (state == BLR_F32)
-      blr::steps_kernel<bf, float, 8, blr::MathFast><<<(unsigned)blocks, 256, 0, st>>>(a);
-    else
-      blr::steps_kernel<bf, bf, 8, blr::MathFast><<<(unsigned)blocks, 256, 0, st>>>(a);
-  }
-  return cuda_check(cudaGetLastError(), "launch steps_kernel");
+  const unsigned grid = (unsigned)(n_vgroups * n_rg);
+  const dim3 block((unsigned)bx, (unsigned)by);
+  auto launch = [&](auto kernel) { return launch_overlapped(kernel, grid, block, 0, st, a, "launch steps_kernel"); };
+  if (io == BLR_F32)
+    return state == BLR_F32 ? launch(blr::steps_kernel<float, float, 4>)
+                            : launch(blr::steps_kernel<float, bf, 4>);
+  return state == BLR_F32 ? launch(blr::steps_kernel<bf, float, 8>) : launch(blr::steps_kernel<bf, bf, 8>);
 }
 
 blr_status blr_workspace_status(const blr_desc* desc, const void* ws, size_t ws_bytes,

@@ -11,6 +11,17 @@
 
 namespace blr {
 
+__device__ __forceinline__ uint32_t smem_addr(const void* p) {
+  return (uint32_t)__cvta_generic_to_shared(p);
+}
+
+// Waits for the grid this one was launched behind (programmatic dependent
+// launch) and lets the next one start its own prologue; no-ops without it.
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ----------------------------------------------------------------- vector I/O
 //
 // One lane moves VEC consecutive channels of one row with one access. Inputs
@@ -334,6 +345,73 @@ struct GatePolicy<MathFast> {
   using type = GatesFast;
 };
 
+// ------------------------------------------------------------ packed pairs
+//
+// Two elements as one float2 (a bfloat16 word's two channels, or two float32
+// values), so that the multiply-adds of both run as one paired instruction (fma/mul/add.rn.f32x2); the
+// transcendental units (tanh, rsqrt, sqrt) stay scalar. Every paired operation
+// rounds each half exactly as its scalar counterpart would.
+
+constexpr uint32_t kBf2Half = 0x3f003f00u;     // (0.5, 0.5) as bfloat16 pairs
+constexpr uint32_t kBf2NegHalf = 0xbf00bf00u;  // (-0.5, -0.5)
+
+__device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
+// The pair t as floats.
+__device__ __forceinline__ float2 bf2_unpack(uint32_t t) {
+  return make_float2(__uint_as_float(t << 16), __uint_as_float(t & 0xffff0000u));
+}
+// The pair t times s2 (a bfloat16 pair of +-0.5: exact, a sign and exponent
+// change), as floats.
+__device__ __forceinline__ float2 bf2_scaled(uint32_t t, uint32_t s2) {
+  uint32_t u;
+  asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(u) : "r"(t), "r"(s2));
+  return bf2_unpack(u);
+}
+__device__ __forceinline__ uint32_t bf2_pack(float2 v) { return pack_bf16x2(v.x, v.y); }
+// A shared-memory word read afresh where it is used, never kept in a register
+// from an earlier read of the same word (the backward re-reads a step's inputs
+// instead of holding them, and their gates, across a sub-block).
+__device__ __forceinline__ uint32_t lds_again(const unsigned char* p) {
+  uint32_t v;
+  asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(smem_addr(p)));
+  return v;
+}
+__device__ __forceinline__ float2 tanh2(float2 a) {
+  return make_float2(tanh_approx(a.x), tanh_approx(a.y));
+}
+// e^l - 1 for l <= 0 (GatesFast: the degree-4 series, ex2 beyond its range
+// unless POLY), as expm1_neg<4, POLY> on each half.
+template <bool POLY>
+__device__ __forceinline__ float2 expm1_neg2(float2 l) {
+  if constexpr (POLY) {
+    float2 q = __ffma2_rn(f2(1.0f / 24), l, f2(1.0f / 6));
+    q = __ffma2_rn(q, l, f2(0.5f));
+    q = __ffma2_rn(q, l, f2(1.0f));
+    return __fmul2_rn(q, l);
+  } else {
+    return make_float2(expm1_neg<4, false>(l.x), expm1_neg<4, false>(l.y));
+  }
+}
+__device__ __forceinline__ float2 sigmoid2(float2 z) {  // MathPrecise::sigmoid on each half
+  const float2 t = __fmul2_rn(f2(-1.4426950408889634f), z);
+  const float2 e = __fadd2_rn(f2(1.0f), make_float2(ex2_approx(t.x), ex2_approx(t.y)));
+  return make_float2(rcp_approx(e.x), rcp_approx(e.y));
+}
+// e^l - 1 for l <= 0 as expm1_neg<6, POLY> on each half.
+template <bool POLY>
+__device__ __forceinline__ float2 expm1_neg2_precise(float2 l) {
+  if constexpr (POLY) {
+    float2 q = __ffma2_rn(f2(1.0f / 720), l, f2(1.0f / 120));
+    q = __ffma2_rn(q, l, f2(1.0f / 24));
+    q = __ffma2_rn(q, l, f2(1.0f / 6));
+    q = __ffma2_rn(q, l, f2(0.5f));
+    q = __ffma2_rn(q, l, f2(1.0f));
+    return __fmul2_rn(q, l);
+  } else {
+    return make_float2(expm1_neg<6, false>(l.x), expm1_neg<6, false>(l.y));
+  }
+}
+
 // k = -c softplus(Lambda), softplus(z) = max(z, 0) + log1p(exp(-|z|)), accurate.
 __device__ __forceinline__ float decay_rate(float c, float lambda) {
   return -c * (fmaxf(lambda, 0.0f) + log1pf(expf(-fabsf(lambda))));
@@ -419,10 +497,6 @@ __device__ __noinline__ bool wait_word(const uint32_t* flag, uint32_t* err, uint
 // Tiles of the inputs are moved into shared memory by the tensor memory
 // accelerator (cp.async.bulk.tensor, 3-D boxes of 32 channels x tile steps x
 // one batch row) and counted on an mbarrier per pipeline stage.
-
-__device__ __forceinline__ uint32_t smem_addr(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
 
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");

@@ -48,6 +48,7 @@ template <typename T, int VEC, class M, int ROWS>
 __global__ void __launch_bounds__(256, kStepBlocksPerSm) step_kernel(const StepArgs a) {
   using IO = Io<T, VEC>;
   __shared__ float s_k[64 * 8];
+  pdl_wait();
   const int64_t vg = blockIdx.x % a.n_vgroups;
   const int64_t rg = blockIdx.x / a.n_vgroups;
   const int64_t n_rg = gridDim.x / a.n_vgroups;  // the grid launches whole channel groups
@@ -116,14 +117,23 @@ __global__ void __launch_bounds__(256, kStepBlocksPerSm) step_kernel(const StepA
 // ------------------------------------------------------- K recurrent steps
 //
 // h_j = alpha_j h_{j-1} + beta_j x_j for j = 1..K and every (row, channel), from
-// h_0 = h_prev: a thread owns VEC channels of one row and walks its K steps
-// serially with the state in float32 registers, whatever the state dtype in
-// memory (a bfloat16 state is rounded once, when it is stored). The loads of
-// kStepsAhead steps are issued before the first of them is used.
+// h_0 = h_prev: a thread owns VEC channels of one row at a time and walks its K
+// steps serially with the state in float32 registers, whatever the state dtype
+// in memory (a bfloat16 state is rounded once, when it is stored).
+//
+// A persistent grid (as the single step's): a thread goes on to its next row
+// without a gap. Its inputs come through kStepsAhead register sets, each
+// refilled as soon as its step is done, across the ends of rows, so that loads
+// are always in flight; the next row's state is requested a row ahead. The
+// arithmetic runs on pairs of channels, and k is computed once a block.
+// 65536 x 8 x 64 bfloat16 with all states written: 47.6 us (0.88 of the
+// measured copy rate); one row a thread, its loads in batches of four steps and
+// the arithmetic unpaired took 55.7.
 
 struct StepsArgs {
   int64_t B, K, D;
   float c;
+  int64_t n_vgroups;   // blocks along the channel vectors
   const void* h_prev;  // (B, D), state dtype
   const void* x;       // (B, K, D), io dtype
   const void* gl;      // (B, K, 2D), io dtype
@@ -133,6 +143,34 @@ struct StepsArgs {
 };
 
 constexpr int kStepsAhead = 4;
+constexpr int kStepsBlocksPerSm = 2;
+
+// One step of a pair of channels from its raw inputs (a bfloat16 word, halved
+// on the packed pair, or two floats): h <- alpha h + sqrt(1 - alpha^2) i x.
+// kp: k/2 of the channels for bfloat16, k for float32.
+template <bool POLY>
+__device__ __forceinline__ void step_pair(uint32_t x, uint32_t r, uint32_t i, float2 kp, float2& h) {
+  const float2 hx = bf2_scaled(x, kBf2Half);
+  const float2 e = expm1_neg2<POLY>(__ffma2_rn(kp, tanh2(bf2_scaled(r, kBf2Half)), kp));
+  const float2 m2 = __fmul2_rn(e, __fadd2_rn(e, f2(2.0f)));  // -(1 - alpha^2)
+  const float2 u = __fmul2_rn(make_float2(sqrt_approx(-m2.x), sqrt_approx(-m2.y)),
+                              __ffma2_rn(hx, tanh2(bf2_scaled(i, kBf2Half)), hx));
+  h = __ffma2_rn(__fadd2_rn(f2(1.0f), e), h, u);
+}
+template <bool POLY>
+__device__ __forceinline__ void step_pair(float2 x, float2 r, float2 i, float2 kp, float2& h) {
+  const float2 e = expm1_neg2_precise<POLY>(__fmul2_rn(kp, sigmoid2(r)));
+  const float2 m2 = __fmul2_rn(e, __fadd2_rn(e, f2(2.0f)));
+  const float2 u = __fmul2_rn(make_float2(sqrt_approx(-m2.x), sqrt_approx(-m2.y)),
+                              __fmul2_rn(sigmoid2(i), x));
+  h = __ffma2_rn(__fadd2_rn(f2(1.0f), e), h, u);
+}
+__device__ __forceinline__ uint32_t raw_pair(const uint4& v, int p) {
+  return p == 0 ? v.x : p == 1 ? v.y : p == 2 ? v.z : v.w;
+}
+__device__ __forceinline__ float2 raw_pair(const float4& v, int p) {
+  return p == 0 ? make_float2(v.x, v.y) : make_float2(v.z, v.w);
+}
 
 template <typename S, int VEC>
 __device__ __forceinline__ void load_state(const S* p, float (&h)[VEC]) {
@@ -153,53 +191,102 @@ __device__ __forceinline__ void store_state(S* p, const float (&h)[VEC]) {
   }
 }
 
-template <typename T, typename S, int VEC, class M>
-__global__ void __launch_bounds__(256) steps_kernel(const StepsArgs a) {
+template <typename T, typename S, int VEC, bool POLY>
+__device__ __forceinline__ void steps_walk(const StepsArgs& a, const float2 (&kp)[VEC / 2], int64_t d0,
+                                           int64_t r, int64_t rstride) {
   using IO = Io<T, VEC>;
   using Raw = typename IO::Raw;
-  const int64_t nv = a.D / VEC;
-  const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (idx >= a.B * nv) return;
-  const int64_t b = idx / nv;
-  const int64_t d0 = (idx - b * nv) * VEC;
-  float k[VEC], h[VEC];
-#pragma unroll
-  for (int v = 0; v < VEC; ++v) k[v] = decay_rate(a.c, a.lambda[d0 + v]);
-  load_state<S, VEC>(static_cast<const S*>(a.h_prev) + b * a.D + d0, h);
-  const T* x = static_cast<const T*>(a.x) + b * a.K * a.D + d0;
-  const T* gl = static_cast<const T*>(a.gl) + b * a.K * 2 * a.D + d0;
-  T* hs = a.h_seq != nullptr ? static_cast<T*>(a.h_seq) + b * a.K * a.D + d0 : nullptr;
-  for (int64_t j0 = 0; j0 < a.K; j0 += kStepsAhead) {
-    Raw rx[kStepsAhead], rr[kStepsAhead], ri[kStepsAhead];
-#pragma unroll
-    for (int u = 0; u < kStepsAhead; ++u) {
-      const int64_t j = j0 + u;
-      if (j < a.K) {
-        rx[u] = IO::load_raw(x + j * a.D);
-        rr[u] = IO::load_raw(gl + j * 2 * a.D);
-        ri[u] = IO::load_raw(gl + j * 2 * a.D + a.D);
+  constexpr int A = kStepsAhead, P = VEC / 2;
+  if (r >= a.B) return;
+  // where the next inputs are: row lr, step lj
+  int64_t lr = r, lj = 0;
+  const T* px = static_cast<const T*>(a.x) + r * a.K * a.D + d0;
+  const T* pg = static_cast<const T*>(a.gl) + r * a.K * 2 * a.D + d0;
+  const int64_t row_x = (rstride * a.K - a.K + 1) * a.D;  // from a row's last step to the next row's first
+  Raw rx[A], rr[A], ri[A];
+  auto request = [&](int u) {
+    if (lr < a.B) {
+      rx[u] = IO::load_raw(px);
+      rr[u] = IO::load_raw(pg);
+      ri[u] = IO::load_raw(pg + a.D);
+      const bool turn = ++lj == a.K;
+      if (turn) {
+        lj = 0;
+        lr += rstride;
       }
+      px += turn ? row_x : a.D;
+      pg += turn ? 2 * row_x : 2 * a.D;
     }
+  };
 #pragma unroll
-    for (int u = 0; u < kStepsAhead; ++u) {
-      const int64_t j = j0 + u;
-      if (j < a.K) {
-        float xv[VEC], rv[VEC], iv[VEC];
-        IO::unpack(rx[u], xv);
-        IO::unpack(rr[u], rv);
-        IO::unpack(ri[u], iv);
+  for (int u = 0; u < A; ++u) request(u);
+  const S* hp = static_cast<const S*>(a.h_prev) + d0;
+  S* ho = static_cast<S*>(a.h_out) + d0;
+  T* hs = a.h_seq != nullptr ? static_cast<T*>(a.h_seq) + r * a.K * a.D + d0 : nullptr;
+  float hv[VEC], hn[VEC];
+  load_state<S, VEC>(hp + r * a.D, hv);
+  float2 h[P];
 #pragma unroll
-        for (int v = 0; v < VEC; ++v) {
-          const float r = M::sigmoid(rv[v]);
-          const float i = M::sigmoid(iv[v]);
-          const float e = M::expm1_any(k[v] * r);
-          h[v] = fmaf(1.0f + e, h[v], M::sqrt(-e * (2.0f + e)) * i * xv[v]);
-        }
-        if (hs != nullptr) IO::store(hs + j * a.D, h);
+  for (int p = 0; p < P; ++p) h[p] = make_float2(hv[2 * p], hv[2 * p + 1]);
+  if (r + rstride < a.B) load_state<S, VEC>(hp + (r + rstride) * a.D, hn);
+  for (int64_t j = 0;;) {
+#pragma unroll
+    for (int u = 0; u < A; ++u) {
+#pragma unroll
+      for (int p = 0; p < P; ++p)
+        step_pair<POLY>(raw_pair(rx[u], p), raw_pair(rr[u], p), raw_pair(ri[u], p), kp[p], h[p]);
+      request(u);
+#pragma unroll
+      for (int p = 0; p < P; ++p) {
+        hv[2 * p] = h[p].x;
+        hv[2 * p + 1] = h[p].y;
+      }
+      const bool turn = ++j == a.K;
+      if (hs != nullptr) {
+        IO::store(hs, hv);
+        hs += turn ? row_x : a.D;
+      }
+      if (turn) {
+        store_state<S, VEC>(ho + r * a.D, hv);
+        j = 0;
+        r += rstride;
+        if (r >= a.B) return;
+#pragma unroll
+        for (int p = 0; p < P; ++p) h[p] = make_float2(hn[2 * p], hn[2 * p + 1]);
+        if (r + rstride < a.B) load_state<S, VEC>(hp + (r + rstride) * a.D, hn);
       }
     }
   }
-  store_state<S, VEC>(static_cast<S*>(a.h_out) + b * a.D + d0, h);
+}
+
+template <typename T, typename S, int VEC>
+__global__ void __launch_bounds__(256, kStepsBlocksPerSm) steps_kernel(const StepsArgs a) {
+  __shared__ float s_k[64 * 8];
+  pdl_wait();
+  const int64_t vg = blockIdx.x % a.n_vgroups;
+  const int64_t rg = blockIdx.x / a.n_vgroups;
+  const int64_t n_rg = gridDim.x / a.n_vgroups;  // the grid launches whole channel groups
+  const int64_t dblock = vg * blockDim.x * VEC;
+  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+  bool poly = true;
+  for (int j = tid; j < (int)blockDim.x * VEC; j += blockDim.x * blockDim.y) {
+    const float k = dblock + j < a.D ? decay_rate(a.c, a.lambda[dblock + j]) : 0.0f;
+    s_k[j] = k;
+    poly = poly && k >= -kExpm1Series;
+  }
+  poly = __syncthreads_and(poly);
+  const int64_t d0 = dblock + threadIdx.x * VEC;
+  if (d0 >= a.D) return;
+  float2 kp[VEC / 2];
+  constexpr float f = sizeof(T) == 4 ? 1.0f : 0.5f;
+#pragma unroll
+  for (int p = 0; p < VEC / 2; ++p)
+    kp[p] = make_float2(f * s_k[threadIdx.x * VEC + 2 * p], f * s_k[threadIdx.x * VEC + 2 * p + 1]);
+  const int64_t r = rg * blockDim.y + threadIdx.y, rstride = n_rg * blockDim.y;
+  if (poly)
+    steps_walk<T, S, VEC, true>(a, kp, d0, r, rstride);
+  else
+    steps_walk<T, S, VEC, false>(a, kp, d0, r, rstride);
 }
 
 // ------------------------------------------------------------ bounded-wait test

@@ -27,7 +27,11 @@
 //
 // The forward's first block also restarts the workspace bookkeeping (error
 // word, problem tag, the backward's exit counter and d Lambda partial sums), so
-// no preparation kernel runs before either scan.
+// no preparation kernel runs before either scan. Both kernels set their
+// barriers up and then wait for the kernel before them on the stream
+// (programmatic dependent launch), so that back-to-back calls do not pay the
+// launch: 256 x 200 x 64 float32 fwd + bwd 41.9 -> 39.0 us, 1000 x 200 x 64
+// bfloat16 with lengths 67.2 -> 62.1.
 #pragma once
 
 #include "blr_kernels.cuh"
@@ -140,54 +144,6 @@ __device__ __forceinline__ void seq_reset_workspace(unsigned char* ws, const Pla
     bh->exited = 0u;
     fh->tag = tag;
     fh->complete = 1u;
-  }
-}
-
-// ------------------------------------------------- packed bfloat16 pairs
-//
-// A bfloat16 lane's two channels as one float2, so that the multiply-adds of
-// both run as one paired instruction (fma/mul/add.rn.f32x2); the
-// transcendental units (tanh, rsqrt, sqrt) stay scalar. Every paired operation
-// rounds each half exactly as its scalar counterpart would.
-
-constexpr uint32_t kBf2Half = 0x3f003f00u;     // (0.5, 0.5) as bfloat16 pairs
-constexpr uint32_t kBf2NegHalf = 0xbf00bf00u;  // (-0.5, -0.5)
-
-__device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
-// The pair t as floats.
-__device__ __forceinline__ float2 bf2_unpack(uint32_t t) {
-  return make_float2(__uint_as_float(t << 16), __uint_as_float(t & 0xffff0000u));
-}
-// The pair t times s2 (a bfloat16 pair of +-0.5: exact, a sign and exponent
-// change), as floats.
-__device__ __forceinline__ float2 bf2_scaled(uint32_t t, uint32_t s2) {
-  uint32_t u;
-  asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(u) : "r"(t), "r"(s2));
-  return bf2_unpack(u);
-}
-__device__ __forceinline__ uint32_t bf2_pack(float2 v) { return pack_bf16x2(v.x, v.y); }
-// A shared-memory word read afresh where it is used, never kept in a register
-// from an earlier read of the same word (the backward re-reads a step's inputs
-// instead of holding them, and their gates, across a sub-block).
-__device__ __forceinline__ uint32_t lds_again(const unsigned char* p) {
-  uint32_t v;
-  asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(smem_addr(p)));
-  return v;
-}
-__device__ __forceinline__ float2 tanh2(float2 a) {
-  return make_float2(tanh_approx(a.x), tanh_approx(a.y));
-}
-// e^l - 1 for l <= 0 (GatesFast: the degree-4 series, ex2 beyond its range
-// unless POLY), as expm1_neg<4, POLY> on each half.
-template <bool POLY>
-__device__ __forceinline__ float2 expm1_neg2(float2 l) {
-  if constexpr (POLY) {
-    float2 q = __ffma2_rn(f2(1.0f / 24), l, f2(1.0f / 6));
-    q = __ffma2_rn(q, l, f2(0.5f));
-    q = __ffma2_rn(q, l, f2(1.0f));
-    return __fmul2_rn(q, l);
-  } else {
-    return make_float2(expm1_neg<4, false>(l.x), expm1_neg<4, false>(l.y));
   }
 }
 
@@ -335,6 +291,11 @@ __global__ void __launch_bounds__(32) seq_fwd_kernel(const __grid_constant__ Seq
   const int64_t BD = p.B * p.D;
   FwdHeader* fh = reinterpret_cast<FwdHeader*>(a.ws + p.off_fhdr);
 
+  if (lane == 0) {
+    for (int s = 0; s < ring.S; ++s) mbar_init(&ring.bars[s], 1);
+    fence_mbar_init();
+  }
+  pdl_wait();
   if (blockIdx.x == 0) seq_reset_workspace(a.ws, p, p.tag, lane);
 
   float k[VEC], kh[VEC], hc[VEC];
@@ -357,8 +318,6 @@ __global__ void __launch_bounds__(32) seq_fwd_kernel(const __grid_constant__ Seq
     if constexpr (GATED) tma_load_3d(dst + 3 * BOX, &a.tm_z, &ring.bars[st], cd, t, cb);
   };
   if (lane == 0) {
-    for (int s = 0; s < ring.S; ++s) mbar_init(&ring.bars[s], 1);
-    fence_mbar_init();
     for (int s = 0; s < ring.S && s < nblk; ++s) issue(s, s);
   }
   __syncwarp();
@@ -624,6 +583,11 @@ __global__ void __launch_bounds__(32, sizeof(T) == 4 ? 8 : 16) seq_bwd_kernel(co
   const int lane = threadIdx.x;
   FwdHeader* fh = reinterpret_cast<FwdHeader*>(a.ws + p.off_fhdr);
   BwdHeader* bh = reinterpret_cast<BwdHeader*>(a.ws + p.off_bhdr);
+  if (lane == 0) {
+    for (int s = 0; s < ring.S; ++s) mbar_init(&ring.bars[s], 1);
+    fence_mbar_init();
+  }
+  pdl_wait();
   {
     int ok = 0;
     if (lane == 0) {
@@ -679,8 +643,6 @@ __global__ void __launch_bounds__(32, sizeof(T) == 4 ? 8 : 16) seq_bwd_kernel(co
     if constexpr (GATED) tma_load_3d(dst + 4 * BOX, &a.tm_z, &ring.bars[st], cd, t, cb);
   };
   if (lane == 0) {
-    for (int s = 0; s < ring.S; ++s) mbar_init(&ring.bars[s], 1);
-    fence_mbar_init();
     for (int s = 0; s < ring.S && s < nblk; ++s) issue(s, nblk - 1 - s);
   }
   __syncwarp();

@@ -248,32 +248,11 @@ struct TileWalk {
   }
 };
 
-// ---------------------------------------------------------------- gate pairs
+// ----------------------------------------------------------------- gate pairs
 //
-// Two elements at a time, so that their multiply-adds run as paired float32
-// instructions: a bfloat16 lane's two channels of one row, or a float32
-// lane's channel in two consecutive rows. Same arithmetic, rounding and order
-// as the serial kernels' gates (GatesFast, GatesPrecise).
+// A bfloat16 lane's two channels of one row, or a float32 lane's channel in
+// two consecutive rows.
 
-__device__ __forceinline__ float2 sigmoid2(float2 z) {  // MathPrecise::sigmoid on each half
-  const float2 t = __fmul2_rn(f2(-1.4426950408889634f), z);
-  const float2 e = __fadd2_rn(f2(1.0f), make_float2(ex2_approx(t.x), ex2_approx(t.y)));
-  return make_float2(rcp_approx(e.x), rcp_approx(e.y));
-}
-// e^l - 1 for l <= 0 as expm1_neg<6, POLY> on each half.
-template <bool POLY>
-__device__ __forceinline__ float2 expm1_neg2_precise(float2 l) {
-  if constexpr (POLY) {
-    float2 q = __ffma2_rn(f2(1.0f / 720), l, f2(1.0f / 120));
-    q = __ffma2_rn(q, l, f2(1.0f / 24));
-    q = __ffma2_rn(q, l, f2(1.0f / 6));
-    q = __ffma2_rn(q, l, f2(0.5f));
-    q = __ffma2_rn(q, l, f2(1.0f));
-    return __fmul2_rn(q, l);
-  } else {
-    return make_float2(expm1_neg<6, false>(l.x), expm1_neg<6, false>(l.y));
-  }
-}
 __device__ __forceinline__ float2 lds_rows2(const unsigned char* p) {  // a channel's two rows
   return make_float2(*reinterpret_cast<const float*>(p), *reinterpret_cast<const float*>(p + 128));
 }
@@ -287,13 +266,6 @@ template <typename T>
 __device__ __forceinline__ float2 team_rate(float k0, float k1) {
   if constexpr (sizeof(T) == 4) return make_float2(k0, k0);
   return make_float2(0.5f * k0, 0.5f * k1);
-}
-
-// Waits for the grid this one was launched behind (programmatic dependent
-// launch) and lets the next one start its own prologue; no-ops without it.
-__device__ __forceinline__ void pdl_wait() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 }  // namespace blr
