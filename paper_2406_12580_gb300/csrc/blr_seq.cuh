@@ -149,9 +149,9 @@ __device__ __forceinline__ void seq_reset_workspace(unsigned char* ws, const Pla
 
 // ------------------------------------------------------------------ forward
 
-// seq_fwd_stage for a bfloat16 lane under GatesFast, without the merge: the
-// same arithmetic in the same order, on packed pairs.
-template <bool POLY, bool FULL, int R, int RB>
+// seq_fwd_stage for a bfloat16 lane under GatesFast: the same arithmetic in
+// the same order, on packed pairs.
+template <bool POLY, bool FULL, int R, int RB, bool GATED>
 __device__ __forceinline__ void seq_fwd_stage_bf16x2(unsigned char* sb, int rows, float2 kh,
                                                      float2& hc, float* carry, int64_t& cidx,
                                                      int64_t n_carry, int64_t BD, bool ch_ok) {
@@ -175,7 +175,12 @@ __device__ __forceinline__ void seq_fwd_stage_bf16x2(unsigned char* sb, int rows
   for (int s = 0; s < R; ++s) {
     if (FULL || s < rows) {
       hc = __ffma2_rn(al[s], hc, uu[s]);
-      *reinterpret_cast<uint32_t*>(sb + s * ROWB) = bf2_pack(hc);
+      float2 out = hc;
+      if constexpr (GATED) {  // y = h SiLU(z), off the gates' dependency chains
+        const float2 hz = bf2_scaled(*reinterpret_cast<const uint32_t*>(sb + 3 * BOX + s * ROWB), kBf2Half);
+        out = __fmul2_rn(hc, __ffma2_rn(hz, tanh2(hz), hz));
+      }
+      *reinterpret_cast<uint32_t*>(sb + s * ROWB) = bf2_pack(out);
       if ((s + 1) % RB == 0) {  // a kept state: after step (cidx + 1) RB - 1
         if (cidx < n_carry && ch_ok) *reinterpret_cast<float2*>(carry + cidx * BD) = hc;
         ++cidx;
@@ -274,8 +279,8 @@ __global__ void __launch_bounds__(32) seq_fwd_kernel(const __grid_constant__ Seq
   constexpr int NB = GATED ? 4 : 3;  // boxes per stage: x, rho, iota (, z)
   constexpr uint32_t BOX = seq_box_bytes<T, VEC, R>();
   static_assert(R % RB == 0, "kept states must fall on stage rows");
-  // bfloat16 lanes without the merge run their arithmetic on packed pairs
-  constexpr bool kPacked = G::kHalfInputs && VEC == 2 && !GATED;
+  // bfloat16 lanes run their arithmetic on packed pairs
+  constexpr bool kPacked = G::kHalfInputs && VEC == 2;
   const Plan& p = a.p;
   extern __shared__ unsigned char seq_smem[];
   SeqRing<NB, BOX> ring{align128(seq_smem), nullptr, a.stages};
@@ -344,11 +349,11 @@ __global__ void __launch_bounds__(32) seq_fwd_kernel(const __grid_constant__ Seq
       const float2 kh2 = make_float2(kh[0], kh[1]);
       if (rows == R) {
         if (poly)
-          seq_fwd_stage_bf16x2<true, true, R, RB>(lb, rows, kh2, hc2, carry, cidx, n_carry, BD, ch_ok);
+          seq_fwd_stage_bf16x2<true, true, R, RB, GATED>(lb, rows, kh2, hc2, carry, cidx, n_carry, BD, ch_ok);
         else
-          seq_fwd_stage_bf16x2<false, true, R, RB>(lb, rows, kh2, hc2, carry, cidx, n_carry, BD, ch_ok);
+          seq_fwd_stage_bf16x2<false, true, R, RB, GATED>(lb, rows, kh2, hc2, carry, cidx, n_carry, BD, ch_ok);
       } else {
-        seq_fwd_stage_bf16x2<false, false, R, RB>(lb, rows, kh2, hc2, carry, cidx, n_carry, BD, ch_ok);
+        seq_fwd_stage_bf16x2<false, false, R, RB, GATED>(lb, rows, kh2, hc2, carry, cidx, n_carry, BD, ch_ok);
       }
       hc[0] = hc2.x;
       hc[1] = hc2.y;
@@ -503,13 +508,14 @@ __device__ __forceinline__ void seq_bwd_sub(unsigned char* lb, int row0, int sro
   }
 }
 
-// seq_bwd_sub for a bfloat16 lane under GatesFast, without the merge, on
-// packed pairs. The forward recompute keeps, per step, alpha, -sqrt(1 - alpha^2)
+// seq_bwd_sub for a bfloat16 lane under GatesFast, on packed pairs. The forward recompute keeps, per step, alpha, -sqrt(1 - alpha^2)
 // and c = h_{t-1} - alpha i x / sqrt(1 - alpha^2) (so that d l = alpha g c);
 // the reverse recurrence re-reads the step's inputs for i and r, and uses
 // r (1 - r) = (1 - tanh(rho/2)^2) / 4, so d rho = d l (k/4) (1 - tanh^2).
-// kq = k/4 and nkq = -k/4 per channel.
-template <bool POLY, bool FULL, int R, int RB>
+// kq = k/4 and nkq = -k/4 per channel. GATED: the recompute also forms
+// dz = dy h SiLU'(z), rounded to the bfloat16 it is written as (one register a
+// step, where h itself would take two).
+template <bool POLY, bool FULL, int R, int RB, bool GATED>
 __device__ __forceinline__ void seq_bwd_sub_bf16x2(unsigned char* lb, int row0, int srows, float2 kh,
                                                    float2 kq, float2 nkq, float2& hc, float2& w,
                                                    float2& dlr) {
@@ -519,7 +525,9 @@ __device__ __forceinline__ void seq_bwd_sub_bf16x2(unsigned char* lb, int row0, 
   const unsigned char* s_x = s_dh + BOX;
   unsigned char* s_r = s_dh + 2 * BOX;
   unsigned char* s_i = s_dh + 3 * BOX;
+  unsigned char* s_z = s_dh + 4 * BOX;
   float2 AL[RB], NQ[RB], CP[RB];
+  uint32_t DZ[GATED ? RB : 1];
 #pragma unroll
   for (int s = 0; s < RB; ++s) {
     if (FULL || s < srows) {
@@ -536,12 +544,25 @@ __device__ __forceinline__ void seq_bwd_sub_bf16x2(unsigned char* lb, int row0, 
       NQ[s] = nq;
       CP[s] = __ffma2_rn(__fmul2_rn(al, rs), nix, hc);
       hc = __ffma2_rn(al, hc, __fmul2_rn(nq, nix));  // alpha h + sqrt(1 - alpha^2) i x
+      if constexpr (GATED) {  // with hz = z/2 and th = tanh(hz) as silu_grad
+        const float2 hz = bf2_scaled(*reinterpret_cast<const uint32_t*>(s_z + s * ROWB), kBf2Half);
+        const float2 th = tanh2(hz);
+        const float2 sg = __ffma2_rn(f2(0.5f), th, f2(0.5f));
+        const float2 df = __ffma2_rn(sg, __ffma2_rn(__fmul2_rn(f2(-1.0f), hz), th, hz), sg);
+        const float2 dy = bf2_unpack(*reinterpret_cast<const uint32_t*>(s_dh + s * ROWB));
+        DZ[s] = bf2_pack(__fmul2_rn(__fmul2_rn(dy, hc), df));
+      }
     }
   }
 #pragma unroll
   for (int s = RB - 1; s >= 0; --s) {
     if (FULL || s < srows) {
-      const float2 dh = bf2_unpack(*reinterpret_cast<const uint32_t*>(s_dh + s * ROWB));
+      float2 dh = bf2_unpack(*reinterpret_cast<const uint32_t*>(s_dh + s * ROWB));
+      if constexpr (GATED) {  // dh = dy SiLU(z)
+        const float2 hz = bf2_scaled(lds_again(s_z + s * ROWB), kBf2Half);
+        dh = __fmul2_rn(dh, __ffma2_rn(hz, tanh2(hz), hz));
+        *reinterpret_cast<uint32_t*>(s_z + s * ROWB) = DZ[s];
+      }
       const float2 nhx = bf2_scaled(lds_again(s_x + s * ROWB), kBf2NegHalf);
       const float2 thr = tanh2(bf2_scaled(lds_again(s_r + s * ROWB), kBf2Half));
       const float2 thi = tanh2(bf2_scaled(lds_again(s_i + s * ROWB), kBf2Half));
@@ -574,7 +595,7 @@ __global__ void __launch_bounds__(32, sizeof(T) == 4 ? 8 : 16) seq_bwd_kernel(co
   constexpr uint32_t BOX = seq_box_bytes<T, VEC, R>();
   constexpr int NSUB = R / RB;
   static_assert(R % RB == 0, "sub-blocks must tile a stage");
-  constexpr bool kPacked = G::kHalfInputs && VEC == 2 && !GATED;  // as seq_fwd_kernel
+  constexpr bool kPacked = G::kHalfInputs && VEC == 2;  // as seq_fwd_kernel
   const Plan& p = a.p;
   extern __shared__ unsigned char seq_smem[];
   SeqRing<NB, BOX> ring{align128(seq_smem), nullptr, a.stages};
@@ -692,11 +713,11 @@ __global__ void __launch_bounds__(32, sizeof(T) == 4 ? 8 : 16) seq_bwd_kernel(co
           const float2 nkq = make_float2(-kq.x, -kq.y);
           if (srows == RB) {
             if (poly)
-              seq_bwd_sub_bf16x2<true, true, R, RB>(lb, row0, srows, kh2, kq, nkq, hc2, w2, dlr2);
+              seq_bwd_sub_bf16x2<true, true, R, RB, GATED>(lb, row0, srows, kh2, kq, nkq, hc2, w2, dlr2);
             else
-              seq_bwd_sub_bf16x2<false, true, R, RB>(lb, row0, srows, kh2, kq, nkq, hc2, w2, dlr2);
+              seq_bwd_sub_bf16x2<false, true, R, RB, GATED>(lb, row0, srows, kh2, kq, nkq, hc2, w2, dlr2);
           } else {
-            seq_bwd_sub_bf16x2<false, false, R, RB>(lb, row0, srows, kh2, kq, nkq, hc2, w2, dlr2);
+            seq_bwd_sub_bf16x2<false, false, R, RB, GATED>(lb, row0, srows, kh2, kq, nkq, hc2, w2, dlr2);
           }
           w[0] = w2.x;
           w[1] = w2.y;
