@@ -280,6 +280,45 @@ BLR_API blr_status blr_steps(int64_t B, int64_t K, int64_t D, blr_dtype io, blr_
                              const float* lambda, void* h_out, void* h_seq, blr_stream_t stream);
 
 /*
+ * The gated recurrent layer's convolution (Alg. 1), with what surrounds it: the
+ * expansion's output H_x | H_z (B, L, 2C) becomes
+ *   x = SiLU(Conv1d(H_x)), causal and depthwise with 4 taps:
+ *       conv_t = bias + sum_k weight[c, k] H_x[t - 3 + k],
+ *   z = H_z,
+ * each (B, L, C), the scan's inputs. The backward returns dhxz (B, L, 2C) for
+ * dx and dz, and the taps' gradients.
+ * hxz, x, z, dx, dz, dhxz, weight (C, 4), bias (C), dweight, dbias: io dtype.
+ * C % 8 == 0, C <= 1024. ws: blr_conv_silu_workspace bytes, backward only. No
+ * output may overlap an input. An empty problem is a no-op.
+ */
+BLR_API size_t blr_conv_silu_workspace(int64_t B, int64_t L, int64_t C);
+BLR_API blr_status blr_conv_silu_fwd(int64_t B, int64_t L, int64_t C, blr_dtype io, const void* hxz,
+                                     const void* weight, const void* bias, void* x, void* z,
+                                     blr_stream_t stream);
+BLR_API blr_status blr_conv_silu_bwd(int64_t B, int64_t L, int64_t C, blr_dtype io, const void* dx,
+                                     const void* dz, const void* hxz, const void* weight,
+                                     const void* bias, void* dhxz, void* dweight, void* dbias,
+                                     void* ws, size_t ws_bytes, blr_stream_t stream);
+
+/*
+ * The layer's linear projections in float32 arithmetic: y = x weight^T + bias
+ * for x (T, K), weight (N, K), bias (N) or NULL, y (T, N). The backward writes
+ * dx = dy weight (added to dx where add_dx is nonzero; dx may be NULL: not
+ * computed; weight is then not read) and
+ * dweight = dy^T x with dbias = the column sums of dy (dweight may be NULL:
+ * neither is computed; x, dbias and ws are then not used). N % 4 == 0, K % 4 == 0.
+ * ws: blr_linear_workspace bytes. No output may overlap an input. An empty
+ * problem is a no-op (nothing is written).
+ */
+BLR_API size_t blr_linear_workspace(int64_t T, int64_t N, int64_t K);
+BLR_API blr_status blr_linear_fwd(int64_t T, int64_t N, int64_t K, const float* x,
+                                  const float* weight, const float* bias, float* y,
+                                  blr_stream_t stream);
+BLR_API blr_status blr_linear_bwd(int64_t T, int64_t N, int64_t K, const float* dy, const float* x,
+                                  const float* weight, float* dx, int add_dx, float* dweight,
+                                  float* dbias, void* ws, size_t ws_bytes, blr_stream_t stream);
+
+/*
  * Synchronises `stream`, then reads the error word that the kernels of
  * earlier calls on this workspace recorded: BLR_OK, BLR_ERR_TIMEOUT or
  * BLR_ERR_WORKSPACE (BLR_ERR_CUDA if the read itself fails). The word is

@@ -189,6 +189,42 @@ def blr_steps(B, K, D, io, state, c, h_prev, x, gate_logits, lam, h_out, h_seq=N
            "blr_steps")
 
 
+def blr_conv_silu_workspace(B: int, L: int, C: int) -> int:
+    return int(load().blr_conv_silu_workspace(B, L, C))
+
+
+def blr_conv_silu_fwd(B, L, C, io, hxz, weight, bias, x, z, stream=None):
+    """x = SiLU(causal 4-tap depthwise convolution of hxz[..., :C]), z = hxz[..., C:]."""
+    _check(load().blr_conv_silu_fwd(B, L, C, io, _ptr(hxz, "hxz"), _ptr(weight, "weight"),
+                                    _ptr(bias, "bias"), _ptr(x, "x"), _ptr(z, "z"),
+                                    _stream(stream)), "blr_conv_silu_fwd")
+
+
+def blr_conv_silu_bwd(B, L, C, io, dx, dz, hxz, weight, bias, dhxz, dweight, dbias, ws, stream=None):
+    _check(load().blr_conv_silu_bwd(B, L, C, io, _ptr(dx, "dx"), _ptr(dz, "dz"), _ptr(hxz, "hxz"),
+                                    _ptr(weight, "weight"), _ptr(bias, "bias"), _ptr(dhxz, "dhxz"),
+                                    _ptr(dweight, "dweight"), _ptr(dbias, "dbias"), _ptr(ws, "ws"),
+                                    ws.numel(), _stream(stream)), "blr_conv_silu_bwd")
+
+
+def blr_linear_workspace(T: int, N: int, K: int) -> int:
+    return int(load().blr_linear_workspace(T, N, K))
+
+
+def blr_linear_fwd(T, N, K, x, weight, bias, y, stream=None):
+    """y = x weight^T + bias in float32."""
+    _check(load().blr_linear_fwd(T, N, K, _ptr(x, "x"), _ptr(weight, "weight"), _ptr(bias, "bias"),
+                                 _ptr(y, "y"), _stream(stream)), "blr_linear_fwd")
+
+
+def blr_linear_bwd(T, N, K, dy, x, weight, dx, dweight, dbias, ws, add_dx=False, stream=None):
+    """dx (or None; added to it with add_dx), and dweight with dbias (or None)."""
+    _check(load().blr_linear_bwd(T, N, K, _ptr(dy, "dy"), _ptr(x, "x"), _ptr(weight, "weight"),
+                                 _ptr(dx, "dx"), add_dx, _ptr(dweight, "dweight"), _ptr(dbias, "dbias"),
+                                 _ptr(ws, "ws"), ws.numel() if ws is not None else 0,
+                                 _stream(stream)), "blr_linear_bwd")
+
+
 def blr_workspace_status(desc, ws, stream=None) -> int:
     """Status recorded in the workspace by earlier calls (synchronises the
     stream); ws None reads the library's scratch (backward calls made without a

@@ -55,6 +55,16 @@ SIGNATURES = {
                                  _VP, _VP, _SZ, _VP]),
 }
 
+_I64 = ctypes.c_int64
+SIGNATURES.update({
+    "blr_conv_silu_workspace": (_SZ, [_I64] * 3),
+    "blr_conv_silu_fwd": (_ST, [_I64, _I64, _I64, ctypes.c_int] + [_VP] * 6),
+    "blr_conv_silu_bwd": (_ST, [_I64, _I64, _I64, ctypes.c_int] + [_VP] * 9 + [_SZ, _VP]),
+    "blr_linear_workspace": (_SZ, [_I64] * 3),
+    "blr_linear_fwd": (_ST, [_I64] * 3 + [_VP] * 5),
+    "blr_linear_bwd": (_ST, [_I64] * 3 + [_VP] * 4 + [ctypes.c_int] + [_VP] * 3 + [_SZ, _VP]),
+})
+
 _lock = threading.Lock()
 _lib = None
 

@@ -12,6 +12,7 @@
 #include <cudaTypedefs.h>
 
 #include "blr.h"
+#include "blr_layer.cuh"
 #include "blr_seq.cuh"
 #include "blr_team_bwd.cuh"
 
@@ -207,10 +208,10 @@ blr_status launch_cooperative(K kernel, unsigned grid, int threads, size_t smem,
 // the stream finishes (programmatic dependent launch): the kernel itself waits
 // for that one (griddepcontrol.wait) before it touches global memory.
 template <typename K, typename A>
-blr_status launch_overlapped(K kernel, unsigned grid, dim3 threads, size_t smem, cudaStream_t st,
+blr_status launch_overlapped(K kernel, dim3 grid, dim3 threads, size_t smem, cudaStream_t st,
                           const A& args, const char* what) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
+  cfg.gridDim = grid;
   cfg.blockDim = threads;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
@@ -732,6 +733,173 @@ blr_status blr_steps(int64_t B, int64_t K, int64_t D, blr_dtype io, blr_dtype st
     return state == BLR_F32 ? launch(blr::steps_kernel<float, float, 4>)
                             : launch(blr::steps_kernel<float, bf, 4>);
   return state == BLR_F32 ? launch(blr::steps_kernel<bf, float, 8>) : launch(blr::steps_kernel<bf, bf, 8>);
+}
+
+// ------------------------------------------------ gated layer: conv and SiLU
+
+}  // extern "C"
+
+namespace {
+
+constexpr int kConvVec = 4;  // channels a thread: 16 bytes float32, 8 bytes bfloat16
+
+blr_status check_conv(int64_t B, int64_t L, int64_t C, blr_dtype io, bool* empty) {
+  if (B < 0 || L < 0 || C < 0) return fail(BLR_ERR_INVALID_ARG, "negative size");
+  if (io != BLR_F32 && io != BLR_BF16) return fail(BLR_ERR_INVALID_ARG, "unknown io dtype %d", (int)io);
+  if (C % 8 != 0) return fail(BLR_ERR_UNSUPPORTED, "C=%lld is not a multiple of 8", (long long)C);
+  *empty = B == 0 || L == 0 || C == 0;
+  if (*empty) return BLR_OK;
+  if (C > 1024 || B > ((int64_t)1 << 30) || L > ((int64_t)1 << 30) ||
+      (double)B * (double)L * (double)C > 1e11)
+    return fail(BLR_ERR_UNSUPPORTED, "problem too large");
+  return BLR_OK;
+}
+
+int64_t conv_chunks(int64_t L) { return (L + blr::kConvRows - 1) / blr::kConvRows; }
+int64_t conv_blocks(int64_t B, int64_t L, int64_t C) {
+  return (B * conv_chunks(L) * (C / kConvVec) + blr::kConvThreads - 1) / blr::kConvThreads;
+}
+
+blr_status launch_sum(blr_dtype io, const blr::SumArgs& a, cudaStream_t st) {
+  const unsigned grid = (unsigned)((a.size + 31) / 32);
+  if (io == BLR_F32)
+    return launch_overlapped(blr::sum_parts_kernel<float>, grid, dim3(blr::kSumThreads), 0, st, a, "launch sum_parts_kernel");
+  return launch_overlapped(blr::sum_parts_kernel<__nv_bfloat16>, grid, dim3(blr::kSumThreads), 0, st, a,
+                           "launch sum_parts_kernel");
+}
+
+// Splits of the long sum of a weight gradient: about three blocks an SM.
+int64_t wgrad_splits(int64_t T, int64_t N, int64_t K) {
+  const int64_t tiles = ((N + blr::kGemmM - 1) / blr::kGemmM) * ((K + blr::kGemmN - 1) / blr::kGemmN);
+  int64_t s = 3 * 152 / tiles;
+  const int64_t most = (T + 127) / 128;
+  if (s > most) s = most;
+  return s > 1 ? s : 1;
+}
+
+template <int FORM>
+blr_status launch_gemm(const blr::GemmArgs& a, int64_t splits, cudaStream_t st) {
+  const int64_t gx = (a.M + blr::kGemmM - 1) / blr::kGemmM, gy = (a.N + blr::kGemmN - 1) / blr::kGemmN;
+  return launch_overlapped(blr::gemm_f32_kernel<FORM>, dim3((unsigned)gx, (unsigned)gy, (unsigned)splits),
+                           dim3(128), 0, st, a, "launch gemm_f32_kernel");
+}
+
+blr_status check_linear(int64_t T, int64_t N, int64_t K, bool* empty) {
+  if (T < 0 || N < 0 || K < 0) return fail(BLR_ERR_INVALID_ARG, "negative size");
+  if (N % 4 != 0 || K % 4 != 0) return fail(BLR_ERR_UNSUPPORTED, "N and K must be multiples of 4");
+  *empty = T == 0 || N == 0 || K == 0;
+  if (T > ((int64_t)1 << 37) || N > 65536 || K > 65536) return fail(BLR_ERR_UNSUPPORTED, "problem too large");
+  return BLR_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
+size_t blr_conv_silu_workspace(int64_t B, int64_t L, int64_t C) {
+  bool empty = false;
+  if (check_conv(B, L, C, BLR_F32, &empty) != BLR_OK || empty) return 0;
+  return (size_t)conv_blocks(B, L, C) * (size_t)C * (blr::kConvWidth + 1) * sizeof(float);
+}
+
+blr_status blr_conv_silu_fwd(int64_t B, int64_t L, int64_t C, blr_dtype io, const void* hxz,
+                             const void* weight, const void* bias, void* x, void* z,
+                             blr_stream_t stream) {
+  bool empty = false;
+  BLR_TRY(check_conv(B, L, C, io, &empty));
+  if (empty) return BLR_OK;
+  BLR_TRY(need(hxz, "hxz", 16));
+  BLR_TRY(need(weight, "weight", 4));
+  BLR_TRY(need(bias, "bias", 4));
+  BLR_TRY(need(x, "x", 16));
+  BLR_TRY(need(z, "z", 16));
+  const blr::ConvArgs a{B, L, C, conv_chunks(L), hxz, weight, bias, x, z, nullptr, nullptr};
+  const unsigned grid = (unsigned)conv_blocks(B, L, C);
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  if (io == BLR_F32)
+    return launch_overlapped(blr::conv_silu_fwd_kernel<float, kConvVec>, grid, dim3(blr::kConvThreads), 0, st, a,
+                             "launch conv_silu_fwd_kernel");
+  return launch_overlapped(blr::conv_silu_fwd_kernel<__nv_bfloat16, kConvVec>, grid, dim3(blr::kConvThreads), 0, st, a,
+                           "launch conv_silu_fwd_kernel");
+}
+
+blr_status blr_conv_silu_bwd(int64_t B, int64_t L, int64_t C, blr_dtype io, const void* dx,
+                             const void* dz, const void* hxz, const void* weight, const void* bias,
+                             void* dhxz, void* dweight, void* dbias, void* ws, size_t ws_bytes,
+                             blr_stream_t stream) {
+  bool empty = false;
+  BLR_TRY(check_conv(B, L, C, io, &empty));
+  if (empty) return BLR_OK;
+  BLR_TRY(need(dx, "dx", 16));
+  BLR_TRY(need(dz, "dz", 16));
+  BLR_TRY(need(hxz, "hxz", 16));
+  BLR_TRY(need(weight, "weight", 4));
+  BLR_TRY(need(bias, "bias", 4));
+  BLR_TRY(need(dhxz, "dhxz", 16));
+  BLR_TRY(need(dweight, "dweight", 4));
+  BLR_TRY(need(dbias, "dbias", 4));
+  BLR_TRY(need(ws, "ws", 16));
+  if (ws_bytes < blr_conv_silu_workspace(B, L, C)) return fail(BLR_ERR_INVALID_ARG, "workspace too small");
+  const blr::ConvArgs a{B, L, C, conv_chunks(L), hxz, weight, bias, const_cast<void*>(dx),
+                        const_cast<void*>(dz), dhxz, static_cast<float*>(ws)};
+  const int64_t blocks = conv_blocks(B, L, C);
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  if (io == BLR_F32)
+    BLR_TRY(launch_overlapped(blr::conv_silu_bwd_kernel<float, kConvVec>, (unsigned)blocks,
+                              dim3(blr::kConvThreads), 0, st,
+                              a, "launch conv_silu_bwd_kernel"));
+  else
+    BLR_TRY(launch_overlapped(blr::conv_silu_bwd_kernel<__nv_bfloat16, kConvVec>, (unsigned)blocks,
+                              dim3(blr::kConvThreads), 0, st, a, "launch conv_silu_bwd_kernel"));
+  return launch_sum(io, blr::SumArgs{a.part, blocks, C * (blr::kConvWidth + 1), 0, blr::kConvWidth + 1,
+                                     dweight, dbias}, st);
+}
+
+// -------------------------------------------- gated layer: float32 projections
+
+size_t blr_linear_workspace(int64_t T, int64_t N, int64_t K) {
+  bool empty = false;
+  if (check_linear(T, N, K, &empty) != BLR_OK || empty) return 0;
+  return (size_t)wgrad_splits(T, N, K) * (size_t)(N * K + N) * sizeof(float);
+}
+
+blr_status blr_linear_fwd(int64_t T, int64_t N, int64_t K, const float* x, const float* weight,
+                          const float* bias, float* y, blr_stream_t stream) {
+  bool empty = false;
+  BLR_TRY(check_linear(T, N, K, &empty));
+  if (empty) return BLR_OK;
+  BLR_TRY(need(x, "x", 16));
+  BLR_TRY(need(weight, "weight", 16));
+  BLR_TRY(optional(bias, "bias", 16));
+  BLR_TRY(need(y, "y", 16));
+  const blr::GemmArgs a{T, N, K, 0, x, weight, bias, y, 0};
+  return launch_gemm<blr::kNT>(a, 1, reinterpret_cast<cudaStream_t>(stream));
+}
+
+blr_status blr_linear_bwd(int64_t T, int64_t N, int64_t K, const float* dy, const float* x,
+                          const float* weight, float* dx, int add_dx, float* dweight, float* dbias,
+                          void* ws, size_t ws_bytes, blr_stream_t stream) {
+  bool empty = false;
+  BLR_TRY(check_linear(T, N, K, &empty));
+  if (empty) return BLR_OK;
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  BLR_TRY(need(dy, "dy", 16));
+  if (dx != nullptr) {
+    BLR_TRY(need(weight, "weight", 16));
+    BLR_TRY(need(dx, "dx", 16));
+    BLR_TRY(launch_gemm<blr::kNN>(blr::GemmArgs{T, K, N, 0, dy, weight, nullptr, dx, add_dx}, 1, st));
+  }
+  if (dweight == nullptr) return BLR_OK;
+  BLR_TRY(need(x, "x", 16));
+  BLR_TRY(need(dbias, "dbias", 4));
+  BLR_TRY(need(ws, "ws", 16));
+  if (ws_bytes < blr_linear_workspace(T, N, K)) return fail(BLR_ERR_INVALID_ARG, "workspace too small");
+  int64_t splits = wgrad_splits(T, N, K);
+  const int64_t rows = ((T + splits - 1) / splits + blr::kGemmK - 1) / blr::kGemmK * blr::kGemmK;
+  splits = (T + rows - 1) / rows;
+  float* part = static_cast<float*>(ws);
+  BLR_TRY(launch_gemm<blr::kTN>(blr::GemmArgs{N, K, T, rows, dy, x, nullptr, part, 0}, splits, st));
+  return launch_sum(BLR_F32, blr::SumArgs{part, splits, N * K + N, N * K, 0, dweight, dbias}, st);
 }
 
 blr_status blr_workspace_status(const blr_desc* desc, const void* ws, size_t ws_bytes,

@@ -557,6 +557,12 @@ __device__ __forceinline__ void mbar_wait(uint64_t* bar, uint32_t parity, uint32
   }
 }
 
+// Requests a tensor map (a kernel parameter: constant, so it may be read before
+// the wait for the kernel before this one), so that its first use finds it cached.
+__device__ __forceinline__ void tensormap_prefetch(const void* tmap) {
+  asm volatile("prefetch.tensormap [%0];" ::"l"(tmap) : "memory");
+}
+
 // One 3-D tile load: box at (c0, c1, c2) of the tensor map into shared memory.
 __device__ __forceinline__ void tma_load_3d(void* dst, const void* tmap, uint64_t* bar, int c0,
                                             int c1, int c2) {

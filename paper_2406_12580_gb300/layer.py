@@ -6,8 +6,12 @@
     H'_y     = BD-LRU(H'_x) * SiLU(H_z)            blr_scan_fwd_gated: the scan and the merge, fused
     H_o      = Linear(H'_y)                        reduce E D -> D
 
-The GEMMs and the convolution are torch operators (cuBLAS, cuDNN); the scan and
-the merge, forward and backward, run in the library (``BDLRUGatedScan``). The
+The scan and the merge, forward and backward, run in the library
+(``BDLRUGatedScan``). So do the convolution with its SiLU (``blr_conv_silu_*``,
+float32 and bfloat16) and the float32 projections (``blr_linear_*``) on a CUDA
+device in plain eager execution; elsewhere (autocast, TF32 allowed, traced or
+transformed by functorch, forward-mode AD, tensor subclasses, other dtypes,
+devices or widths, hooks on the convolution) they are the torch operators. The
 decay parameter Lambda is initialised as in Sec. 3.2: exp(-softplus(Lambda))
 uniform in [0.9, 0.999]. The convolution width is not given in the paper; it
 is a parameter (default 4).
@@ -17,7 +21,9 @@ from __future__ import annotations
 import torch
 from torch import nn
 
-from . import (Desc, _dtype_code, blr_scan_bwd_gated, blr_scan_fwd_gated, blr_workspace_bytes)
+from . import (Desc, _dtype_code, blr_conv_silu_bwd, blr_conv_silu_fwd, blr_conv_silu_workspace,
+               blr_linear_bwd, blr_linear_fwd, blr_linear_workspace, blr_scan_bwd_gated,
+               blr_scan_fwd_gated, blr_workspace_bytes)
 
 
 class BDLRUGatedScan(torch.autograd.Function):
@@ -57,6 +63,188 @@ class BDLRUGatedScan(torch.autograd.Function):
         return dx, dgl, dlam.to(ctx.lam_dtype), dz, dh0, None
 
 
+def _plain_cuda(dtype, *tensors) -> bool:
+    """Whether the library's kernels may stand in for torch operators on these
+    tensors: ordinary CUDA tensors of one dtype on the current device, in eager
+    execution without autocast, functorch transforms or forward-mode AD."""
+    if (torch.is_autocast_enabled() or torch.compiler.is_compiling()
+            or torch._C._are_functorch_transforms_active()
+            or torch.autograd.forward_ad._current_level >= 0):
+        return False
+    for t in tensors:
+        if type(t) not in (torch.Tensor, nn.Parameter) or t.dtype != dtype or not t.is_cuda:
+            return False
+        if (t.layout != torch.strided or t.numel() == 0 or t.data_ptr() % 16 != 0
+                or t.get_device() != torch._C._cuda_getDevice()):
+            return False
+    return True
+
+
+def _differentiable(fn, inputs, grads):
+    """Gradients of torch operators, themselves differentiable (create_graph)."""
+    with torch.enable_grad():
+        outs = fn(*inputs)
+        outs = outs if isinstance(outs, tuple) else (outs,)
+        need = [t for t in inputs if t.requires_grad]
+        got = iter(torch.autograd.grad(outs, need, grads, create_graph=True))
+    return tuple(next(got) if t.requires_grad else None for t in inputs)
+
+
+def _linear_fwd(x, weight, bias):
+    N, K = weight.shape
+    y = x.new_empty(*x.shape[:-1], N)
+    blr_linear_fwd(x.numel() // K, N, K, x, weight, bias, y)
+    return y
+
+
+def _linear_bwd(dy, x, weight, dx, with_weight, add_dx=False):
+    """dx into `dx` (None: not computed); returns (dweight, dbias), or Nones."""
+    N, K = weight.shape
+    T = x.numel() // K
+    dw = db = ws = None
+    if with_weight:
+        dw, db = torch.empty_like(weight), weight.new_empty(N)
+        ws = torch.empty(blr_linear_workspace(T, N, K), dtype=torch.uint8, device=x.device)
+    if with_weight or dx is not None:
+        blr_linear_bwd(T, N, K, dy, x, weight, dx, dw, db, ws, add_dx)
+    return dw, db
+
+
+class _LinearF32(torch.autograd.Function):
+    """torch.nn.functional.linear on the library's float32 kernels."""
+
+    @staticmethod
+    def forward(ctx, x, weight, bias):
+        x, weight, bias = x.contiguous(), weight.contiguous(), bias.contiguous()
+        ctx.save_for_backward(x, weight, bias)
+        return _linear_fwd(x, weight, bias)
+
+    @staticmethod
+    def backward(ctx, dy):
+        x, weight, bias = ctx.saved_tensors
+        if torch.is_grad_enabled() or not _plain_cuda(torch.float32, dy, x, weight):
+            return _differentiable(nn.functional.linear, (x, weight, bias), (dy,))
+        dx = torch.empty_like(x) if ctx.needs_input_grad[0] else None
+        dw, db = _linear_bwd(dy.contiguous(), x, weight, dx, any(ctx.needs_input_grad[1:]))
+        return dx, dw if ctx.needs_input_grad[1] else None, db if ctx.needs_input_grad[2] else None
+
+
+class _Linear(nn.Linear):
+    """nn.Linear whose float32 product runs in the library (in float32: where
+    TF32 is allowed it stays with torch)."""
+
+    def forward(self, x):
+        if (self.bias is not None and self.weight.dtype == torch.float32
+                and self.in_features % 4 == 0 and self.out_features % 4 == 0
+                and x.dim() > 1 and x.shape[-1] == self.in_features
+                and not torch.backends.cuda.matmul.allow_tf32
+                and _plain_cuda(torch.float32, x, self.weight, self.bias)):
+            return _LinearF32.apply(x, self.weight, self.bias)
+        return super().forward(x)
+
+
+def _conv_silu_torch(hxz, weight, bias):
+    """(SiLU of the causal depthwise convolution of the first half, the second half)."""
+    hx, hz = hxz.chunk(2, dim=-1)
+    xc = nn.functional.conv1d(hx.transpose(1, 2), weight, bias, padding=weight.shape[-1] - 1,
+                              groups=weight.shape[0])[..., :hxz.shape[1]].transpose(1, 2)
+    return nn.functional.silu(xc).contiguous(), hz.contiguous()
+
+
+def _conv_fwd(hxz, weight, bias):
+    B, L, C2 = hxz.shape
+    x, z = hxz.new_empty(B, L, C2 // 2), hxz.new_empty(B, L, C2 // 2)
+    blr_conv_silu_fwd(B, L, C2 // 2, _dtype_code(hxz), hxz, weight, bias, x, z)
+    return x, z
+
+
+def _conv_bwd(dx, dz, hxz, weight, bias):
+    B, L, C2 = hxz.shape
+    dhxz, dw, db = torch.empty_like(hxz), torch.empty_like(weight), torch.empty_like(bias)
+    ws = torch.empty(blr_conv_silu_workspace(B, L, C2 // 2), dtype=torch.uint8, device=hxz.device)
+    blr_conv_silu_bwd(B, L, C2 // 2, _dtype_code(hxz), dx, dz, hxz, weight, bias, dhxz, dw, db, ws)
+    return dhxz, dw, db
+
+
+class _ConvSiLU(torch.autograd.Function):
+    """_conv_silu_torch on the library's kernels."""
+
+    @staticmethod
+    def forward(ctx, hxz, weight, bias):
+        hxz, weight, bias = hxz.contiguous(), weight.contiguous(), bias.contiguous()
+        ctx.save_for_backward(hxz, weight, bias)
+        return _conv_fwd(hxz, weight, bias)
+
+    @staticmethod
+    def backward(ctx, dx, dz):
+        hxz, weight, bias = ctx.saved_tensors
+        if torch.is_grad_enabled() or not _plain_cuda(hxz.dtype, dx, dz, hxz):
+            return _differentiable(_conv_silu_torch, (hxz, weight, bias), (dx, dz))
+        grads = _conv_bwd(dx.contiguous(), dz.contiguous(), hxz, weight, bias)
+        return tuple(g if n else None for g, n in zip(grads, ctx.needs_input_grad))
+
+
+def _layer_torch(c, h, w_in, b_in, w_conv, b_conv, w_gate, b_gate, lam, w_out, b_out):
+    """The layer's operators one by one (gradients of gradients)."""
+    x, z = _conv_silu_torch(nn.functional.linear(h, w_in, b_in), w_conv, b_conv)
+    y, _ = BDLRUGatedScan.apply(x, nn.functional.linear(x, w_gate, b_gate), lam, z, None, c)
+    return nn.functional.linear(y, w_out, b_out)
+
+
+class _LayerF32(torch.autograd.Function):
+    """The whole layer in float32 on the library's kernels: one node in the graph
+    instead of five, and the gate projection's gradient of the scan's input added
+    to the scan's in the kernel that computes it."""
+
+    @staticmethod
+    def forward(ctx, c, h, w_in, b_in, w_conv, b_conv, w_gate, b_gate, lam, w_out, b_out):
+        hxz = _linear_fwd(h.contiguous(), w_in, b_in)
+        x, z = _conv_fwd(hxz, w_conv, b_conv)
+        gl = _linear_fwd(x, w_gate, b_gate)
+        B, L, D = x.shape
+        desc = Desc(B, L, D, 0, c)
+        ws = torch.empty(blr_workspace_bytes(desc), dtype=torch.uint8, device=x.device)
+        y = torch.empty_like(x)
+        blr_scan_fwd_gated(desc, x, gl, lam, None, z, y, None, ws)
+        ctx.desc = desc
+        ctx.save_for_backward(h, w_in, b_in, w_conv, b_conv, w_gate, b_gate, lam, w_out, b_out,
+                              hxz, x, z, gl, y, ws)
+        return _linear_fwd(y, w_out, b_out)
+
+    @staticmethod
+    def backward(ctx, dout):
+        (h, w_in, b_in, w_conv, b_conv, w_gate, b_gate, lam, w_out, b_out,
+         hxz, x, z, gl, y, ws) = ctx.saved_tensors
+        need = ctx.needs_input_grad[1:]
+        if torch.is_grad_enabled() or not _plain_cuda(torch.float32, dout):
+            c = ctx.desc.c
+            return (None, *_differentiable(lambda *t: _layer_torch(c, *t),
+                                           (h, w_in, b_in, w_conv, b_conv, w_gate, b_gate, lam,
+                                            w_out, b_out), (dout,)))
+        dout, h = dout.contiguous(), h.contiguous()
+        dy = torch.empty_like(y)
+        dw_out, db_out = _linear_bwd(dout, y, w_out, dy, need[8] or need[9])
+        dx, dz, dgl, dlam = (torch.empty_like(t) for t in (x, z, gl, lam))
+        blr_scan_bwd_gated(ctx.desc, dy, None, x, gl, lam, None, z, dx, dgl, dz, dlam, None, ws)
+        dw_gate, db_gate = _linear_bwd(dgl, x, w_gate, dx, need[5] or need[6], add_dx=True)
+        dhxz, dw_conv, db_conv = _conv_bwd(dx, dz, hxz, w_conv, b_conv)
+        dh = torch.empty_like(h) if need[0] else None
+        dw_in, db_in = _linear_bwd(dhxz, h, w_in, dh, need[1] or need[2])
+        grads = (dh, dw_in, db_in, dw_conv, db_conv, dw_gate, db_gate, dlam, dw_out, db_out)
+        return (None, *(g if n else None for g, n in zip(grads, need)))
+
+
+_GLOBAL_HOOKS = ("_global_forward_hooks", "_global_forward_pre_hooks", "_global_backward_hooks",
+                 "_global_backward_pre_hooks")
+
+
+def _bare(module, kind) -> bool:
+    """Whether calling the module is its forward and nothing else."""
+    return (type(module) is kind and module.bias is not None and not module._forward_hooks
+            and not module._forward_pre_hooks and not module._backward_hooks
+            and not module._backward_pre_hooks and "forward" not in module.__dict__)
+
+
 def lambda_init(n: int, lo: float = 0.9, hi: float = 0.999, generator=None) -> torch.Tensor:
     """Lambda with exp(-softplus(Lambda)) ~ U[lo, hi] (Sec. 3.2)."""
     u = torch.rand(n, generator=generator, dtype=torch.float64) * (hi - lo) + lo
@@ -74,19 +262,48 @@ class GatedRecurrentLayer(nn.Module):
             raise ValueError("expand * d_model must be a multiple of 8")
         kw = dict(device=device, dtype=dtype)
         self.ed, self.c = ed, c
-        self.in_proj = nn.Linear(d_model, 2 * ed, **kw)         # H_x | H_z
+        self.in_proj = _Linear(d_model, 2 * ed, **kw)           # H_x | H_z
         self.conv = nn.Conv1d(ed, ed, conv_width, groups=ed, padding=conv_width - 1, **kw)
-        self.gate_proj = nn.Linear(ed, 2 * ed, **kw)            # rho | iota
-        self.out_proj = nn.Linear(ed, d_model, **kw)
+        self.gate_proj = _Linear(ed, 2 * ed, **kw)              # rho | iota
+        self.out_proj = _Linear(ed, d_model, **kw)
         self.lam = nn.Parameter(lambda_init(ed).to(device=device))
 
+    def _conv_ok(self) -> bool:
+        return (_bare(self.conv, nn.Conv1d) and self.conv.weight.shape == (self.ed, 1, 4)
+                and self.ed <= 1024)
+
+    def _conv_silu(self, hxz):
+        """The scan's inputs from the expansion's output: SiLU(conv(H_x)) and H_z."""
+        conv = self.conv
+        if (self._conv_ok() and hxz.dtype in (torch.float32, torch.bfloat16)
+                and _plain_cuda(hxz.dtype, hxz, conv.weight, conv.bias)):
+            return _ConvSiLU.apply(hxz, conv.weight, conv.bias)
+        hx, hz = hxz.split(self.ed, dim=-1)
+        xc = conv(hx.transpose(1, 2))[..., :hxz.shape[1]].transpose(1, 2)  # causal: drop the tail
+        return nn.functional.silu(xc).contiguous(), hz.contiguous()
+
+    def _whole(self, h):
+        """The layer's parameters if all of it can run as one function, else None."""
+        i, g, o = self.in_proj, self.gate_proj, self.out_proj
+        if not (self._conv_ok() and _bare(i, _Linear) and _bare(g, _Linear) and _bare(o, _Linear)):
+            return None
+        if (torch.backends.cuda.matmul.allow_tf32 or h.dim() != 3 or h.shape[-1] % 4 != 0
+                or h.shape[-1] != i.in_features or o.out_features % 4 != 0
+                or any(getattr(nn.modules.module, n) for n in _GLOBAL_HOOKS)):
+            return None
+        p = (i.weight, i.bias, self.conv.weight, self.conv.bias, g.weight, g.bias, self.lam,
+             o.weight, o.bias)
+        if not _plain_cuda(torch.float32, h, *p) or not all(t.is_contiguous() for t in p):
+            return None
+        return p
+
     def forward(self, h: torch.Tensor) -> torch.Tensor:
-        B, L, _ = h.shape
-        hx, hz = self.in_proj(h).split(self.ed, dim=-1)
-        xc = self.conv(hx.transpose(1, 2))[..., :L].transpose(1, 2)   # causal: drop the tail
-        x = nn.functional.silu(xc).contiguous()
+        params = self._whole(h)
+        if params is not None:
+            return _LayerF32.apply(self.c, h, *params)
+        x, z = self._conv_silu(self.in_proj(h))
         gl = self.gate_proj(x).contiguous()
-        y, _ = BDLRUGatedScan.apply(x, gl, self.lam, hz.contiguous(), None, self.c)
+        y, _ = BDLRUGatedScan.apply(x, gl, self.lam, z, None, self.c)
         return self.out_proj(y)
 
 
