@@ -67,18 +67,30 @@ def _dtype_code(t) -> int:
     raise TypeError(f"unsupported dtype {t.dtype}")
 
 
+_torch = None  # the torch module, once a call has needed it
+
+
+def _import_torch():
+    global _torch
+    import torch
+    _torch = torch
+    return torch
+
+
+# The calls below marshal up to 14 pointers each, on programs whose kernels take
+# a few microseconds: one attribute read per check, no imports or device objects.
 def _ptr(t, name: str):
     """Device pointer of a CUDA tensor on the current device (or a raw int / None)."""
     if t is None:
         return None
-    if isinstance(t, int):
-        return t
-    import torch
+    torch = _torch or _import_torch()
     if not isinstance(t, torch.Tensor):
+        if isinstance(t, int):
+            return t
         raise TypeError(f"{name}: expected a CUDA tensor, an int pointer or None")
     if t.numel() == 0:
         return None
-    if not t.is_cuda or t.device.index != torch.cuda.current_device():
+    if not t.is_cuda or t.get_device() != torch._C._cuda_getDevice():
         raise ValueError(f"{name}: tensor must be on the current CUDA device")
     if not t.is_contiguous():
         raise ValueError(f"{name}: tensor must be contiguous")
@@ -87,8 +99,10 @@ def _ptr(t, name: str):
 
 def _stream(stream):
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        torch = _torch or _import_torch()
+        if not torch.cuda.is_initialized():
+            return torch.cuda.current_stream().cuda_stream
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream

@@ -253,11 +253,24 @@ int seq_stages(int64_t n_chain, size_t stage_bytes) {
   return (int)s;
 }
 
+// Raises a kernel's limit of dynamic shared memory, once per device and kernel.
 template <typename K>
 blr_status allow_smem(K kernel, size_t smem) {
+  constexpr size_t kMost = 227u << 10;
   if (smem <= (48u << 10)) return BLR_OK;
-  return cuda_check(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-                    "set dynamic shared memory size");
+  static std::mutex m;
+  static struct { int dev; const void* fn; } done[128];
+  static int n = 0;
+  int dev = 0;
+  BLR_TRY(cuda_check(cudaGetDevice(&dev), "cudaGetDevice"));
+  const void* fn = reinterpret_cast<const void*>(kernel);
+  std::lock_guard<std::mutex> lock(m);
+  for (int i = 0; i < n; ++i)
+    if (done[i].dev == dev && done[i].fn == fn) return BLR_OK;
+  BLR_TRY(cuda_check(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMost),
+                     "set dynamic shared memory size"));
+  if (n < 128) done[n++] = {dev, fn};
+  return BLR_OK;
 }
 
 // float32 rings deep enough run the LATE form (refill after the next stage's
