@@ -299,6 +299,11 @@ __global__ void __launch_bounds__(32) seq_fwd_kernel(const __grid_constant__ Seq
   if (lane == 0) {
     for (int s = 0; s < ring.S; ++s) mbar_init(&ring.bars[s], 1);
     fence_mbar_init();
+    tensormap_prefetch(&a.tm_x);
+    tensormap_prefetch(&a.tm_r);
+    tensormap_prefetch(&a.tm_i);
+    if constexpr (GATED) tensormap_prefetch(&a.tm_z);
+    if (a.write_h) tensormap_prefetch(&a.tm_h);
   }
   pdl_wait();
   if (blockIdx.x == 0) seq_reset_workspace(a.ws, p, p.tag, lane);
@@ -607,6 +612,11 @@ __global__ void __launch_bounds__(32, sizeof(T) == 4 ? 8 : 16) seq_bwd_kernel(co
   if (lane == 0) {
     for (int s = 0; s < ring.S; ++s) mbar_init(&ring.bars[s], 1);
     fence_mbar_init();
+    tensormap_prefetch(&a.tm_dh);
+    tensormap_prefetch(&a.tm_x);
+    tensormap_prefetch(&a.tm_r);
+    tensormap_prefetch(&a.tm_i);
+    if constexpr (GATED) tensormap_prefetch(&a.tm_z);
   }
   pdl_wait();
   {

@@ -333,6 +333,11 @@ __global__ void __maxnreg__(kTeamMaxRegs)
       mbar_init(&maps_read[m], ns);
     }
     fence_mbar_init();
+    tensormap_prefetch(&a.tm_dh);
+    tensormap_prefetch(&a.tm_x);
+    tensormap_prefetch(&a.tm_r);
+    tensormap_prefetch(&a.tm_i);
+    if constexpr (GATED) tensormap_prefetch(&a.tm_z);
   }
   pdl_wait();
   {

@@ -170,6 +170,10 @@ __global__ void __maxnreg__(kTeamMaxRegs)
       mbar_init(&maps_read[m], ns);
     }
     fence_mbar_init();
+    tensormap_prefetch(&a.tm_x);
+    tensormap_prefetch(&a.tm_r);
+    tensormap_prefetch(&a.tm_i);
+    if constexpr (GATED) tensormap_prefetch(&a.tm_z);
   }
   __syncthreads();  // the roles part here and meet again at the end
   pdl_wait();
