@@ -15,10 +15,11 @@ __device__ __forceinline__ uint32_t smem_addr(const void* p) {
   return (uint32_t)__cvta_generic_to_shared(p);
 }
 
-// Waits for the grid this one was launched behind (programmatic dependent
-// launch) and lets the next one start its own prologue; no-ops without it.
-__device__ __forceinline__ void pdl_wait() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+// Programmatic dependent launch (no-ops without it): pdl_wait waits for the grid
+// this one was launched behind; pdl_release lets the next one start, whose
+// blocks then take the places that this grid's leave, up to its own pdl_wait.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_release() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 

@@ -49,6 +49,7 @@ __global__ void __launch_bounds__(256, kStepBlocksPerSm) step_kernel(const StepA
   using IO = Io<T, VEC>;
   __shared__ float s_k[64 * 8];
   pdl_wait();
+  pdl_release();
   const int64_t vg = blockIdx.x % a.n_vgroups;
   const int64_t rg = blockIdx.x / a.n_vgroups;
   const int64_t n_rg = gridDim.x / a.n_vgroups;  // the grid launches whole channel groups
@@ -263,6 +264,7 @@ template <typename T, typename S, int VEC>
 __global__ void __launch_bounds__(256, kStepsBlocksPerSm) steps_kernel(const StepsArgs a) {
   __shared__ float s_k[64 * 8];
   pdl_wait();
+  pdl_release();
   const int64_t vg = blockIdx.x % a.n_vgroups;
   const int64_t rg = blockIdx.x / a.n_vgroups;
   const int64_t n_rg = gridDim.x / a.n_vgroups;  // the grid launches whole channel groups

@@ -69,6 +69,7 @@ __global__ void __launch_bounds__(kConvThreads, 4) conv_silu_fwd_kernel(const Co
   using IO = Io<T, VEC>;
   constexpr int H = kConvWidth - 1;
   pdl_wait();
+  pdl_release();
   const int64_t nv = a.C / VEC;
   const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t unit = idx / nv, c0 = (idx - unit * nv) * VEC;
@@ -129,6 +130,7 @@ __global__ void __launch_bounds__(kConvThreads, 3) conv_silu_bwd_kernel(const Co
   constexpr int NS = (W + 1) * VEC;  // a thread's sums: dw and db of its channels
   __shared__ float red[kConvThreads][VEC];
   pdl_wait();
+  pdl_release();
   const int64_t nv = a.C / VEC;
   const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t unit = idx / nv, c0 = (idx - unit * nv) * VEC;
@@ -254,6 +256,7 @@ __global__ void __launch_bounds__(kSumThreads) sum_parts_kernel(const SumArgs s_
   T* b = static_cast<T*>(s_.b);
   __shared__ float red[kSumThreads / 32][33];
   pdl_wait();
+  pdl_release();
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int64_t i = blockIdx.x * (int64_t)32 + tx;
   float s = 0.0f;
@@ -314,6 +317,7 @@ __global__ void __launch_bounds__(128, 3) gemm_f32_kernel(const GemmArgs a) {
   __shared__ __align__(16) float sA[2][BK][PA];
   __shared__ __align__(16) float sB[2][BK][PB];
   pdl_wait();
+  pdl_release();
   const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
   const int64_t m0 = (int64_t)blockIdx.x * BM, n0 = (int64_t)blockIdx.y * BN;
   const int64_t k_lo = FORM == kTN ? blockIdx.z * a.k_split : 0;

@@ -30,8 +30,11 @@
 // no preparation kernel runs before either scan. Both kernels set their
 // barriers up and then wait for the kernel before them on the stream
 // (programmatic dependent launch), so that back-to-back calls do not pay the
-// launch: 256 x 200 x 64 float32 fwd + bwd 41.9 -> 39.0 us, 1000 x 200 x 64
-// bfloat16 with lengths 67.2 -> 62.1.
+// launch: 256 x 200 x 64 float32 fwd + bwd 41.9 -> 37.7 us, 1000 x 200 x 64
+// bfloat16 with lengths 67.0 -> 60.5. They release the next kernel when their
+// last row is done, not at their start: a grid let in early fills the SMs that
+// have room first and runs unevenly (1500 x 800 x 64 bfloat16 364 against
+// 292 us).
 #pragma once
 
 #include "blr_kernels.cuh"
@@ -388,6 +391,7 @@ __global__ void __launch_bounds__(32) seq_fwd_kernel(const __grid_constant__ Seq
       phase ^= 1u;
     }
   }
+  pdl_release();
   if (lane == 0 && a.write_h) bulk_wait_all();
   if (a.h_last != nullptr && ch_ok) {
 #pragma unroll
@@ -764,6 +768,7 @@ __global__ void __launch_bounds__(32, sizeof(T) == 4 ? 8 : 16) seq_bwd_kernel(co
       phase ^= 1u;
     }
   }
+  pdl_release();
   if (lane == 0) bulk_wait_all();
 
   double* acc = reinterpret_cast<double*>(a.ws + p.off_dlam);

@@ -340,6 +340,7 @@ __global__ void __maxnreg__(kTeamMaxRegs)
     if constexpr (GATED) tensormap_prefetch(&a.tm_z);
   }
   pdl_wait();
+  pdl_release();
   {
     __shared__ int s_ok;
     if (threadIdx.x == 0) {

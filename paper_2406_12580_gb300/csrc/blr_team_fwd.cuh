@@ -177,6 +177,7 @@ __global__ void __maxnreg__(kTeamMaxRegs)
   }
   __syncthreads();  // the roles part here and meet again at the end
   pdl_wait();
+  pdl_release();
   if (blockIdx.x == 0 && warp == 0) seq_reset_workspace(a.ws, p, a.tag, lane);
 
   if (scanner) {
