@@ -481,8 +481,6 @@ blr_status scan_bwd_team(const Plan& plan, const void* dh, const float* dh_last,
   else memset(&a.tm_z, 0, sizeof(a.tm_z));
   a.p = plan;
   a.lengths = lengths;
-  a.dy = dh;
-  a.z = z;
   a.dz = dz;
   a.dh_last = dh_last;
   a.lambda = lambda;

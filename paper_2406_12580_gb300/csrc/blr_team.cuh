@@ -37,7 +37,7 @@
 // What bounds them: HBM bandwidth for float32 (8 x 8192 x 512 fwd + bwd 261 us,
 // 0.84 of the measured copy rate on the compulsory bytes), and for bfloat16 a
 // mix of issue slots (60 % of cycles) and bandwidth (8 x 32768 x 512 fwd + bwd
-// 530 us, 0.82; with the merge 784 us, 0.71). Slices of 16 steps: the fixed cost
+// 530 us, 0.82; with the merge 671 us, 0.83). Slices of 16 steps: the fixed cost
 // of a slice (waits, TMEM transfers, map, addresses) is spread over twice the
 // steps of an 8-step slice, and the kept states take half the bytes. 8 warps a
 // team: one 16-warp team of 8-step slices idles whenever its carry is late.

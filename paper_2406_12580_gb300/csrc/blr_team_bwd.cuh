@@ -26,8 +26,8 @@
 //             slice of x, rho and iota (ring C) and moves it by itself: a TMA
 //             store sends the outputs out, and during the next pass A, when
 //             the store has read them, the next tile's slice is requested.
-//             GATED: dy and z are read again (from L2) for dz = dy h SiLU'(z),
-//             written directly.
+//             GATED: dz = dy SiLU'(z) h is written directly, dy SiLU'(z) having
+//             been parked by pass A.
 // The gradient formulas are those of the serial backward kernels (the chain
 // rule of Sec. 3.2's definitions).
 //
@@ -57,9 +57,7 @@ struct TeamBwdArgs {
   CUtensorMap tm_di;
   Plan p;
   const int32_t* lengths;  // as TeamFwdArgs
-  const void* dy;          // gated: dy, z and dz
-  const void* z;
-  void* dz;
+  void* dz;                // gated
   const float* dh_last;
   const float* lambda;
   const float* h0;
@@ -93,17 +91,25 @@ struct TeamBwdSmem {
 // Pass A, one part of a slice (16 TMEM columns), last row first; rows from
 // `valid` on lie past the sequence and act as the identity (alpha = 1,
 // dh = 0). (w, m): the fold of the slice's later rows, zero at the slice's
-// end; on return the map of the rows folded so far. bfloat16: 4 rows, two
-// channels a lane, park[4r ..] = (g.x, sm.x, g.y, sm.y).
+// end; on return the map of the rows folded so far. GATED: dh = dy SiLU(z), and
+// merge gets dy SiLU'(z) of every element. bfloat16: 4 rows, two channels a
+// lane, park[4r ..] = (g.x, sm.x, g.y, sm.y).
 template <bool FAST, bool GATED, uint32_t BOX>
 __device__ __forceinline__ void team_rfold_bf16(const unsigned char* lb, float2 kh, int valid,
-                                                float2& w, float2& m, float (&park)[16]) {
+                                                float2& w, float2& m, float (&park)[16],
+                                                float (&merge)[8]) {
 #pragma unroll
   for (int r = 3; r >= 0; --r) {
     float2 dh = bf2_unpack(lds_u32(lb + r * 128));
-    if constexpr (GATED) {  // dh = dy SiLU(z)
-      const float2 hz = bf2_scaled(lds_u32(lb + 2 * BOX + r * 128), kBf2Half);
-      dh = __fmul2_rn(dh, __ffma2_rn(hz, tanh2(hz), hz));
+    if constexpr (GATED) {  // with hz = z/2 and th = tanh(hz), as silu_grad
+      const float2 hz = bf2_scaled(lds_u32(lb + 2 * BOX + r * 128), kBf2Half), th = tanh2(hz);
+      const float2 sg = __ffma2_rn(f2(0.5f), th, f2(0.5f));
+      const float2 f = __ffma2_rn(hz, th, hz);
+      const float2 df = __ffma2_rn(sg, __ffma2_rn(__fmul2_rn(f2(-1.0f), hz), th, hz), sg);
+      const float2 pd = __fmul2_rn(dh, df);
+      merge[2 * r] = pd.x;
+      merge[2 * r + 1] = pd.y;
+      dh = __fmul2_rn(dh, f);
     }
     const float2 hr = bf2_scaled(lds_u32(lb + BOX + r * 128), kBf2Half);
     float2 e = expm1_neg2<FAST>(__ffma2_rn(kh, tanh2(hr), kh));
@@ -124,13 +130,17 @@ __device__ __forceinline__ void team_rfold_bf16(const unsigned char* lb, float2 
 // float32: 8 rows of one channel by row pairs; park[2r ..] = (g, sm).
 template <bool FAST, bool GATED, uint32_t BOX>
 __device__ __forceinline__ void team_rfold_f32(const unsigned char* lb, float2 k, int valid,
-                                               float& w, float& m, float (&park)[16]) {
+                                               float& w, float& m, float (&park)[16],
+                                               float (&merge)[8]) {
 #pragma unroll
   for (int j = 3; j >= 0; --j) {
     float2 dh = lds_rows2(lb + j * 256);
     if constexpr (GATED) {
-      const float2 z = lds_rows2(lb + 2 * BOX + j * 256);
-      dh = __fmul2_rn(dh, __fmul2_rn(z, sigmoid2(z)));
+      const float2 z = lds_rows2(lb + 2 * BOX + j * 256), sg = sigmoid2(z), f = __fmul2_rn(z, sg);
+      const float2 pd = __fmul2_rn(dh, __ffma2_rn(sg, __ffma2_rn(f2(-1.0f), f, z), sg));
+      merge[2 * j] = pd.x;
+      merge[2 * j + 1] = pd.y;
+      dh = __fmul2_rn(dh, f);
     }
     float2 e = expm1_neg2_precise<FAST>(__fmul2_rn(k, sigmoid2(lds_rows2(lb + BOX + j * 256))));
     if (!FAST && 2 * j >= valid) e.x = dh.x = 0.0f;
@@ -149,25 +159,6 @@ __device__ __forceinline__ void team_rfold_f32(const unsigned char* lb, float2 k
   }
 }
 
-// Gated pass C: the raw words of dy and z of a part's rows, and where the next
-// rows' are (byte offset `off`, in rows left `left`). A row's words are replaced
-// by those of the row PR later as soon as they are used.
-template <int PR>
-struct GateRows {
-  uint32_t dy[PR], z[PR];
-  const unsigned char *dy_base, *z_base;
-  int64_t off;
-  int left;  // rows of the slice not yet requested
-  __device__ __forceinline__ void load(int r, int64_t pitch) {
-    if (left > 0) {
-      dy[r] = __ldcs(reinterpret_cast<const uint32_t*>(dy_base + off));
-      z[r] = __ldcs(reinterpret_cast<const uint32_t*>(z_base + off));
-    }
-    off += pitch;
-    --left;
-  }
-};
-
 // Pass C, one part of a slice: its rows forward in time from the state hp
 // before them (updated), with the parked (gl, sm) in pr and the adjoint win
 // entering the slice; dx, d rho and d iota overwrite x, rho and iota in the
@@ -178,7 +169,7 @@ struct GateRows {
 template <bool FAST, bool GATED, uint32_t BOX>
 __device__ __forceinline__ void team_rows_bf16(unsigned char* lb, const uint32_t (&pr)[16], float2 win,
                                                float2 kh, int rows, float2& hp, float2& dlr,
-                                               GateRows<4>& gr, unsigned char*& dz, int64_t pitch) {
+                                               const uint32_t (&merge)[8], unsigned char*& dz, int64_t pitch) {
 #pragma unroll
   for (int r = 0; r < 4; ++r) {
     const float2 gl = make_float2(__uint_as_float(pr[4 * r]), __uint_as_float(pr[4 * r + 2]));
@@ -210,25 +201,18 @@ __device__ __forceinline__ void team_rows_bf16(unsigned char* lb, const uint32_t
     *reinterpret_cast<uint32_t*>(lb + 2 * BOX + r * 128) = bf2_pack(oi);
     if (FAST || r < rows) {
       dlr = __ffma2_rn(dl, __ffma2_rn(f2(0.5f), thr, f2(0.5f)), dlr);  // += d l r
-      if constexpr (GATED) {  // dz = dy h SiLU'(z), with hz = z/2 and th = tanh(hz) as silu_grad
-        const float2 hz = bf2_scaled(gr.z[r], kBf2Half), th = tanh2(hz);
-        const float2 sg = __ffma2_rn(f2(0.5f), th, f2(0.5f));
-        const float2 nh = __fmul2_rn(f2(-1.0f), hz);
-        const float2 df = __ffma2_rn(sg, __ffma2_rn(nh, th, hz), sg);
-        const float2 o = __fmul2_rn(__fmul2_rn(bf2_unpack(gr.dy[r]), hp), df);
-        __stcs(reinterpret_cast<unsigned int*>(dz), bf2_pack(o));
+      if constexpr (GATED) {  // dz = dy SiLU'(z) h
+        const float2 pd = make_float2(__uint_as_float(merge[2 * r]), __uint_as_float(merge[2 * r + 1]));
+        __stcs(reinterpret_cast<unsigned int*>(dz), bf2_pack(__fmul2_rn(pd, hp)));
       }
     }
-    if constexpr (GATED) {
-      dz += pitch;
-      gr.load(r, pitch);
-    }
+    if constexpr (GATED) dz += pitch;
   }
 }
 template <bool FAST, bool GATED, uint32_t BOX>
 __device__ __forceinline__ void team_rows_f32(unsigned char* lb, const uint32_t (&pr)[16], float win,
                                               float2 k, int rows, float& hp, float& dlr,
-                                              GateRows<8>& gr, unsigned char*& dz, int64_t pitch) {
+                                              const uint32_t (&merge)[8], unsigned char*& dz, int64_t pitch) {
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     const float2 gl = make_float2(__uint_as_float(pr[4 * j]), __uint_as_float(pr[4 * j + 2]));
@@ -262,15 +246,9 @@ __device__ __forceinline__ void team_rows_f32(unsigned char* lb, const uint32_t 
     si[0] = oi.x;
     si[32] = oi.y;
     float2 oz = f2(0.0f);
-    if constexpr (GATED) {  // dz = dy h SiLU'(z)
-      const float2 z = make_float2(__uint_as_float(gr.z[2 * j]), __uint_as_float(gr.z[2 * j + 1]));
-      const float2 dy = make_float2(__uint_as_float(gr.dy[2 * j]), __uint_as_float(gr.dy[2 * j + 1]));
-      const float2 sg = sigmoid2(z);
-      const float2 f = __fmul2_rn(z, sg);
-      const float2 df = __ffma2_rn(sg, __ffma2_rn(f2(-1.0f), f, z), sg);
-      oz = __fmul2_rn(__fmul2_rn(dy, make_float2(h1, hp)), df);
-      gr.load(2 * j, pitch);
-      gr.load(2 * j + 1, pitch);
+    if constexpr (GATED) {  // dz = dy SiLU'(z) h
+      const float2 pd = make_float2(__uint_as_float(merge[2 * j]), __uint_as_float(merge[2 * j + 1]));
+      oz = __fmul2_rn(pd, make_float2(h1, hp));
     }
     if (FAST || 2 * j < rows) {
       dlr = fmaf(dl.x, r.x, dlr);
@@ -293,8 +271,16 @@ __global__ void __maxnreg__(kTeamMaxRegs)
   constexpr int VEC = team_vec<T>(), CHW = 32 * VEC, NW = kTeamWidth;
   constexpr int MS = kTeamSlots, TS = kTeamSlice, NBA = SM::NBA;
   constexpr uint32_t BOX = kTeamBox;
-  constexpr uint32_t COLS = team_cols<T>();
-  constexpr int NP = COLS / 16, PR = TS / NP;  // TMEM parts of a slice, rows per part
+  // TMEM columns of a slot: the parked (gl, sm), and dy SiLU'(z) when gated. Two
+  // slots let pass C run a tile behind pass A; the gated bfloat16 states take
+  // more than half of the TMEM, so there pass C follows its own pass A and the
+  // block's other team fills the wait for the carry.
+  constexpr uint32_t COLS = team_cols<T>() + (GATED ? TS * VEC : 0);
+  constexpr int LAG = GATED && !F32 ? 0 : 1;
+  constexpr uint32_t TSLOTS = LAG + 1;
+  constexpr uint32_t TCOLS = 4 * TSLOTS * COLS <= 256 ? 256 : 512;
+  constexpr int NP = team_cols<T>() / 16, PR = TS / NP;  // TMEM parts of a slice, rows per part
+  static_assert(PR * VEC == 8 && 4 * TSLOTS * COLS <= TCOLS, "a part's merge values are 8 columns");
   const Plan& p = a.p;
   extern __shared__ unsigned char team_smem[];
   unsigned char* base = align128(team_smem);
@@ -351,7 +337,7 @@ __global__ void __maxnreg__(kTeamMaxRegs)
     if (!s_ok) return;  // no forward states for this problem: write nothing
   }
   if (warp == 0) {  // the block's TMEM, freed by this warp after the final barrier
-    tmem_alloc(tslot, team_tmem_cols<T>());
+    tmem_alloc(tslot, TCOLS);
     tmem_fence_before_sync();
   }
   __syncthreads();  // the roles part here and meet again at the end
@@ -478,7 +464,7 @@ __global__ void __maxnreg__(kTeamMaxRegs)
     // Pass A of tile n, then pass C of tile n - 1 (as the forward).
     tmem_fence_after_sync();
     const int w = warp - team * NW;
-    const uint32_t tq = *tslot + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(warp >> 2) * (MS * COLS);
+    const uint32_t tq = *tslot + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(warp >> 2) * (TSLOTS * COLS);
     const float* kept = reinterpret_cast<const float*>(a.ws + p.off_kept);
     unsigned char* wb = tb + (uint32_t)w * (TS * 128u);  // this warp's slices of the rings
     auto load_a = [&](uint32_t n) {  // tile n's dh and rho (gated: dy, rho and z), if there is one
@@ -513,32 +499,12 @@ __global__ void __maxnreg__(kTeamMaxRegs)
       float2 nhp = f2(0.0f);
       if (lane == 0) {
         if (n == 0 && !tm.end) load_c(0);
-        if (tm.end && n >= 2) {  // no pass A left to hide this in
+        if (LAG == 1 && tm.end && n >= 2) {  // no pass A left to hide this in
           bulk_wait_read<0>();
           load_c(n - 1);
         }
       }
       __syncwarp();
-      // gated: the first rows of dy and z that pass C of tile n - 1 reads again
-      [[maybe_unused]] const int64_t pitch = p.D * (int64_t)sizeof(T);
-      [[maybe_unused]] int64_t off0 = 0;
-      GateRows<PR> gr;
-      if constexpr (GATED) {
-        if (n > 0) {
-          const TileMeta& tc = meta[(n - 1) % kTeamMeta];
-          const int d0 = tc.d + lane * VEC;
-          off0 = (((int64_t)tc.b * p.L + tc.t0 + w * TS) * p.D + d0) * (int64_t)sizeof(T);
-          gr.dy_base = static_cast<const unsigned char*>(a.dy);
-          gr.z_base = static_cast<const unsigned char*>(a.z);
-          gr.off = off0;
-          gr.left = d0 < p.D ? min(tc.len - tc.rel0 - w * TS, TS) : 0;
-#pragma unroll
-          for (int r = 0; r < PR; ++r) {
-            gr.dy[r] = gr.z[r] = 0u;
-            gr.load(r, pitch);
-          }
-        }
-      }
       if (!tm.end) {
         // ---- A
         const int rel = tm.rel0 + w * TS;
@@ -562,17 +528,20 @@ __global__ void __maxnreg__(kTeamMaxRegs)
           constexpr bool FAST = decltype(fast_c)::value;
 #pragma unroll 1  // the instruction cache holds both passes
           for (int part = NP - 1; part >= 0; --part) {
-            float park[16];
+            float park[16], merge[8];
             const unsigned char* lp = lb + part * PR * 128;
             if constexpr (F32)
-              team_rfold_f32<FAST, GATED, BOX>(lp, k, valid - part * PR, W.x, M.x, park);
+              team_rfold_f32<FAST, GATED, BOX>(lp, k, valid - part * PR, W.x, M.x, park, merge);
             else
-              team_rfold_bf16<FAST, GATED, BOX>(lp, k, valid - part * PR, W, M, park);
+              team_rfold_bf16<FAST, GATED, BOX>(lp, k, valid - part * PR, W, M, park, merge);
             __syncwarp();
-            tmem_st16(tq + m * COLS + part * 16, park);
-            if (part == NP / 2 && n >= 2 && lane == 0) {  // tile n - 2's outputs have been read by now
+            const uint32_t to = tq + (n % TSLOTS) * COLS;
+            tmem_st16(to + part * 16, park);
+            if constexpr (GATED) tmem_st8(to + team_cols<T>() + part * 8, merge);
+            // the outputs of the last pass C have been read by now: the next one's inputs
+            if (part == NP / 2 && n >= 1 + LAG && lane == 0) {
               bulk_wait_read<0>();
-              load_c(n - 1);
+              load_c(n - LAG);
             }
           }
         };
@@ -592,19 +561,25 @@ __global__ void __maxnreg__(kTeamMaxRegs)
         }
         __syncwarp();
       }
-      if (n > 0) {
-        // ---- C: tile n - 1
-        const uint32_t q = n - 1, mq = q % MS;
+      if (LAG == 0 ? !tm.end : n > 0) {
+        // ---- C: tile n - LAG
+        const uint32_t q = n - LAG, mq = q % MS;
+        if (LAG == 0) hp = nhp;
         const TileMeta tc = meta[q % kTeamMeta];
         const int rel = tc.rel0 + w * TS;
         const int d0 = tc.d + lane * VEC;
         const bool ch_ok = d0 < p.D;
         const int rows = ch_ok ? min(tc.len - rel, TS) : 0;
         const bool fast = polys[q % kTeamMeta] != 0 && __all_sync(kFull, rows == TS);
-        [[maybe_unused]] unsigned char* dz = static_cast<unsigned char*>(a.dz) + off0;
-        uint32_t pr[16];
+        [[maybe_unused]] const int64_t pitch = p.D * (int64_t)sizeof(T);
+        [[maybe_unused]] unsigned char* dz =
+            static_cast<unsigned char*>(a.dz) + ((int64_t)tc.b * p.L + tc.t0 + w * TS) * pitch + d0 * (int64_t)sizeof(T);
+        uint32_t pr[16], merge[8];
+        if constexpr (LAG == 0) tmem_wait_st();
         __syncwarp();  // tcgen05 accesses are warp-collective
-        tmem_ld16_start(tq + mq * COLS, pr);
+        const uint32_t from = tq + (q % TSLOTS) * COLS;
+        tmem_ld16_start(from, pr);
+        if constexpr (GATED) tmem_ld8_start(from + team_cols<T>(), merge);
         mbar_wait(&carry_ready[mq], (q / MS) & 1u, err);
         // the adjoint entering the slice: the tile's, through the slices after it
         float2 win;
@@ -627,15 +602,17 @@ __global__ void __maxnreg__(kTeamMaxRegs)
           for (int part = 0; part < NP; ++part) {
             __syncwarp();
             tmem_ld_wait(pr);
+            if constexpr (GATED) tmem_ld8_ready(merge);
             unsigned char* lp = lb + part * PR * 128;
             const int pv = rows - part * PR;
             if constexpr (F32)
-              team_rows_f32<FAST, GATED, BOX>(lp, pr, win.x, k, pv, hp.x, dlr.x, gr, dz, pitch);
+              team_rows_f32<FAST, GATED, BOX>(lp, pr, win.x, k, pv, hp.x, dlr.x, merge, dz, pitch);
             else
-              team_rows_bf16<FAST, GATED, BOX>(lp, pr, win, k, pv, hp, dlr, gr, dz, pitch);
+              team_rows_bf16<FAST, GATED, BOX>(lp, pr, win, k, pv, hp, dlr, merge, dz, pitch);
             if (part + 1 < NP) {
               __syncwarp();
-              tmem_ld16_start(tq + mq * COLS + (part + 1) * 16, pr);
+              tmem_ld16_start(from + (part + 1) * 16, pr);
+              if constexpr (GATED) tmem_ld8_start(from + team_cols<T>() + (part + 1) * 8, merge);
             }
           }
         };
@@ -665,7 +642,7 @@ __global__ void __maxnreg__(kTeamMaxRegs)
           if constexpr (!F32) ds[VEC - 1] += (double)dlr.y;
         }
       }
-      hp = nhp;
+      if (LAG == 1) hp = nhp;
       if (tm.end) break;
     }
     if (lane == 0) bulk_wait_all();  // every store complete before the block ends
@@ -675,7 +652,7 @@ __global__ void __maxnreg__(kTeamMaxRegs)
   __syncthreads();  // every role is done with the block's TMEM
   if (warp == 0) {
     tmem_fence_after_sync();
-    tmem_dealloc(*tslot, team_tmem_cols<T>());
+    tmem_dealloc(*tslot, TCOLS);
   }
   // The warps' last d Lambda sums: added up per team, one reduction per team
   // and channel.
