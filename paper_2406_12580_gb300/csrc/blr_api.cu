@@ -273,11 +273,11 @@ blr_status allow_smem(K kernel, size_t smem) {
   return BLR_OK;
 }
 
-// float32 rings deep enough run the LATE form (refill after the next stage's
-// arithmetic); bfloat16 always the early one.
+// Rings deep enough run the LATE form (refill after the next stage's
+// arithmetic): float32 ones and the bfloat16 forward without the merge.
 template <typename T>
 bool late_refill(int stages) {
-  return sizeof(T) == 4 && stages >= blr::kSeqLateRefillStages;
+  return stages >= (sizeof(T) == 4 ? blr::kSeqLateRefillStages : blr::kSeqLateRefillStagesBf16);
 }
 
 template <typename T, class M, int VEC, int R, int RB, bool GATED, int MODE = blr::kSeqPlain>
@@ -287,7 +287,7 @@ blr_status launch_seq_fwd(blr::SeqFwdArgs& a, cudaStream_t st) {
   a.stages = seq_stages(blocks, NB * (size_t)blr::seq_box_bytes<T, VEC, R>());
   const size_t smem = blr::seq_smem_bytes<T, VEC, R>(a.stages, NB);
   auto kernel = blr::seq_fwd_kernel<T, M, VEC, R, RB, GATED, MODE, false>;
-  if constexpr (sizeof(T) == 4) {
+  if constexpr (sizeof(T) == 4 || !GATED) {
     if (late_refill<T>(a.stages)) kernel = blr::seq_fwd_kernel<T, M, VEC, R, RB, GATED, MODE, true>;
   }
   BLR_TRY(allow_smem(kernel, smem));

@@ -44,10 +44,10 @@ namespace blr {
 constexpr int kSeqMaxStages = 8;   // ring stages per warp
 // Rings of at least this many stages may refill a consumed stage after the
 // next stage's arithmetic rather than before it (the kernels' LATE form;
-// measured on GB300: float32 rings of 4-8 stages up to 5 % faster that way,
-// bfloat16 rings of 2-3 stages 3-7 % slower, so bfloat16 keeps the early
-// form).
-constexpr int kSeqLateRefillStages = 4;
+// measured on GB300: float32 rings of 4-8 stages up to 5 % faster that way; of
+// the bfloat16 kernels the forward without the merge from 3 stages, 1500 x 800
+// x 64 111 -> 99 us, the others 3-7 % slower).
+constexpr int kSeqLateRefillStages = 4, kSeqLateRefillStagesBf16 = 3;
 
 // Tensor maps: (channels, time, batch) views with boxes of 32 * VEC channels x
 // R steps x 1 row. gate_logits is seen as two views of D channels each
@@ -282,8 +282,13 @@ __global__ void __launch_bounds__(32) seq_fwd_kernel(const __grid_constant__ Seq
   constexpr int NB = GATED ? 4 : 3;  // boxes per stage: x, rho, iota (, z)
   constexpr uint32_t BOX = seq_box_bytes<T, VEC, R>();
   static_assert(R % RB == 0, "kept states must fall on stage rows");
-  // bfloat16 lanes run their arithmetic on packed pairs
-  constexpr bool kPacked = G::kHalfInputs && VEC == 2;
+  // bfloat16 lanes run their arithmetic on packed pairs with the merge, whose
+  // instructions fill the scheduler, and one channel at a time without it: a
+  // paired instruction holds the one pipe that has it for two cycles, and the
+  // few warps of a scheduler wait for it (fwd, us, paired / single: 1000 x 200 x 64
+  // 24.1 / 21.8, 700 x 200 x 64 23.8 / 21.2; with the merge 2048 x 50 x 64
+  // 19.4 / 19.7).
+  constexpr bool kPacked = G::kHalfInputs && VEC == 2 && GATED;
   const Plan& p = a.p;
   extern __shared__ unsigned char seq_smem[];
   SeqRing<NB, BOX> ring{align128(seq_smem), nullptr, a.stages};
@@ -604,7 +609,7 @@ __global__ void __launch_bounds__(32, sizeof(T) == 4 ? 8 : 16) seq_bwd_kernel(co
   constexpr uint32_t BOX = seq_box_bytes<T, VEC, R>();
   constexpr int NSUB = R / RB;
   static_assert(R % RB == 0, "sub-blocks must tile a stage");
-  constexpr bool kPacked = G::kHalfInputs && VEC == 2;  // as seq_fwd_kernel
+  constexpr bool kPacked = G::kHalfInputs && VEC == 2;  // bfloat16 on packed pairs
   const Plan& p = a.p;
   extern __shared__ unsigned char seq_smem[];
   SeqRing<NB, BOX> ring{align128(seq_smem), nullptr, a.stages};
