@@ -430,9 +430,9 @@ blr_status launch_team_fwd(blr::TeamFwdArgs& a, cudaStream_t st) {
   return launch_team(blr::team_fwd_kernel<T, GATED>, blr::TeamFwdSmem<T>::bytes, a, st,
                      "launch team_fwd_kernel");
 }
-template <typename T, bool GATED>
+template <typename T, bool GATED, bool ROUND = false>
 blr_status launch_team_bwd(blr::TeamBwdArgs& a, cudaStream_t st) {
-  return launch_team(blr::team_bwd_kernel<T, GATED>, blr::TeamBwdSmem<T, GATED>::bytes, a, st,
+  return launch_team(blr::team_bwd_kernel<T, GATED, ROUND>, blr::TeamBwdSmem<T, GATED>::bytes, a, st,
                      "launch team_bwd_kernel");
 }
 
@@ -492,7 +492,9 @@ blr_status scan_bwd_team(const Plan& plan, const void* dh, const float* dh_last,
   using bf = __nv_bfloat16;
   if (plan.io == BLR_F32)
     return z != nullptr ? launch_team_bwd<float, true>(a, st) : launch_team_bwd<float, false>(a, st);
-  return z != nullptr ? launch_team_bwd<bf, true>(a, st) : launch_team_bwd<bf, false>(a, st);
+  if (z == nullptr) return launch_team_bwd<bf, false>(a, st);
+  const bool small = plan.n_chain < blr::kManyChains && !plan.segmented;
+  return small ? launch_team_bwd<bf, true, true>(a, st) : launch_team_bwd<bf, true>(a, st);
 }
 
 // The address of the library's scratch on the current device, after checking

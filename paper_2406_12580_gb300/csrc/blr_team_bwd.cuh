@@ -93,15 +93,25 @@ struct TeamBwdSmem {
 // dh = 0). (w, m): the fold of the slice's later rows, zero at the slice's
 // end; on return the map of the rows folded so far. GATED: dh = dy SiLU(z), and
 // merge gets dy SiLU'(z) of every element. bfloat16: 4 rows, two channels a
-// lane, park[4r ..] = (g.x, sm.x, g.y, sm.y).
-template <bool FAST, bool GATED, uint32_t BOX>
+// lane, park[4r ..] = (g.x, sm.x, g.y, sm.y). ROUND: the merge as an operator of
+// its own would hand dh on, with the sigmoid of float32 data and dh rounded to
+// bfloat16: so the float32 gradients (d Lambda, dh0) of small problems, whose
+// merge is defined that way, do not depend on how it is computed (with tanh and
+// an unrounded dh they lie up to 3e-3 elsewhere).
+template <bool FAST, bool GATED, bool ROUND, uint32_t BOX>
 __device__ __forceinline__ void team_rfold_bf16(const unsigned char* lb, float2 kh, int valid,
                                                 float2& w, float2& m, float (&park)[16],
                                                 float (&merge)[8]) {
 #pragma unroll
   for (int r = 3; r >= 0; --r) {
     float2 dh = bf2_unpack(lds_u32(lb + r * 128));
-    if constexpr (GATED) {  // with hz = z/2 and th = tanh(hz), as silu_grad
+    if constexpr (ROUND) {
+      const float2 z = bf2_unpack(lds_u32(lb + 2 * BOX + r * 128)), sg = sigmoid2(z), f = __fmul2_rn(z, sg);
+      const float2 pd = __fmul2_rn(dh, __ffma2_rn(sg, __ffma2_rn(f2(-1.0f), f, z), sg));
+      merge[2 * r] = pd.x;
+      merge[2 * r + 1] = pd.y;
+      dh = bf2_unpack(bf2_pack(__fmul2_rn(dh, f)));
+    } else if constexpr (GATED) {  // with hz = z/2 and th = tanh(hz), as silu_grad
       const float2 hz = bf2_scaled(lds_u32(lb + 2 * BOX + r * 128), kBf2Half), th = tanh2(hz);
       const float2 sg = __ffma2_rn(f2(0.5f), th, f2(0.5f));
       const float2 f = __ffma2_rn(hz, th, hz);
@@ -263,7 +273,8 @@ __device__ __forceinline__ void team_rows_f32(unsigned char* lb, const uint32_t 
   }
 }
 
-template <typename T, bool GATED>
+// ROUND: as team_rfold_bf16 (bfloat16 with the merge only).
+template <typename T, bool GATED, bool ROUND>
 __global__ void __maxnreg__(kTeamMaxRegs)
     team_bwd_kernel(const __grid_constant__ TeamBwdArgs a) {
   using SM = TeamBwdSmem<T, GATED>;
@@ -533,7 +544,7 @@ __global__ void __maxnreg__(kTeamMaxRegs)
             if constexpr (F32)
               team_rfold_f32<FAST, GATED, BOX>(lp, k, valid - part * PR, W.x, M.x, park, merge);
             else
-              team_rfold_bf16<FAST, GATED, BOX>(lp, k, valid - part * PR, W, M, park, merge);
+              team_rfold_bf16<FAST, GATED, ROUND, BOX>(lp, k, valid - part * PR, W, M, park, merge);
             __syncwarp();
             const uint32_t to = tq + (n % TSLOTS) * COLS;
             tmem_st16(to + part * 16, park);

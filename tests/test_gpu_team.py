@@ -98,3 +98,30 @@ def test_scratch_call_takes_the_local_order():
     # the two orders differ in the order of float32 compositions only
     assert normwise(h2.cpu().numpy(), h.cpu().numpy()) <= TOL[I.F32]
     assert normwise(h_last2.cpu().numpy(), h_last.cpu().numpy()) <= TOL[I.F32]
+
+
+@pytest.mark.parametrize("B,L,D", [(1, 20, 8), (12, 300, 72), (127, 150, 128), (250, 40, 16)])
+def test_small_gated_bf16_gradients_are_the_separate_merges(B, L, D):
+    """d Lambda and dh0 of small bfloat16 problems with the merge are those of
+    the plain scan given dh = dy SiLU(z) rounded to bfloat16. Both sides round the
+    same float32 product but for its last bits (2e-6 of 2^-9: one value in a
+    thousand lands on the other side, 2^-9 sqrt(1e-3) = 6e-5 of the sums; without
+    the rounding, or with tanh for the sigmoid, they differ by 1e-3 and more)."""
+    from paper_2406_12580_gb300 import (BLR_BF16, Desc, blr_scan_bwd, blr_scan_bwd_gated,
+                                        blr_scan_fwd, blr_scan_fwd_gated, blr_workspace_bytes)
+    g = torch.Generator(device="cuda").manual_seed(B + L + D)
+    rand = lambda *s: torch.randn(*s, device="cuda", generator=g).bfloat16()  # noqa: E731
+    x, z, dy, gl = rand(B, L, D), rand(B, L, D), rand(B, L, D), rand(B, L, 2 * D)
+    h0 = torch.randn(B, D, device="cuda", generator=g)
+    lam = torch.from_numpy(I.lambda_from_decay(np.linspace(0.9, 0.999, D)).astype(np.float32)).cuda()
+    desc = Desc(B, L, D, BLR_BF16, 1.0)
+    ws = torch.empty(blr_workspace_bytes(desc), dtype=torch.uint8, device="cuda")
+    y, dx, dz, dgl = (torch.empty_like(t) for t in (x, x, z, gl))
+    got, want = ([torch.empty_like(lam), torch.empty_like(h0)] for _ in range(2))
+    blr_scan_fwd_gated(desc, x, gl, lam, h0, z, y, None, ws)
+    blr_scan_bwd_gated(desc, dy, None, x, gl, lam, h0, z, dx, dgl, dz, *got, ws)
+    dh = (dy.float() * torch.nn.functional.silu(z.float())).bfloat16()
+    blr_scan_fwd(desc, x, gl, lam, h0, y, None, ws)
+    blr_scan_bwd(desc, dh, None, x, gl, lam, h0, dx, dgl, *want, ws)
+    for a, b in zip(got, want):
+        assert (a - b).norm().item() <= 2e-4 * b.norm().item()
