@@ -144,12 +144,14 @@ def kernel_sources_sha() -> str:
 def scan_kernels(cfg):
     """(forward kernels, backward kernels, our kernels per forward call, per
     backward call) the library runs on this shape: the serial kernels from 512
-    float32 or 640 bfloat16 chains on, else the team kernels. (In their
+    float32 or 780 bfloat16 chains on (bfloat16 also from 304 where L is at most
+    5/4 of their number), else the team kernels. (In their
     look-back order those also clear their records with one cudaMemsetAsync a
     call, which is not counted as a kernel of ours.)"""
     f32 = cfg.io == "f32"
     width = 32 if f32 else 64
-    if cfg.B * ((cfg.D + width - 1) // width) >= (512 if f32 else 640):
+    chains = cfg.B * ((cfg.D + width - 1) // width)
+    if chains >= (512 if f32 else 780) or (not f32 and chains >= 304 and 4 * cfg.L <= 5 * chains):
         return "seq_fwd_kernel", "seq_bwd_kernel", 1, 1
     return "team_fwd_kernel", "team_bwd_kernel", 1, 1
 

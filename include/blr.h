@@ -115,8 +115,10 @@ BLR_API size_t blr_workspace_bytes(const blr_desc* desc);
  *                         the reverse.
  *   BLR_FAMILY_TILED      otherwise.
  *   BLR_FAMILY_NONE       an invalid or empty problem (nothing is launched).
- * From 512 float32 or 640 bfloat16 chains on the serial kernels run: one warp
- * walks each chain through the whole sequence. Below, the team kernels: teams
+ * From 512 float32 or 780 bfloat16 chains on (bfloat16 also from 304 where L is
+ * at most 5/4 of their number) the serial kernels run: one warp walks each chain
+ * (bfloat16: each half of it, where there are few) through the whole sequence.
+ * Elsewhere the team kernels: teams
  * of 8 warps scan tiles of up to 128 steps of a chain, 16 steps a warp, whole
  * chains at a time where there are enough of them, else tiles of all chains in
  * time order, chained by a decoupled look-back (the operator of Sec. 3.3) after

@@ -274,7 +274,7 @@ blr_status allow_smem(K kernel, size_t smem) {
 }
 
 // Rings deep enough run the LATE form (refill after the next stage's
-// arithmetic): float32 ones and the bfloat16 forward without the merge.
+// arithmetic): float32 and narrow ones and the bfloat16 forward without the merge.
 template <typename T>
 bool late_refill(int stages) {
   return stages >= (sizeof(T) == 4 ? blr::kSeqLateRefillStages : blr::kSeqLateRefillStagesBf16);
@@ -287,7 +287,7 @@ blr_status launch_seq_fwd(blr::SeqFwdArgs& a, cudaStream_t st) {
   a.stages = seq_stages(blocks, NB * (size_t)blr::seq_box_bytes<T, VEC, R>());
   const size_t smem = blr::seq_smem_bytes<T, VEC, R>(a.stages, NB);
   auto kernel = blr::seq_fwd_kernel<T, M, VEC, R, RB, GATED, MODE, false>;
-  if constexpr (sizeof(T) == 4 || !GATED) {
+  if constexpr (sizeof(T) == 4 || !GATED || VEC == 1) {
     if (late_refill<T>(a.stages)) kernel = blr::seq_fwd_kernel<T, M, VEC, R, RB, GATED, MODE, true>;
   }
   BLR_TRY(allow_smem(kernel, smem));
@@ -301,7 +301,7 @@ blr_status launch_seq_bwd(blr::SeqBwdArgs& a, cudaStream_t st) {
   a.stages = seq_stages(blocks, NB * (size_t)blr::seq_box_bytes<T, VEC, R>());
   const size_t smem = blr::seq_smem_bytes<T, VEC, R>(a.stages, NB);
   auto kernel = blr::seq_bwd_kernel<T, M, VEC, R, RB, GATED, MODE, false>;
-  if constexpr (sizeof(T) == 4) {
+  if constexpr (sizeof(T) == 4 || VEC == 1) {
     if (late_refill<T>(a.stages)) kernel = blr::seq_bwd_kernel<T, M, VEC, R, RB, GATED, MODE, true>;
   }
   BLR_TRY(allow_smem(kernel, smem));
@@ -345,6 +345,7 @@ blr_status scan_fwd_seq(const Plan& plan, const void* x, const void* gl, const f
       if (plan.sr == 32) return launch_seq_fwd<float, blr::MathPrecise, 1, 32, 16, true>(a, st);
       return launch_seq_fwd<float, blr::MathPrecise, 1, 16, 16, true>(a, st);
     }
+    if (plan.sv == 1) return launch_seq_fwd<__nv_bfloat16, blr::MathFast, 1, 16, 8, true>(a, st);
     return launch_seq_fwd<__nv_bfloat16, blr::MathFast, 2, 16, 8, true>(a, st);
   }
   if (lengths != nullptr) {
@@ -353,12 +354,14 @@ blr_status scan_fwd_seq(const Plan& plan, const void* x, const void* gl, const f
       if (plan.sr == 32) return launch_seq_fwd<float, blr::MathPrecise, 1, 32, 16, false, V>(a, st);
       return launch_seq_fwd<float, blr::MathPrecise, 1, 16, 16, false, V>(a, st);
     }
+    if (plan.sv == 1) return launch_seq_fwd<__nv_bfloat16, blr::MathFast, 1, 16, 8, false, V>(a, st);
     return launch_seq_fwd<__nv_bfloat16, blr::MathFast, 2, 16, 8, false, V>(a, st);
   }
   if (plan.io == BLR_F32) {
     if (plan.sr == 32) return launch_seq_fwd<float, blr::MathPrecise, 1, 32, 16, false>(a, st);
     return launch_seq_fwd<float, blr::MathPrecise, 1, 16, 16, false>(a, st);
   }
+  if (plan.sv == 1) return launch_seq_fwd<__nv_bfloat16, blr::MathFast, 1, 16, 8, false>(a, st);
   return launch_seq_fwd<__nv_bfloat16, blr::MathFast, 2, 16, 8, false>(a, st);
 }
 
@@ -392,14 +395,17 @@ blr_status scan_bwd_seq(const Plan& plan, const void* dh, const float* dh_last, 
   a.stages = 2;
   if (gated) {
     if (plan.io == BLR_F32) return launch_seq_bwd<float, blr::MathPrecise, 1, 16, 16, true>(a, st);
+    if (plan.sv == 1) return launch_seq_bwd<__nv_bfloat16, blr::MathFast, 1, 16, 8, true>(a, st);
     return launch_seq_bwd<__nv_bfloat16, blr::MathFast, 2, 8, 8, true>(a, st);
   }
   if (lengths != nullptr) {
     constexpr int V = blr::kSeqVarlen;
     if (plan.io == BLR_F32) return launch_seq_bwd<float, blr::MathPrecise, 1, 16, 16, false, V>(a, st);
+    if (plan.sv == 1) return launch_seq_bwd<__nv_bfloat16, blr::MathFast, 1, 16, 8, false, V>(a, st);
     return launch_seq_bwd<__nv_bfloat16, blr::MathFast, 2, 8, 8, false, V>(a, st);
   }
   if (plan.io == BLR_F32) return launch_seq_bwd<float, blr::MathPrecise, 1, 16, 16, false>(a, st);
+  if (plan.sv == 1) return launch_seq_bwd<__nv_bfloat16, blr::MathFast, 1, 16, 8, false>(a, st);
   return launch_seq_bwd<__nv_bfloat16, blr::MathFast, 2, 8, 8, false>(a, st);
 }
 
@@ -608,7 +614,7 @@ int blr_scan_family(const blr_desc* desc, int with_lengths) {
   Plan plan;
   bool empty = false;
   if (check_desc(desc, &plan, &empty) != BLR_OK || empty || desc->L == 0) return BLR_FAMILY_NONE;
-  if (plan.n_chain >= blr::kManyChains) return BLR_FAMILY_SERIAL;
+  if (plan.many) return BLR_FAMILY_SERIAL;
   if (plan.segmented && !with_lengths) return BLR_FAMILY_SEGMENTED;
   return BLR_FAMILY_TILED;
 }

@@ -149,6 +149,23 @@ struct Io<__nv_bfloat16, 2> {  // 4 bytes
   }
 };
 
+template <>
+struct Io<__nv_bfloat16, 1> {  // 2 bytes
+  using T = __nv_bfloat16;
+  using Raw = uint16_t;
+  static constexpr int VEC = 1;
+  static __device__ __forceinline__ void unpack(const Raw& t, float (&v)[1]) {
+    v[0] = __uint_as_float((uint32_t)t << 16);
+  }
+  static __device__ __forceinline__ void unpack_half(const Raw& t, float (&v)[1]) {
+    unpack(t, v);
+    v[0] *= 0.5f;
+  }
+  static __device__ __forceinline__ void store_smem(unsigned char* p, const float (&v)[1]) {
+    *reinterpret_cast<__nv_bfloat16*>(p) = __float2bfloat16_rn(v[0]);
+  }
+};
+
 template <int N>
 __device__ __forceinline__ void load_f32(const float* p, float (&v)[N]) {
 #pragma unroll
@@ -317,9 +334,6 @@ struct GatesFast : MathFast {
   }
   static __device__ __forceinline__ float gated_x_half(float hiota, float hx) {
     return fmaf(hx, tanh_approx(hiota), hx);
-  }
-  static __device__ __forceinline__ float sigmoid_half(float hz) {  // sigmoid(2 hz)
-    return fmaf(0.5f, tanh_approx(hz), 0.5f);
   }
   static __device__ __forceinline__ float decay_log(float rho, float, float kh) {
     return fmaf(kh, tanh_approx(0.5f * rho), kh);

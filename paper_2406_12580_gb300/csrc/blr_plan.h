@@ -1,7 +1,8 @@
 // Plan and workspace layout of the BD-LRU scan kernels (host and device).
 //
 // A chain is a 128-byte row segment, 32 float32 or 64 bfloat16 channels of one
-// batch row, followed through time. Problems with many chains run the serial
+// batch row (in the narrow serial kernels 32 bfloat16 ones), followed through
+// time. Problems with many chains run the serial
 // kernels (blr_seq.cuh): one warp walks one chain through the whole sequence.
 // The others run the team kernels (blr_team.cuh): teams of warps scan tiles of
 // `ts` steps of a chain, whole chains at a time (local order) or tiles of all
@@ -55,15 +56,11 @@ constexpr int64_t kSegLongL = 16384;
 
 constexpr int64_t kSeqTallRowsMinL = 1024;
 
-// Problems with at least this many chains run the serial kernels, one warp a
-// chain; the GPU's 608 schedulers are then close to one warp each or above.
-// Measured on GB300 (fwd + bwd, us, serial / team kernels). float32: 600
-// chains x 800 steps 119 / 124, x 3000 399 / 431, 400 x 3000 320 / 297, 512 x
-// 2048 251 / 274. bfloat16 lanes carry two channels, so a chain takes a warp
-// longer: 700 chains x 800 steps 213 / 178, x 3000 748 / 546, x 200 67 / 66
-// (with the merge 82 / 86); 1500 x 200 88 / 108, x 800 294 / 319.
+// float32 problems with at least this many chains run the serial kernels, one
+// warp a chain; the GPU's 608 schedulers are then close to one warp each or
+// above. Measured on GB300 (fwd + bwd, us, serial / team kernels): 600 chains x
+// 800 steps 119 / 124, x 3000 399 / 431, 400 x 3000 320 / 297, 512 x 2048 251 / 274.
 constexpr int64_t kSeqMinChainsF32 = 512;
-constexpr int64_t kSeqMinChainsBf16 = 640;
 
 // Team kernels: kTeamWarps compute warps a block, in teams of kTeamWidth;
 // a warp takes kTeamSlice steps of a tile. The plan (and with it the workspace)
@@ -72,6 +69,34 @@ constexpr int kTeamWarps = 16;
 constexpr int kTeamWidth = 8;
 constexpr int kTeamSlice = 16;
 constexpr int64_t kPlanTeams = 152 * (kTeamWarps / kTeamWidth);
+
+// bfloat16: a chain of the serial kernels is 64 channels, two a lane, or, in
+// their narrow form, 32, one a lane: twice the warps with about 0.6 of the
+// instructions each. `wide` and `narrow` count a problem's chains either way.
+//
+// Serial from this many wide chains, and from one a team where the sequences
+// are no longer than 5/4 of that number: a serial chain takes its steps one by
+// one however few chains there are, the team kernels' time follows the work
+// (fwd + bwd, us, narrow serial / team kernels: 330 chains x 50 steps 19.4 / 21.6, x
+// 400 72 / 73, x 800 136 / 98; 450 x 50 20.4 / 23.5, x 800 140 / 123; 700 x 200
+// 52 / 65, x 800 170 / 176, x 2000 407 / 374; 780 x 200 53 / 71, x 2000 415 / 417;
+// with the merge 450 x 200 50.0 / 54.3, 700 x 800 204 / 224, x 2000 490 / 464).
+constexpr int64_t kSeqMinChainsBf16 = 780;
+inline bool plan_seq_bf16(int64_t wide, int64_t L) {
+  return wide >= kSeqMinChainsBf16 || (wide >= kPlanTeams && 4 * L <= 5 * wide);
+}
+// Narrow up to three narrow warps a scheduler (608 of them). There the busiest
+// scheduler walks three narrow chains instead of two wide ones; beyond, the wide
+// form has the fewer instructions (fwd + bwd, us, wide / narrow: 650 wide chains x 200
+// steps 57.8 / 52.5, with the merge 74.8 / 61.8; 850 x 200 58.8 / 53.4; 950 x 200
+// 60.1 / 63.1; 1500 x 200 80.0 / 95.6). And wherever a third or more of the wide
+// lanes lie past D (1000 x 200 x 32 62.4 / 43.9, 4000 x 50 x 32 with the merge
+// 76 / 48, 1500 x 100 x 96 81.3 / 70.6, 3000 x 50 x 96 82.2 / 80.7).
+constexpr int64_t kSeqMaxNarrow = 3 * 608;
+inline bool plan_narrow(int64_t wide, int64_t narrow) {
+  return narrow <= kSeqMaxNarrow || 2 * narrow <= 3 * wide;
+}
+
 // The look-back reads this many predecessors a round trip; kFarWindow where the
 // chains are so few (kFarChains) that the tiles scanned at one time are many
 // predecessors deep.
@@ -83,13 +108,13 @@ struct Plan {
   int io;           // 0 = float32, 1 = bfloat16
   float c;
   int seq;          // 1: serial kernels, 0: team kernels
-  int sv;           // channels per lane (row segment of 32 * sv channels)
+  int sv;           // channels per lane (a chain is a row segment of 32 * sv channels)
   int rb;           // steps between the forward's kept states
   int sr, srb;      // serial: rows per TMA box, forward and backward (multiples of rb)
   int ts;           // team: steps per tile (a multiple of kTeamSlice)
   int lookback;     // team: 1 look-back order, 0 local order
   int far_window;   // team: the look-back's window
-  int segmented;    // the shape class BLR_FAMILY_SEGMENTED
+  int many, segmented;  // the shape classes BLR_FAMILY_SERIAL and BLR_FAMILY_SEGMENTED
   int64_t n_chain;  // chains = B * ceil(D / (32 * sv))
   int64_t n_carry;  // kept states per chain = ceil(L / rb) - 1
   int64_t n_tc;     // team: tiles per chain
@@ -144,14 +169,20 @@ inline void make_plan(int64_t B, int64_t L, int64_t D, int io, float c, bool loc
   p->tag = h | 1u;  // never 0, the value of a cleared header
   p->sv = io == 0 ? 1 : 2;
   p->n_chain = B * ((D + 32 * p->sv - 1) / (32 * p->sv));
-  p->seq = p->n_chain >= (io == 0 ? kSeqMinChainsF32 : kSeqMinChainsBf16) ? 1 : 0;
-  p->segmented = p->n_chain < kManyChains && io == 1 && L >= kSegMinL &&
+  p->seq = io == 0 ? p->n_chain >= kSeqMinChainsF32 : plan_seq_bf16(p->n_chain, L);
+  p->many = p->n_chain >= kManyChains;
+  p->segmented = !p->many && io == 1 && L >= kSegMinL &&
                  (B * L * D >= kSegMinElems || L >= kSegLongL);
+  const int64_t narrow = B * ((D + 31) / 32);
+  if (p->seq && io == 1 && plan_narrow(p->n_chain, narrow)) {
+    p->sv = 1;
+    p->n_chain = narrow;
+  }
   // Long float32 sequences stream the serial forward in 32-row boxes (fewer,
   // larger TMA loads per chain); shorter ones in 16-row boxes, which reach the
   // first rows sooner.
   p->sr = (io == 0 && L >= kSeqTallRowsMinL) ? 32 : 16;
-  p->srb = io == 0 ? 16 : 8;
+  p->srb = p->sv == 1 ? 16 : 8;
   p->rb = !p->seq ? kTeamSlice : io == 0 ? 16 : 8;
   p->n_carry = (L + p->rb - 1) / p->rb - 1;
   // Tiles of equal height, as few as cover L.

@@ -2,7 +2,9 @@
 // (batch row, channel group) chains to fill the GPU by itself.
 //
 // One warp (one thread block) owns CHW = 32 * VEC consecutive channels of one
-// batch row, a 128-byte row segment, and walks the whole sequence: each lane
+// batch row (a 128-byte row segment; bfloat16's narrow form, VEC = 1, a 64-byte
+// one, for problems with few chains or few channels: plan_narrow) and walks the
+// whole sequence: each lane
 // runs the recurrence h_t = alpha_t h_{t-1} + beta_t x_t of Sec. 3.2 serially
 // for its VEC channels, one multiply-add per element, with the state in
 // registers. There is no cross-lane or cross-block combine and no second pass.
@@ -46,7 +48,8 @@ constexpr int kSeqMaxStages = 8;   // ring stages per warp
 // next stage's arithmetic rather than before it (the kernels' LATE form;
 // measured on GB300: float32 rings of 4-8 stages up to 5 % faster that way; of
 // the bfloat16 kernels the forward without the merge from 3 stages, 1500 x 800
-// x 64 111 -> 99 us, the others 3-7 % slower).
+// x 64 111 -> 99 us, and the narrow form's, with the merge 650 x 400 x 64 107.3 ->
+// 105.6; the others 3-7 % slower).
 constexpr int kSeqLateRefillStages = 4, kSeqLateRefillStagesBf16 = 3;
 
 // Tensor maps: (channels, time, batch) views with boxes of 32 * VEC channels x
@@ -407,7 +410,7 @@ __global__ void __launch_bounds__(32) seq_fwd_kernel(const __grid_constant__ Seq
 // ----------------------------------------------------------------- backward
 
 // One sub-block of RB steps (rows [0, srows) when not FULL) starting at row
-// `row0` of the stage: forward recompute from the state hc, then the reverse
+// `row0` of the stage, float32: forward recompute from the state hc, then the reverse
 // recurrence carrying w = alpha g. dx, d rho and d iota overwrite dh, rho and
 // iota of the same rows in the stage. GATED: the first box holds dy, the
 // gradient of y = h SiLU(z) (Alg. 1), so dh = dy SiLU(z), and
@@ -432,24 +435,13 @@ __device__ __forceinline__ void seq_bwd_sub(unsigned char* lb, int row0, int sro
   for (int s = 0; s < RB; ++s) {
     if (FULL || s < srows) {
       float xv[V], rv[V], iv[V], ix[V], l[V];
-      if constexpr (G::kHalfInputs) {
-        IO::unpack_half(*reinterpret_cast<const Raw*>(s_x + s * ROWB), xv);
-        IO::unpack_half(*reinterpret_cast<const Raw*>(s_r + s * ROWB), rv);
-        IO::unpack_half(*reinterpret_cast<const Raw*>(s_i + s * ROWB), iv);
+      IO::unpack(*reinterpret_cast<const Raw*>(s_x + s * ROWB), xv);
+      IO::unpack(*reinterpret_cast<const Raw*>(s_r + s * ROWB), rv);
+      IO::unpack(*reinterpret_cast<const Raw*>(s_i + s * ROWB), iv);
 #pragma unroll
-        for (int v = 0; v < V; ++v) {
-          l[v] = G::decay_log_half(rv[v], kh[v]);
-          ix[v] = G::gated_x_half(iv[v], xv[v]);
-        }
-      } else {
-        IO::unpack(*reinterpret_cast<const Raw*>(s_x + s * ROWB), xv);
-        IO::unpack(*reinterpret_cast<const Raw*>(s_r + s * ROWB), rv);
-        IO::unpack(*reinterpret_cast<const Raw*>(s_i + s * ROWB), iv);
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-          l[v] = G::decay_log(rv[v], k[v], kh[v]);
-          ix[v] = G::sigmoid(iv[v]) * xv[v];
-        }
+      for (int v = 0; v < V; ++v) {
+        l[v] = G::decay_log(rv[v], k[v], kh[v]);
+        ix[v] = G::sigmoid(iv[v]) * xv[v];
       }
 #pragma unroll
       for (int v = 0; v < V; ++v) {
@@ -470,35 +462,19 @@ __device__ __forceinline__ void seq_bwd_sub(unsigned char* lb, int row0, int sro
       IO::unpack(*reinterpret_cast<const Raw*>(s_dh + s * ROWB), gv);
       if constexpr (GATED) {
         float zv[V];
-        if constexpr (G::kHalfInputs)
-          IO::unpack_half(*reinterpret_cast<const Raw*>(s_z + s * ROWB), zv);
-        else
-          IO::unpack(*reinterpret_cast<const Raw*>(s_z + s * ROWB), zv);
+        IO::unpack(*reinterpret_cast<const Raw*>(s_z + s * ROWB), zv);
 #pragma unroll
         for (int v = 0; v < V; ++v) G::silu_grad(zv[v], sf[v], sdf[v]);
       }
-      if constexpr (G::kHalfInputs) {  // bfloat16 pairs: re-read, not held from the recompute
-        IO::unpack(lds_again(s_x + s * ROWB), xv);
-        IO::unpack_half(lds_again(s_r + s * ROWB), rv);
-        IO::unpack_half(lds_again(s_i + s * ROWB), iv);
-      } else {
-        IO::unpack(*reinterpret_cast<const Raw*>(s_x + s * ROWB), xv);
-        IO::unpack(*reinterpret_cast<const Raw*>(s_r + s * ROWB), rv);
-        IO::unpack(*reinterpret_cast<const Raw*>(s_i + s * ROWB), iv);
-      }
+      IO::unpack(*reinterpret_cast<const Raw*>(s_x + s * ROWB), xv);
+      IO::unpack(*reinterpret_cast<const Raw*>(s_r + s * ROWB), rv);
+      IO::unpack(*reinterpret_cast<const Raw*>(s_i + s * ROWB), iv);
 #pragma unroll
       for (int v = 0; v < V; ++v) {
         const float e = E[s][v], rs = RS[s][v];
         const float alpha = 1.0f + e;
         const float q = -e * (e + 2.0f);
-        float r, i;
-        if constexpr (G::kHalfInputs) {
-          r = G::sigmoid_half(rv[v]);
-          i = G::sigmoid_half(iv[v]);
-        } else {
-          r = G::sigmoid(rv[v]);
-          i = G::sigmoid(iv[v]);
-        }
+        const float r = G::sigmoid(rv[v]), i = G::sigmoid(iv[v]);
         float dhv = gv[v];
         if constexpr (GATED) dhv *= sf[v];
         const float g = dhv + w[v];
@@ -522,7 +498,8 @@ __device__ __forceinline__ void seq_bwd_sub(unsigned char* lb, int row0, int sro
   }
 }
 
-// seq_bwd_sub for a bfloat16 lane under GatesFast, on packed pairs. The forward recompute keeps, per step, alpha, -sqrt(1 - alpha^2)
+// seq_bwd_sub for a bfloat16 lane of two channels under GatesFast, on packed
+// pairs. The forward recompute keeps, per step, alpha, -sqrt(1 - alpha^2)
 // and c = h_{t-1} - alpha i x / sqrt(1 - alpha^2) (so that d l = alpha g c);
 // the reverse recurrence re-reads the step's inputs for i and r, and uses
 // r (1 - r) = (1 - tanh(rho/2)^2) / 4, so d rho = d l (k/4) (1 - tanh^2).
@@ -598,6 +575,68 @@ __device__ __forceinline__ void seq_bwd_sub_bf16x2(unsigned char* lb, int row0, 
   }
 }
 
+// The same for a lane of one bfloat16 channel: the recompute also keeps the
+// step's inputs and gates (there are registers for them).
+template <bool POLY, bool FULL, int R, int RB, bool GATED>
+__device__ __forceinline__ void seq_bwd_sub_bf16(unsigned char* lb, int row0, int srows, float kh,
+                                                 float kq, float& hc, float& w, float& dlr) {
+  using IO = Io<__nv_bfloat16, 1>;
+  using G = GatesFast;
+  constexpr uint32_t ROWB = 64;
+  constexpr uint32_t BOX = R * ROWB;
+  unsigned char* s_dh = lb + row0 * ROWB;
+  const unsigned char* s_x = s_dh + BOX;
+  unsigned char* s_r = s_dh + 2 * BOX;
+  unsigned char* s_i = s_dh + 3 * BOX;
+  unsigned char* s_z = s_dh + 4 * BOX;
+  auto full = [](const unsigned char* p) {
+    float v[1];
+    IO::unpack(*reinterpret_cast<const uint16_t*>(p), v);
+    return v[0];
+  };
+  auto put = [](unsigned char* p, float v) {
+    const float t[1] = {v};
+    IO::store_smem(p, t);
+  };
+  float AL[RB], NQ[RB], CP[RB], NX[RB], TR[RB], TI[RB], DH[RB];
+#pragma unroll
+  for (int s = 0; s < RB; ++s) {
+    if (FULL || s < srows) {
+      const float nhx = -0.5f * full(s_x + s * ROWB);
+      TR[s] = tanh_approx(0.5f * full(s_r + s * ROWB));
+      TI[s] = tanh_approx(0.5f * full(s_i + s * ROWB));
+      const float e = expm1_neg<G::kDeg, POLY>(fmaf(kh, TR[s], kh));
+      const float m2 = e * (e + 2.0f);  // -(1 - alpha^2)
+      const float rs = rsqrt_approx(fmaxf(-m2, 1e-30f));
+      AL[s] = 1.0f + e;
+      NQ[s] = m2 * rs;                    // -sqrt(1 - alpha^2)
+      NX[s] = fmaf(nhx, TI[s], nhx);      // -i x
+      CP[s] = fmaf(AL[s] * rs, NX[s], hc);
+      hc = fmaf(AL[s], hc, NQ[s] * NX[s]);  // alpha h + sqrt(1 - alpha^2) i x
+      DH[s] = full(s_dh + s * ROWB);
+      if constexpr (GATED) {
+        float f, df;
+        G::silu_grad(0.5f * full(s_z + s * ROWB), f, df);
+        put(s_z + s * ROWB, (DH[s] * hc) * df);  // dz = dy h SiLU'(z)
+        DH[s] *= f;
+      }
+    }
+  }
+#pragma unroll
+  for (int s = RB - 1; s >= 0; --s) {
+    if (FULL || s < srows) {
+      const float g = DH[s] + w;
+      w = AL[s] * g;
+      const float gnq = g * NQ[s];                                      // -g sqrt(1 - alpha^2)
+      const float dl = w * CP[s];
+      put(s_dh + s * ROWB, gnq * fmaf(-0.5f, TI[s], -0.5f));            // g sqrt(1 - alpha^2) i
+      put(s_i + s * ROWB, (gnq * NX[s]) * fmaf(-0.5f, TI[s], 0.5f));    // g u (1 - i)
+      put(s_r + s * ROWB, dl * fmaf(-kq, TR[s] * TR[s], kq));
+      dlr = fmaf(dl, fmaf(0.5f, TR[s], 0.5f), dlr);                     // += d l r
+    }
+  }
+}
+
 // MODE as seq_fwd_kernel's.
 template <typename T, class M, int VEC, int R, int RB, bool GATED, int MODE, bool LATE>
 __global__ void __launch_bounds__(32, sizeof(T) == 4 ? 8 : 16) seq_bwd_kernel(const __grid_constant__ SeqBwdArgs a) {
@@ -609,7 +648,7 @@ __global__ void __launch_bounds__(32, sizeof(T) == 4 ? 8 : 16) seq_bwd_kernel(co
   constexpr uint32_t BOX = seq_box_bytes<T, VEC, R>();
   constexpr int NSUB = R / RB;
   static_assert(R % RB == 0, "sub-blocks must tile a stage");
-  constexpr bool kPacked = G::kHalfInputs && VEC == 2;  // bfloat16 on packed pairs
+  constexpr bool kBf16 = sizeof(T) == 2, kPacked = kBf16 && VEC == 2;  // bfloat16, on packed pairs
   const Plan& p = a.p;
   extern __shared__ unsigned char seq_smem[];
   SeqRing<NB, BOX> ring{align128(seq_smem), nullptr, a.stages};
@@ -742,6 +781,16 @@ __global__ void __launch_bounds__(32, sizeof(T) == 4 ? 8 : 16) seq_bwd_kernel(co
           w[1] = w2.y;
           dlr[0] = dlr2.x;
           dlr[1] = dlr2.y;
+        } else if constexpr (kBf16) {
+          const float kq = 0.25f * k[0];
+          if (srows == RB) {
+            if (poly)
+              seq_bwd_sub_bf16<true, true, R, RB, GATED>(lb, row0, srows, kh[0], kq, hc[0], w[0], dlr[0]);
+            else
+              seq_bwd_sub_bf16<false, true, R, RB, GATED>(lb, row0, srows, kh[0], kq, hc[0], w[0], dlr[0]);
+          } else {
+            seq_bwd_sub_bf16<false, false, R, RB, GATED>(lb, row0, srows, kh[0], kq, hc[0], w[0], dlr[0]);
+          }
         } else if (srows == RB) {
           if (poly)
             seq_bwd_sub<IO, G, true, true, R, RB, GATED>(lb, row0, srows, k, kh, hc, w, dlr);

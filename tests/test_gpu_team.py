@@ -1,4 +1,5 @@
-"""GPU: the team kernels at the edges of their tiles, against the oracle.
+"""GPU: the team kernels and the narrow serial ones at the edges of their tiles,
+against the oracle.
 
 Tiles are up to 128 steps, slices 16 steps a warp; a chain is 32 float32 or 64
 bfloat16 channels of one batch row. The bounds are those of the other parity
@@ -34,6 +35,17 @@ EDGES = [
     dict(B=2, L=300, D=1400, random_h0=True, random_dh_last=True),
     # the general e^l - 1 branch
     dict(B=4, L=200, D=40, decay=(0.05, 0.95), c=3.0, random_h0=True, random_dh_last=True),
+    # bfloat16: the serial kernels' narrow form, by few chains (a step, a kept
+    # state's and a box's steps and one more, several boxes; a channel tail, an odd
+    # number of groups) and by few channels; and the general branch in it
+    dict(B=304, L=1, D=64, random_h0=True, random_dh_last=True),
+    dict(B=305, L=8, D=8, random_dh_last=True),
+    dict(B=304, L=9, D=40, random_h0=True),
+    dict(B=170, L=16, D=120, random_h0=True, random_dh_last=True),
+    dict(B=110, L=17, D=160),
+    dict(B=330, L=100, D=72, random_h0=True, random_dh_last=True, decay=(0.99, 0.9999)),
+    dict(B=2100, L=33, D=24, random_h0=True, random_dh_last=True),
+    dict(B=320, L=50, D=56, decay=(0.05, 0.95), c=3.0, random_h0=True, random_dh_last=True),
 ]
 
 
