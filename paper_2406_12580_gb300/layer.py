@@ -9,8 +9,8 @@
 The scan and the merge, forward and backward, run in the library
 (``BDLRUGatedScan``). So do the convolution with its SiLU (``blr_conv_silu_*``,
 float32 and bfloat16) and the float32 projections (``blr_linear_*``) on a CUDA
-device in plain eager execution; elsewhere (autocast, TF32 allowed, traced or
-transformed by functorch, forward-mode AD, tensor subclasses, other dtypes,
+device in plain eager execution; elsewhere (autocast, TF32 allowed, traced, under
+a dispatch or function mode or transformed by functorch, forward-mode AD, tensor subclasses, other dtypes,
 devices or widths, hooks on the convolution) they are the torch operators. The
 decay parameter Lambda is initialised as in Sec. 3.2: exp(-softplus(Lambda))
 uniform in [0.9, 0.999]. The convolution width is not given in the paper; it
@@ -20,6 +20,7 @@ from __future__ import annotations
 
 import torch
 from torch import nn
+from torch.utils._device import DeviceContext
 
 from . import (Desc, _dtype_code, blr_conv_silu_bwd, blr_conv_silu_fwd, blr_conv_silu_workspace,
                blr_linear_bwd, blr_linear_fwd, blr_linear_workspace, blr_scan_bwd_gated,
@@ -66,15 +67,20 @@ class BDLRUGatedScan(torch.autograd.Function):
 def _plain_cuda(dtype, *tensors) -> bool:
     """Whether the library's kernels may stand in for torch operators on these
     tensors: ordinary CUDA tensors of one dtype on the current device, in eager
-    execution without autocast, functorch transforms or forward-mode AD."""
+    execution without autocast, tracing, functorch transforms, forward-mode AD or
+    a mode that sees operators (the one of torch.set_default_device does not mind)."""
     if (torch.is_autocast_enabled() or torch.compiler.is_compiling()
             or torch._C._are_functorch_transforms_active()
-            or torch.autograd.forward_ad._current_level >= 0):
+            or torch.autograd.forward_ad._current_level >= 0
+            or torch._C._get_tracing_state() is not None
+            or torch._C._len_torch_dispatch_stack() > 0
+            or any(type(torch._C._get_function_stack_at(i)) is not DeviceContext
+                   for i in range(torch._C._len_torch_function_stack()))):
         return False
     for t in tensors:
         if type(t) not in (torch.Tensor, nn.Parameter) or t.dtype != dtype or not t.is_cuda:
             return False
-        if (t.layout != torch.strided or t.numel() == 0 or t.data_ptr() % 16 != 0
+        if (t.layout != torch.strided or t.is_neg() or t.numel() == 0 or t.data_ptr() % 16 != 0
                 or t.get_device() != torch._C._cuda_getDevice()):
             return False
     return True

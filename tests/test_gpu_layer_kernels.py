@@ -94,3 +94,42 @@ def test_layer_keeps_torch_where_it_must():
         g, = torch.autograd.grad(fn(*c)[0].square().sum(), c[0], create_graph=True)
         two.append(torch.autograd.grad(g.square().sum(), c[1])[0])
     assert normwise(two[0].cpu().numpy(), two[1].cpu().numpy()) <= 1e-4
+
+
+def test_modes_and_tracing_see_torch_operators():
+    """A dispatch or function mode and torch.jit.trace get the projections and the
+    convolution as torch operators; a negative view is read as the values it has."""
+    from torch.overrides import TorchFunctionMode
+    from torch.utils._python_dispatch import TorchDispatchMode
+
+    from paper_2406_12580_gb300.layer import GatedRecurrentLayer, _Linear
+    seen = []
+
+    class Dispatch(TorchDispatchMode):
+        def __torch_dispatch__(self, func, types, args=(), kwargs=None):
+            seen.append(str(func))
+            return func(*args, **(kwargs or {}))
+
+    class Function(TorchFunctionMode):
+        def __torch_function__(self, func, types, args=(), kwargs=None):
+            seen.append(getattr(func, "__name__", ""))
+            return func(*args, **(kwargs or {}))
+
+    torch.manual_seed(7)
+    layer = GatedRecurrentLayer(16, device="cuda")
+    h = torch.randn(2, 12, 16, device="cuda")
+    want = layer(h)
+    for mode, ops in ((Dispatch, ("mm", "conv")), (Function, ("linear", "conv1d"))):
+        seen.clear()
+        with mode():
+            got = layer(h)
+        assert all(any(op in s for s in seen) for op in ops), (mode, seen)
+        assert normwise(got.detach().cpu().numpy(), want.detach().cpu().numpy()) <= 1e-5
+    with torch.device("cuda"):
+        assert "LayerF32" in type(layer(h).grad_fn).__name__
+    lin = _Linear(16, 8, device="cuda")
+    graph = str(torch.jit.trace(lin, h).inlined_graph)
+    assert "aten::linear" in graph and "PythonOp" not in graph
+    neg = torch.randn(5, 16, dtype=torch.complex64, device="cuda").conj().imag
+    ref = torch.nn.functional.linear(neg.clone().resolve_neg(), lin.weight, lin.bias)
+    assert neg.is_neg() and normwise(lin(neg).detach().cpu().numpy(), ref.detach().cpu().numpy()) <= 1e-5
