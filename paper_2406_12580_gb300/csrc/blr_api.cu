@@ -321,10 +321,25 @@ blr_status seq_maps_gl(CUtensorMap* mr, CUtensorMap* mi, const void* base, const
                          plan.D, plan.L, plan.B, rows, cols, 2 * plan.D);
 }
 
+// The plan of a serial problem in the narrow form (bfloat16), if that is to run.
+int64_t narrow_chains(const Plan& p) { return p.B * ((p.D + 31) / 32); }
+Plan seq_form(const Plan& wide, bool narrow) {
+  Plan p = wide;
+  if (p.io == BLR_BF16 && narrow) {
+    p.sv = 1;
+    p.srb = 16;
+    p.n_chain = narrow_chains(wide);
+  }
+  return p;
+}
+
 // z given: the merge of the gated layer is fused, and h receives y = h SiLU(z).
-blr_status scan_fwd_seq(const Plan& plan, const void* x, const void* gl, const float* lambda,
+blr_status scan_fwd_seq(const Plan& wide, const void* x, const void* gl, const float* lambda,
                         const float* h0, void* h, float* h_last, unsigned char* w, cudaStream_t st,
                         const void* z, const int32_t* lengths) {
+  const int64_t n = wide.n_chain, nn = narrow_chains(wide);
+  const Plan plan = seq_form(wide, blr::plan_narrow(n, nn) ||
+                                       (z != nullptr && blr::plan_narrow_merge(n, nn, wide.L)));
   blr::SeqFwdArgs a;
   a.lengths = lengths;
   BLR_TRY(seq_maps_x(&a.tm_x, x, plan, plan.sr));
@@ -366,10 +381,11 @@ blr_status scan_fwd_seq(const Plan& plan, const void* x, const void* gl, const f
 }
 
 // z and dz given: dh is dy, the gradient of y = h SiLU(z), and dz is written.
-blr_status scan_bwd_seq(const Plan& plan, const void* dh, const float* dh_last, const void* x,
+blr_status scan_bwd_seq(const Plan& wide, const void* dh, const float* dh_last, const void* x,
                         const void* gl, const float* lambda, const float* h0, void* dx, void* dgl,
                         float* dlambda, float* dh0, unsigned char* w, cudaStream_t st,
                         const void* z, void* dz, const int32_t* lengths) {
+  const Plan plan = seq_form(wide, blr::plan_narrow_bwd(wide.n_chain, narrow_chains(wide), wide.L));
   blr::SeqBwdArgs a;
   a.lengths = lengths;
   BLR_TRY(seq_maps_x(&a.tm_dh, dh, plan, plan.srb));
@@ -614,7 +630,7 @@ int blr_scan_family(const blr_desc* desc, int with_lengths) {
   Plan plan;
   bool empty = false;
   if (check_desc(desc, &plan, &empty) != BLR_OK || empty || desc->L == 0) return BLR_FAMILY_NONE;
-  if (plan.many) return BLR_FAMILY_SERIAL;
+  if (plan.n_chain >= blr::kManyChains) return BLR_FAMILY_SERIAL;
   if (plan.segmented && !with_lengths) return BLR_FAMILY_SEGMENTED;
   return BLR_FAMILY_TILED;
 }

@@ -85,16 +85,31 @@ constexpr int64_t kSeqMinChainsBf16 = 780;
 inline bool plan_seq_bf16(int64_t wide, int64_t L) {
   return wide >= kSeqMinChainsBf16 || (wide >= kPlanTeams && 4 * L <= 5 * wide);
 }
-// Narrow up to three narrow warps a scheduler (608 of them). There the busiest
-// scheduler walks three narrow chains instead of two wide ones; beyond, the wide
-// form has the fewer instructions (fwd + bwd, us, wide / narrow: 650 wide chains x 200
-// steps 57.8 / 52.5, with the merge 74.8 / 61.8; 850 x 200 58.8 / 53.4; 950 x 200
-// 60.1 / 63.1; 1500 x 200 80.0 / 95.6). And wherever a third or more of the wide
+// Forward and backward choose by themselves: the states kept between them lie
+// the same way. Both are narrow up to three narrow warps a scheduler (608 of
+// them), the backward of short sequences up to four. Up to there the busiest
+// scheduler has less to walk; beyond, the wide form has the fewer instructions (fwd + bwd, us, wide / narrow: 650 wide chains x 200 steps 57.8 /
+// 52.5, with the merge 74.8 / 61.8; 850 x 200 58.8 / 53.4; forward alone 950 x 200
+// 20.1 / 21.6, x 800 67.9 / 80.3; backward narrow after a wide forward 950 x 50
+// 26.4 / 24.7, 1216 x 50 28.7 / 26.6, with the merge 33.7 / 30.9, 1000 x 200 with
+// lengths 56.0 / 57.1, 950 x 800 202.6 / 205.3, 1500 x 200 80.0 / 92.7). And wherever a third or more of the wide
 // lanes lie past D (1000 x 200 x 32 62.4 / 43.9, 4000 x 50 x 32 with the merge
 // 76 / 48, 1500 x 100 x 96 81.3 / 70.6, 3000 x 50 x 96 82.2 / 80.7).
-constexpr int64_t kSeqMaxNarrow = 3 * 608;
-inline bool plan_narrow(int64_t wide, int64_t narrow) {
-  return narrow <= kSeqMaxNarrow || 2 * narrow <= 3 * wide;
+constexpr int64_t kSeqMaxNarrow = 3 * 608, kSeqMaxNarrowBwd = 4 * 608, kSeqNarrowBwdL = 128;
+inline bool plan_narrow(int64_t wide, int64_t narrow, int64_t most = kSeqMaxNarrow) {
+  return narrow <= most || 2 * narrow <= 3 * wide;
+}
+inline bool plan_narrow_bwd(int64_t wide, int64_t narrow, int64_t L) {
+  return plan_narrow(wide, narrow, L <= kSeqNarrowBwdL ? kSeqMaxNarrowBwd : kSeqMaxNarrow);
+}
+// With the merge, whose work a lane of one channel spreads over more warps, the
+// forward is narrow again for many short chains, and for longer ones where a
+// sixth or more of the wide lanes lie past D (fwd + bwd, us, wide / narrow forward:
+// 2048 x 50 x 64 47.5 / 45.0, x 100 76.4 / 74.7, 3000 x 50 73.0 / 72.2, 8000 x 50
+// 142.8 / 141.3, 700 x 200 x 160 137.6 / 122.9, 3000 x 50 x 160 144.2 / 140.2; but
+// 3000 x 160 x 64 171 / 177, 1500 x 200 99 / 101, 2100 x 800 x 160 1337 / 1347).
+inline bool plan_narrow_merge(int64_t wide, int64_t narrow, int64_t L) {
+  return wide >= kSeqMaxNarrow && (L <= 100 || (L <= 256 && 3 * narrow <= 5 * wide));
 }
 
 // The look-back reads this many predecessors a round trip; kFarWindow where the
@@ -114,7 +129,7 @@ struct Plan {
   int ts;           // team: steps per tile (a multiple of kTeamSlice)
   int lookback;     // team: 1 look-back order, 0 local order
   int far_window;   // team: the look-back's window
-  int many, segmented;  // the shape classes BLR_FAMILY_SERIAL and BLR_FAMILY_SEGMENTED
+  int segmented;    // the shape class BLR_FAMILY_SEGMENTED
   int64_t n_chain;  // chains = B * ceil(D / (32 * sv))
   int64_t n_carry;  // kept states per chain = ceil(L / rb) - 1
   int64_t n_tc;     // team: tiles per chain
@@ -170,14 +185,8 @@ inline void make_plan(int64_t B, int64_t L, int64_t D, int io, float c, bool loc
   p->sv = io == 0 ? 1 : 2;
   p->n_chain = B * ((D + 32 * p->sv - 1) / (32 * p->sv));
   p->seq = io == 0 ? p->n_chain >= kSeqMinChainsF32 : plan_seq_bf16(p->n_chain, L);
-  p->many = p->n_chain >= kManyChains;
-  p->segmented = !p->many && io == 1 && L >= kSegMinL &&
+  p->segmented = p->n_chain < kManyChains && io == 1 && L >= kSegMinL &&
                  (B * L * D >= kSegMinElems || L >= kSegLongL);
-  const int64_t narrow = B * ((D + 31) / 32);
-  if (p->seq && io == 1 && plan_narrow(p->n_chain, narrow)) {
-    p->sv = 1;
-    p->n_chain = narrow;
-  }
   // Long float32 sequences stream the serial forward in 32-row boxes (fewer,
   // larger TMA loads per chain); shorter ones in 16-row boxes, which reach the
   // first rows sooner.

@@ -46,6 +46,10 @@ EDGES = [
     dict(B=330, L=100, D=72, random_h0=True, random_dh_last=True, decay=(0.99, 0.9999)),
     dict(B=2100, L=33, D=24, random_h0=True, random_dh_last=True),
     dict(B=320, L=50, D=56, decay=(0.05, 0.95), c=3.0, random_h0=True, random_dh_last=True),
+    # only the backward narrow, and with the merge only the forward
+    dict(B=1000, L=41, D=64, random_h0=True, random_dh_last=True),
+    dict(B=1830, L=23, D=64, random_h0=True),
+    dict(B=620, L=170, D=160, random_dh_last=True),
 ]
 
 
