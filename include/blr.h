@@ -96,8 +96,8 @@ typedef struct {
  *   serial: the state every 16 float32 / 8 bfloat16 steps, 0.25-0.5 bytes per
  *           element;
  *   team:   the state every 16 steps, 0.25 bytes per element, and where tiles
- *           are chained by a look-back its records, 12 bytes per channel per
- *           tile of up to 128 steps (0.1 bytes per element);
+ *           are chained by a look-back its records, 24 bytes per channel per
+ *           tile of up to 128 steps (0.2 bytes per element);
  * plus the float64 partial sums of dlambda and a small header (about 64 bytes
  * per channel). It depends only on B, L, D and the I/O dtype.
  */

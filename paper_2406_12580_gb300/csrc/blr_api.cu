@@ -428,9 +428,11 @@ blr_status scan_bwd_seq(const Plan& wide, const void* dh, const float* dh_last, 
 // ------------------------------------------------------------- team kernels
 
 // One block per SM (its shared memory fills one), at most one team per unit of
-// work: a chain in the local order, a tile with the look-back.
+// work: a chain in the local order, a tile with the look-back. fill: empty the
+// forward's records first.
 template <typename K, typename A>
-blr_status launch_team(K kernel, size_t smem, A& args, cudaStream_t st, const char* what) {
+blr_status launch_team(K kernel, size_t smem, A& args, cudaStream_t st, const char* what,
+                       bool fill) {
   constexpr int threads = blr::kTeamThreads;
   const Plan& p = args.p;
   const int64_t units = p.lookback ? p.n_tc * p.n_chain : p.n_chain;
@@ -442,20 +444,21 @@ blr_status launch_team(K kernel, size_t smem, A& args, cudaStream_t st, const ch
   const int64_t n_g = p.n_chain / p.B;
   if (args.teams >= 8 * n_g) args.teams -= args.teams % (unsigned)n_g;
   if (!p.lookback) return launch_overlapped(kernel, grid, dim3((unsigned)threads), smem, st, args, what);
-  BLR_TRY(cuda_check(cudaMemsetAsync(args.ws + p.off_cinc, 0xff, p.off_cend - p.off_cinc, st),
-                     "empty the look-back records"));
+  if (fill)
+    BLR_TRY(cuda_check(cudaMemsetAsync(args.ws + p.off_cinc, 0xff, p.rec_set, st),
+                       "empty the look-back records"));
   return launch_cooperative(kernel, grid, threads, smem, st, args, what);
 }
 
 template <typename T, bool GATED>
 blr_status launch_team_fwd(blr::TeamFwdArgs& a, cudaStream_t st) {
   return launch_team(blr::team_fwd_kernel<T, GATED>, blr::TeamFwdSmem<T>::bytes, a, st,
-                     "launch team_fwd_kernel");
+                     "launch team_fwd_kernel", true);
 }
 template <typename T, bool GATED, bool ROUND = false>
 blr_status launch_team_bwd(blr::TeamBwdArgs& a, cudaStream_t st) {
   return launch_team(blr::team_bwd_kernel<T, GATED, ROUND>, blr::TeamBwdSmem<T, GATED>::bytes, a, st,
-                     "launch team_bwd_kernel");
+                     "launch team_bwd_kernel", false);
 }
 
 // The problem tag a forward leaves in the workspace. The plain and gated scans

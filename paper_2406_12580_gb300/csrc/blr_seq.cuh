@@ -148,6 +148,7 @@ __device__ __forceinline__ void seq_reset_workspace(unsigned char* ws, const Pla
   if (lane == 0) {
     fh->err = 0u;
     bh->exited = 0u;
+    bh->set = 0u;
     fh->tag = tag;
     fh->complete = 1u;
   }
@@ -670,7 +671,8 @@ __global__ void __launch_bounds__(32, sizeof(T) == 4 ? 8 : 16) seq_bwd_kernel(co
   {
     int ok = 0;
     if (lane == 0) {
-      ok = __ldcg(&fh->tag) == p.tag && __ldcg(&fh->complete) == 1u;
+      const uint32_t tag = __ldcg(&fh->tag), complete = __ldcg(&fh->complete);  // one round trip
+      ok = tag == p.tag && complete == 1u;
       if (!ok) atomicOr(&fh->err, kErrWorkspace);
     }
     if (!__shfl_sync(kFull, ok, 0)) return;  // no forward states for this problem: write nothing

@@ -28,8 +28,8 @@
 // Sec. 3.3).
 //
 // Records validate themselves: a record is one relaxed 32- or 64-bit store of
-// a value that is never the all-ones pattern the records are filled with
-// before the call (A - 1 lies in [-1, 0]; a float state is never that NaN).
+// a value that is never the all-ones pattern the records hold
+// before the scan (A - 1 lies in [-1, 0]; a float state is never that NaN).
 //
 // Rows with lengths: a row's tiles count from its first real step, so padding
 // is neither loaded nor stored; time blocks a row does not have are skipped.
@@ -83,7 +83,19 @@ __device__ __forceinline__ float2 map_apply2(float2 m, float2 h, float2 U) {
 __device__ __forceinline__ float m_compose(float m1, float m2) { return fmaf(m1, m2, m1 + m2); }
 
 // ------------------------------------------------------------------ look-back
-//
+
+// Empties a lane's records of one tile in a set no scan uses meanwhile.
+template <int VEC>
+__device__ __forceinline__ void clear_records(unsigned char* set, const Plan& p, int64_t rec) {
+  uint32_t* inc = reinterpret_cast<uint32_t*>(set) + rec;
+  unsigned long long* agg = reinterpret_cast<unsigned long long*>(set + (p.off_cagg - p.off_cinc)) + rec;
+#pragma unroll
+  for (int v = 0; v < VEC; ++v) {
+    inc[v] = kEmpty;
+    agg[v] = ~0ull;
+  }
+}
+
 // One channel's walk over the tile's nprev predecessors, nearest first: the
 // q-th has its records at inc[q * step] and agg[q * step] (step = -BD when
 // the predecessors are the earlier time blocks, as in the forward; +BD when

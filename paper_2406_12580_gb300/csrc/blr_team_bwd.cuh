@@ -338,10 +338,13 @@ __global__ void __maxnreg__(kTeamMaxRegs)
   }
   pdl_wait();
   pdl_release();
+  __shared__ uint32_t s_set;  // the record set to use; changed by the last block out only
   {
     __shared__ int s_ok;
-    if (threadIdx.x == 0) {
-      s_ok = __ldcg(&fh->tag) == a.tag && __ldcg(&fh->complete) == 1u;
+    if (threadIdx.x == 0) {  // one round trip: no load waits for another
+      const uint32_t tag = __ldcg(&fh->tag), complete = __ldcg(&fh->complete), set = __ldcg(&bh->set);
+      s_ok = tag == a.tag && complete == 1u;
+      s_set = set & 1u;
       if (!s_ok) atomicOr(&fh->err, kErrWorkspace);
     }
     __syncthreads();
@@ -369,8 +372,11 @@ __global__ void __maxnreg__(kTeamMaxRegs)
     const uint32_t teams = a.teams;
     const uint32_t n_g = (uint32_t)((p.D + CHW - 1) / CHW);
     TileWalk<true> walk(p, blockIdx.x + team * gridDim.x, teams, n_g);
-    unsigned long long* agg = reinterpret_cast<unsigned long long*>(a.ws + p.off_cagg);
-    uint32_t* inc = reinterpret_cast<uint32_t*>(a.ws + p.off_cinc);
+    const uint32_t set = s_set;
+    unsigned char* recs = a.ws + (set ? p.off_cinc : p.off_cend);
+    unsigned char* spare = a.ws + (set ? p.off_cend : p.off_cinc);  // emptied for the next backward
+    uint32_t* inc = reinterpret_cast<uint32_t*>(recs);
+    unsigned long long* agg = reinterpret_cast<unsigned long long*>(recs + (p.off_cagg - p.off_cinc));
     TileMeta nm;  // the tile to be loaded next, and its decay constants
     float nk[VEC], nkh[VEC];
     bool npoly = true;
@@ -465,6 +471,7 @@ __global__ void __maxnreg__(kTeamMaxRegs)
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(&carry_ready[m]);
+      if (records) clear_records<VEC>(spare, p, rec);
       if (last && a.dh0 != nullptr && ch_ok) {  // the adjoint leaving the row's first step
 #pragma unroll
         for (int v = 0; v < VEC; ++v) a.dh0[ch0 + v] = carry[v];
@@ -701,7 +708,10 @@ __global__ void __maxnreg__(kTeamMaxRegs)
       const double sig = 1.0 / (1.0 + exp(-lam));  // d softplus / d Lambda
       a.dlambda[d] = (float)(-(double)p.c * sig * sum);
     }
-    if (threadIdx.x == 0) bh->exited = 0u;
+    if (threadIdx.x == 0) {
+      bh->exited = 0u;
+      bh->set = s_set ^ 1u;
+    }
   }
 }
 

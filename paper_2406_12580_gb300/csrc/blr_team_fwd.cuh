@@ -295,6 +295,7 @@ __global__ void __maxnreg__(kTeamMaxRegs)
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(&carry_ready[m]);
+      if (records) clear_records<VEC>(a.ws + p.off_cend, p, rec);  // the backward's set
       if (tm.len == 0 && a.h_last != nullptr && ch_ok) {  // an empty row: the state is unchanged
 #pragma unroll
         for (int v = 0; v < VEC; ++v) a.h_last[ch0 + v] = a.h0 != nullptr ? a.h0[ch0 + v] : 0.0f;

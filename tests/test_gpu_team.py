@@ -92,6 +92,39 @@ def test_team_edges(case, mode, io):
         assert normwise(got[k], want) <= TOL[io], k
 
 
+@pytest.mark.parametrize("io", [I.F32, I.BF16])
+@pytest.mark.parametrize("mode", ["plain", "gated", "varlen"])
+def test_backward_again_on_one_workspace(mode, io):
+    """Backwards that follow one forward find their look-back records empty,
+    whatever the workspace held before (zeros would read as published states)."""
+    cfg = I.ScanConfig(f"again {mode}", io=io, seed=77, gated=mode == "gated", B=3, L=1500, D=136,
+                       random_h0=True, random_dh_last=True)
+    inp = I.make_scan_inputs(cfg)
+    from paper_2406_12580_gb300.device import ScanBuffers
+    buf = ScanBuffers.from_inputs(inp)
+    lengths = torch.tensor([cfg.L, 1025, 300], dtype=torch.int32, device="cuda")
+    first, want = None, None if mode == "varlen" else oracle_outputs(inp)
+    for fill in (0, 255, 0):
+        buf.ws.fill_(fill)
+        if mode == "varlen":
+            buf.h.zero_(), buf.dx.zero_(), buf.dgl.zero_()
+            buf.fwd_varlen(lengths)
+        else:
+            (buf.fwd_gated if mode == "gated" else buf.fwd)()
+        for _ in range(4):
+            if mode == "varlen":
+                buf.bwd_varlen(lengths)
+            else:
+                (buf.bwd_gated if mode == "gated" else buf.bwd)()
+            torch.cuda.synchronize()
+            got = gpu_outputs(buf)
+            if mode != "varlen":
+                for k, v in want.items():
+                    assert normwise(got[k], v) <= TOL[io], k
+            first = first or got
+            for k, v in got.items():
+                assert v is None or normwise(v, first[k]) <= TOL[io], k
+
 def test_scratch_call_takes_the_local_order():
     """A problem whose look-back records do not fit the library's scratch still
     runs there: the forward without a workspace takes the local order."""
