@@ -159,15 +159,16 @@ inline uint32_t fnv1a(uint32_t h, uint64_t v) {
 
 // Whether the team kernels take the look-back order: when the tiles of the
 // busiest team, spread over all teams, plus the look-back's own cost (about
-// 5 % a tile, and its records and cooperative launch, worth about 3
-// tiles) still come to less than whole chains a team. Measured on GB300 (fwd +
-// bwd, us, look-back / local): bfloat16 200 chains x 130 steps 38 / 33, 300 x
-// 800 94 / 84, 700 x 800 178 / 182, 700 x 3000 547 / 588, 48 x 1031 42 / 95;
+// 5 % a tile, and its records and cooperative launch, worth about 2 tiles) still
+// come to less than whole chains a team. Measured on GB300 (fwd + bwd, us,
+// look-back / local): bfloat16 20 chains x 300 steps 31.2 / 37.8 (the forward alone 13.5 /
+// 12.6), 30 x 500 31.7 / 47.2, with the merge 33.4 / 55.9, 100 x 600 39.3 / 55.3, 150 x
+// 800 57.0 / 75.1, 200 x 130 38 / 33, 300 x 800 94 / 84, 700 x 3000 547 / 588;
 // float32 400 x 3000 297 / 326.
 inline bool plan_lookback(int64_t chains, int64_t tiles) {
   const int64_t local = (chains + kPlanTeams - 1) / kPlanTeams * tiles;
   const int64_t spread = (chains * tiles + kPlanTeams - 1) / kPlanTeams;
-  return tiles > 1 && 20 * local > 21 * spread + 60;
+  return tiles > 1 && 20 * local > 21 * spread + 38;
 }
 
 // Fills `p` for a validated problem (B, L, D >= 1, D % 8 == 0). local_only
