@@ -275,8 +275,11 @@ class GatedRecurrentLayer(nn.Module):
         self.lam = nn.Parameter(lambda_init(ed).to(device=device))
 
     def _conv_ok(self) -> bool:
-        return (_bare(self.conv, nn.Conv1d) and self.conv.weight.shape == (self.ed, 1, 4)
-                and self.ed <= 1024)
+        """Whether the convolution is the kernels': depthwise, 4 taps, causal by zeros."""
+        c = self.conv
+        return (_bare(c, nn.Conv1d) and c.weight.shape == (self.ed, 1, 4) and c.groups == self.ed
+                and c.stride == (1,) and c.dilation == (1,) and c.padding == (3,)
+                and c.padding_mode == "zeros" and self.ed <= 1024)
 
     def _conv_silu(self, hxz):
         """The scan's inputs from the expansion's output: SiLU(conv(H_x)) and H_z."""
