@@ -86,6 +86,18 @@ def _plain_cuda(dtype, *tensors) -> bool:
     return True
 
 
+def _tf32() -> bool:
+    """Whether torch may run float32 products in TF32, by either of its settings
+    (reading the older one raises once the newer one says something else)."""
+    mm = torch.backends.cuda.matmul
+    try:
+        if hasattr(mm, "fp32_precision"):
+            return mm.fp32_precision not in ("none", "ieee")
+        return mm.allow_tf32
+    except RuntimeError:
+        return True
+
+
 def _differentiable(fn, inputs, grads):
     """Gradients of torch operators, themselves differentiable (create_graph)."""
     with torch.enable_grad():
@@ -143,8 +155,7 @@ class _Linear(nn.Linear):
         if (self.bias is not None and self.weight.dtype == torch.float32
                 and self.in_features % 4 == 0 and self.out_features % 4 == 0
                 and x.dim() > 1 and x.shape[-1] == self.in_features
-                and not torch.backends.cuda.matmul.allow_tf32
-                and _plain_cuda(torch.float32, x, self.weight, self.bias)):
+                and _plain_cuda(torch.float32, x, self.weight, self.bias) and not _tf32()):
             return _LinearF32.apply(x, self.weight, self.bias)
         return super().forward(x)
 
@@ -296,13 +307,13 @@ class GatedRecurrentLayer(nn.Module):
         i, g, o = self.in_proj, self.gate_proj, self.out_proj
         if not (self._conv_ok() and _bare(i, _Linear) and _bare(g, _Linear) and _bare(o, _Linear)):
             return None
-        if (torch.backends.cuda.matmul.allow_tf32 or h.dim() != 3 or h.shape[-1] % 4 != 0
-                or h.shape[-1] != i.in_features or o.out_features % 4 != 0
+        if (h.dim() != 3 or h.shape[-1] % 4 != 0 or h.shape[-1] != i.in_features or o.out_features % 4 != 0
                 or any(getattr(nn.modules.module, n) for n in _GLOBAL_HOOKS)):
             return None
         p = (i.weight, i.bias, self.conv.weight, self.conv.bias, g.weight, g.bias, self.lam,
              o.weight, o.bias)
-        if not _plain_cuda(torch.float32, h, *p) or not all(t.is_contiguous() for t in p):
+        if (not _plain_cuda(torch.float32, h, *p) or not all(t.is_contiguous() for t in p)
+                or _tf32()):
             return None
         return p
 
