@@ -99,13 +99,17 @@ def _tf32() -> bool:
 
 
 def _differentiable(fn, inputs, grads):
-    """Gradients of torch operators, themselves differentiable (create_graph)."""
+    """Gradients of torch operators, differentiable in turn under create_graph.
+    They are taken at aliases of the inputs: an input may itself depend on another
+    (a layer applied twice), and what reaches it that way is not this call's."""
+    graph = torch.is_grad_enabled()
     with torch.enable_grad():
-        outs = fn(*inputs)
+        at = [t.view_as(t) if graph else t.detach().requires_grad_(t.requires_grad) for t in inputs]
+        outs = fn(*at)
         outs = outs if isinstance(outs, tuple) else (outs,)
-        need = [t for t in inputs if t.requires_grad]
-        got = iter(torch.autograd.grad(outs, need, grads, create_graph=True))
-    return tuple(next(got) if t.requires_grad else None for t in inputs)
+        need = [t for t in at if t.requires_grad]
+        got = iter(torch.autograd.grad(outs, need, grads, create_graph=graph))
+    return tuple(next(got) if t.requires_grad else None for t in at)
 
 
 def _linear_fwd(x, weight, bias):
@@ -133,15 +137,15 @@ class _LinearF32(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, x, weight, bias):
-        x, weight, bias = x.contiguous(), weight.contiguous(), bias.contiguous()
-        ctx.save_for_backward(x, weight, bias)
-        return _linear_fwd(x, weight, bias)
+        ctx.save_for_backward(x, weight, bias)  # as they came: create_graph needs their history
+        return _linear_fwd(x.contiguous(), weight.contiguous(), bias.contiguous())
 
     @staticmethod
     def backward(ctx, dy):
         x, weight, bias = ctx.saved_tensors
         if torch.is_grad_enabled() or not _plain_cuda(torch.float32, dy, x, weight):
             return _differentiable(nn.functional.linear, (x, weight, bias), (dy,))
+        x, weight = x.contiguous(), weight.contiguous()
         dx = torch.empty_like(x) if ctx.needs_input_grad[0] else None
         dw, db = _linear_bwd(dy.contiguous(), x, weight, dx, any(ctx.needs_input_grad[1:]))
         return dx, dw if ctx.needs_input_grad[1] else None, db if ctx.needs_input_grad[2] else None
@@ -188,15 +192,15 @@ class _ConvSiLU(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, hxz, weight, bias):
-        hxz, weight, bias = hxz.contiguous(), weight.contiguous(), bias.contiguous()
         ctx.save_for_backward(hxz, weight, bias)
-        return _conv_fwd(hxz, weight, bias)
+        return _conv_fwd(hxz.contiguous(), weight.contiguous(), bias.contiguous())
 
     @staticmethod
     def backward(ctx, dx, dz):
         hxz, weight, bias = ctx.saved_tensors
         if torch.is_grad_enabled() or not _plain_cuda(hxz.dtype, dx, dz, hxz):
             return _differentiable(_conv_silu_torch, (hxz, weight, bias), (dx, dz))
+        hxz, weight, bias = hxz.contiguous(), weight.contiguous(), bias.contiguous()
         grads = _conv_bwd(dx.contiguous(), dz.contiguous(), hxz, weight, bias)
         return tuple(g if n else None for g, n in zip(grads, ctx.needs_input_grad))
 

@@ -52,3 +52,50 @@ assert isinstance(lin(x), str) != {tf32}
 assert (layer._whole(h) is None) == {tf32}
 """
     subprocess.run([sys.executable, "-W", "ignore", "-c", code], check=True, cwd=ROOT)
+
+
+@pytest.fixture
+def kernels_on_cpu(monkeypatch):
+    """Stands torch operators in for the library's calls, out of autograd's sight as those are."""
+    def linear_fwd(T, N, K, x, w, b, y):
+        assert x.is_contiguous() and w.is_contiguous()
+        y.copy_(nn.functional.linear(x, w, b))
+
+    def conv_fwd(B, L, C, io, hxz, w, b, x, z):
+        assert hxz.is_contiguous()
+        for to, of in zip((x, z), layer_module._conv_silu_torch(hxz, w, b)):
+            to.copy_(of)
+
+    monkeypatch.setattr(layer_module, "_dtype_code", lambda t: 0)
+    monkeypatch.setattr(layer_module, "blr_linear_fwd", linear_fwd)
+    monkeypatch.setattr(layer_module, "blr_conv_silu_fwd", conv_fwd)
+
+
+def _grads(out, inputs, create_graph):
+    """First gradients of a scalar and, with create_graph, those of their squares."""
+    first = torch.autograd.grad(out, inputs, create_graph=create_graph)
+    if not create_graph:
+        return first
+    return first + torch.autograd.grad(sum(g.square().sum() for g in first), inputs)
+
+
+@pytest.mark.parametrize("graph", [True, False])
+def test_gradients_by_torch_operators_are_this_calls_own(kernels_on_cpu, graph):
+    """Where a backward uses torch operators (create_graph; gradients the kernels
+    do not take), its gradients are those of its own call: of a projection or a
+    convolution applied twice, whose second input depends on the same weights, and
+    of inputs that are views of other strides."""
+    torch.manual_seed(5)
+    rand = lambda *s: torch.randn(*s, dtype=torch.float64, requires_grad=True)  # noqa: E731
+    w, b, x = rand(6, 6), rand(6), rand(6, 5)
+    k, c, h = rand(4, 1, 4), rand(4), rand(8, 7, 2)
+    lin, conv = layer_module._LinearF32.apply, layer_module._ConvSiLU.apply
+    for lin_, conv_ in ((lin, conv), (nn.functional.linear, layer_module._conv_silu_torch)):
+        y = lin_(lin_(x.t(), w.t(), b), w.t(), b)
+        once = torch.cat(conv_(h.transpose(0, 2), k, c), dim=-1)
+        z, _ = conv_(once, k, c)
+        got = _grads(y.square().sum(), (x, w, b), graph) + _grads(z.square().sum(), (h, k, c), graph)
+        if lin_ is lin:
+            kernel = got
+    for a, r in zip(kernel, got):  # the same operators in the same precision: float64's rounding
+        assert (a - r).abs().max() <= 1e-12 * r.abs().max() and a.requires_grad == r.requires_grad
