@@ -261,6 +261,8 @@ _GLOBAL_HOOKS = ("_global_forward_hooks", "_global_forward_pre_hooks", "_global_
 
 def _bare(module, kind) -> bool:
     """Whether calling the module is its forward and nothing else."""
+    if any(getattr(nn.modules.module, n) for n in _GLOBAL_HOOKS):
+        return False
     return (type(module) is kind and module.bias is not None and not module._forward_hooks
             and not module._forward_pre_hooks and not module._backward_hooks
             and not module._backward_pre_hooks and "forward" not in module.__dict__)
@@ -311,8 +313,8 @@ class GatedRecurrentLayer(nn.Module):
         i, g, o = self.in_proj, self.gate_proj, self.out_proj
         if not (self._conv_ok() and _bare(i, _Linear) and _bare(g, _Linear) and _bare(o, _Linear)):
             return None
-        if (h.dim() != 3 or h.shape[-1] % 4 != 0 or h.shape[-1] != i.in_features or o.out_features % 4 != 0
-                or any(getattr(nn.modules.module, n) for n in _GLOBAL_HOOKS)):
+        if (h.dim() != 3 or h.shape[-1] % 4 != 0 or h.shape[-1] != i.in_features
+                or o.out_features % 4 != 0):
             return None
         p = (i.weight, i.bias, self.conv.weight, self.conv.bias, g.weight, g.bias, self.lam,
              o.weight, o.bias)

@@ -22,6 +22,17 @@ def test_the_convolutions_settings_are_honoured():
         assert not layer._conv_ok(), kw
 
 
+def test_a_hook_on_every_module_sees_the_convolution():
+    layer, seen = layer_module.GatedRecurrentLayer(8), []
+    hook = nn.modules.module.register_module_forward_hook(lambda m, i, o: seen.append(type(m)))
+    try:
+        assert not layer._conv_ok()
+        layer._conv_silu(torch.randn(2, 5, 32))
+    finally:
+        hook.remove()
+    assert seen == [nn.Conv1d] and layer._conv_ok()
+
+
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
