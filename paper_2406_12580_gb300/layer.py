@@ -151,14 +151,18 @@ class _LinearF32(torch.autograd.Function):
         return dx, dw if ctx.needs_input_grad[1] else None, db if ctx.needs_input_grad[2] else None
 
 
+def _linear_ok(n: int, k: int) -> bool:
+    """Whether the kernels take a projection of n outputs and k inputs."""
+    return n % 4 == 0 and k % 4 == 0 and n <= 65536 and k <= 65536
+
+
 class _Linear(nn.Linear):
     """nn.Linear whose float32 product runs in the library (in float32: where
     TF32 is allowed it stays with torch)."""
 
     def forward(self, x):
         if (self.bias is not None and self.weight.dtype == torch.float32
-                and self.in_features % 4 == 0 and self.out_features % 4 == 0
-                and x.dim() > 1 and x.shape[-1] == self.in_features
+                and _linear_ok(*self.weight.shape) and x.dim() > 1 and x.shape[-1] == self.in_features
                 and _plain_cuda(torch.float32, x, self.weight, self.bias) and not _tf32()):
             return _LinearF32.apply(x, self.weight, self.bias)
         return super().forward(x)
@@ -313,8 +317,8 @@ class GatedRecurrentLayer(nn.Module):
         i, g, o = self.in_proj, self.gate_proj, self.out_proj
         if not (self._conv_ok() and _bare(i, _Linear) and _bare(g, _Linear) and _bare(o, _Linear)):
             return None
-        if (h.dim() != 3 or h.shape[-1] % 4 != 0 or h.shape[-1] != i.in_features
-                or o.out_features % 4 != 0):
+        if (h.dim() != 3 or h.shape[-1] != i.in_features or not _linear_ok(self.ed, i.in_features)
+                or not _linear_ok(o.out_features, self.ed)):
             return None
         p = (i.weight, i.bias, self.conv.weight, self.conv.bias, g.weight, g.bias, self.lam,
              o.weight, o.bias)

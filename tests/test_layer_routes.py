@@ -110,3 +110,11 @@ def test_gradients_by_torch_operators_are_this_calls_own(kernels_on_cpu, graph):
             kernel = got
     for a, r in zip(kernel, got):  # the same operators in the same precision: float64's rounding
         assert (a - r).abs().max() <= 1e-12 * r.abs().max() and a.requires_grad == r.requires_grad
+
+
+@pytest.mark.parametrize("n,k,kernel", [(65536, 4, True), (65540, 4, False), (4, 65540, False),
+                                        (6, 4, False), (4, 6, False)])
+def test_projections_the_kernels_refuse_stay_with_torch(monkeypatch, n, k, kernel):
+    monkeypatch.setattr(layer_module, "_plain_cuda", lambda *a: True)
+    monkeypatch.setattr(layer_module._LinearF32, "apply", staticmethod(lambda x, w, b: "kernel"))
+    assert isinstance(layer_module._Linear(k, n)(torch.randn(2, k)), str) == kernel
