@@ -36,6 +36,10 @@ class BDLRUGatedScan(torch.autograd.Function):
     @staticmethod
     def forward(ctx, x, gate_logits, lam, z, h0=None, c: float = 1.0):
         B, L, D = x.shape
+        for name, t, n in (("gate_logits", gate_logits, 2 * B * L * D), ("lam", lam, D),
+                           ("z", z, B * L * D), ("h0", h0, B * D)):
+            if t is not None and t.numel() < n:
+                raise ValueError(f"{name}: fewer values ({t.numel()}) than the scan reads ({n})")
         x, gate_logits, z = x.contiguous(), gate_logits.contiguous(), z.contiguous()
         ctx.lam_dtype = lam.dtype
         lam = lam.contiguous().float()
@@ -161,10 +165,11 @@ class _Linear(nn.Linear):
     TF32 is allowed it stays with torch)."""
 
     def forward(self, x):
-        if (self.bias is not None and self.weight.dtype == torch.float32
-                and _linear_ok(*self.weight.shape) and x.dim() > 1 and x.shape[-1] == self.in_features
-                and _plain_cuda(torch.float32, x, self.weight, self.bias) and not _tf32()):
-            return _LinearF32.apply(x, self.weight, self.bias)
+        w, b = self.weight, self.bias
+        if (b is not None and w.dtype == torch.float32 and w.dim() == 2 and _linear_ok(*w.shape)
+                and b.shape == w.shape[:1] and x.dim() > 1 and x.shape[-1] == w.shape[1]
+                and _plain_cuda(torch.float32, x, w, b) and not _tf32()):
+            return _LinearF32.apply(x, w, b)
         return super().forward(x)
 
 
@@ -298,14 +303,14 @@ class GatedRecurrentLayer(nn.Module):
     def _conv_ok(self) -> bool:
         """Whether the convolution is the kernels': depthwise, 4 taps, causal by zeros."""
         c = self.conv
-        return (_bare(c, nn.Conv1d) and c.weight.shape == (self.ed, 1, 4) and c.groups == self.ed
-                and c.stride == (1,) and c.dilation == (1,) and c.padding == (3,)
+        return (_bare(c, nn.Conv1d) and c.weight.shape == (self.ed, 1, 4)
+                and c.bias.shape == (self.ed,) and c.groups == self.ed and c.stride == (1,) and c.dilation == (1,) and c.padding == (3,)
                 and c.padding_mode == "zeros" and self.ed <= 1024)
 
     def _conv_silu(self, hxz):
         """The scan's inputs from the expansion's output: SiLU(conv(H_x)) and H_z."""
         conv = self.conv
-        if (self._conv_ok() and hxz.dtype in (torch.float32, torch.bfloat16)
+        if (self._conv_ok() and hxz.dim() == 3 and hxz.shape[-1] == 2 * self.ed and hxz.dtype in (torch.float32, torch.bfloat16)
                 and _plain_cuda(hxz.dtype, hxz, conv.weight, conv.bias)):
             return _ConvSiLU.apply(hxz, conv.weight, conv.bias)
         hx, hz = hxz.split(self.ed, dim=-1)
@@ -317,11 +322,15 @@ class GatedRecurrentLayer(nn.Module):
         i, g, o = self.in_proj, self.gate_proj, self.out_proj
         if not (self._conv_ok() and _bare(i, _Linear) and _bare(g, _Linear) and _bare(o, _Linear)):
             return None
-        if (h.dim() != 3 or h.shape[-1] != i.in_features or not _linear_ok(self.ed, i.in_features)
-                or not _linear_ok(o.out_features, self.ed)):
+        ed, d, n = self.ed, h.shape[-1], o.bias.shape[0]
+        if h.dim() != 3 or not _linear_ok(ed, d) or not _linear_ok(n, ed):
             return None
         p = (i.weight, i.bias, self.conv.weight, self.conv.bias, g.weight, g.bias, self.lam,
              o.weight, o.bias)
+        # the kernels take the sizes as given: parameters of others go to the operators, which refuse them
+        if [t.shape for t in p] != [(2 * ed, d), (2 * ed,), (ed, 1, 4), (ed,), (2 * ed, ed), (2 * ed,),
+                                    (ed,), (n, ed), (n,)]:
+            return None
         if (not _plain_cuda(torch.float32, h, *p) or not all(t.is_contiguous() for t in p)
                 or _tf32()):
             return None

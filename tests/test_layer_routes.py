@@ -118,3 +118,36 @@ def test_projections_the_kernels_refuse_stay_with_torch(monkeypatch, n, k, kerne
     monkeypatch.setattr(layer_module, "_plain_cuda", lambda *a: True)
     monkeypatch.setattr(layer_module._LinearF32, "apply", staticmethod(lambda x, w, b: "kernel"))
     assert isinstance(layer_module._Linear(k, n)(torch.randn(2, k)), str) == kernel
+
+
+@pytest.mark.parametrize("name,shape", [
+    ("in_proj.weight", (40, 8)), ("in_proj.bias", (16,)), ("conv.bias", (8,)),
+    ("gate_proj.weight", (32, 8)), ("gate_proj.bias", (16,)), ("lam", (8,)),
+    ("out_proj.weight", (8, 32)), ("out_proj.bias", (4,)), ("in_proj.weight", (48, 8))])
+def test_parameters_of_other_sizes_never_reach_the_kernels(monkeypatch, name, shape):
+    """The kernels read as many values as the sizes say: a parameter of another size
+    goes to the operators one by one, which refuse it."""
+    layer, h = layer_module.GatedRecurrentLayer(8), torch.randn(2, 5, 8)
+    monkeypatch.setattr(layer_module, "_plain_cuda", lambda *a: True)
+    assert layer._whole(h) is not None
+    module, _, attr = name.rpartition(".")
+    setattr(layer.get_submodule(module), attr, nn.Parameter(torch.randn(shape)))
+    assert layer._whole(h) is None
+    refuse = lambda *a: pytest.fail("a kernel was called")  # noqa: E731
+    if module == "conv":
+        monkeypatch.setattr(layer_module._ConvSiLU, "apply", staticmethod(refuse))
+        with pytest.raises(RuntimeError):
+            layer._conv_silu(torch.randn(2, 5, 32))
+    elif name == "in_proj.weight":
+        monkeypatch.setattr(layer_module._ConvSiLU, "apply", staticmethod(refuse))
+        with pytest.raises((RuntimeError, ValueError)):
+            layer._conv_silu(torch.randn(2, 5, shape[0]))
+    elif name == "lam":
+        x = torch.randn(2, 5, 16)
+        with pytest.raises(ValueError, match="lam: fewer values"):
+            layer_module.BDLRUGatedScan.apply(x, torch.randn(2, 5, 32), layer.lam, x)
+    else:
+        monkeypatch.setattr(layer_module._LinearF32, "apply", staticmethod(refuse))
+        lin = getattr(layer, module)
+        with pytest.raises(RuntimeError):
+            lin(torch.randn(3, 16 if module != "in_proj" else 8))
