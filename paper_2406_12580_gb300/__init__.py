@@ -83,7 +83,11 @@ def _ptr(t, name: str):
     """Device pointer of a CUDA tensor on the current device (or a raw int / None)."""
     if t is None:
         return None
-    torch = _torch or _import_torch()
+    torch = _torch
+    if torch is None:
+        if isinstance(t, int):  # raw addresses need no torch
+            return t
+        torch = _import_torch()
     if not isinstance(t, torch.Tensor):
         if isinstance(t, int):
             return t
