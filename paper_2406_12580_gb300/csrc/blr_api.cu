@@ -920,18 +920,20 @@ blr_status blr_linear_bwd(int64_t T, int64_t N, int64_t K, const float* dy, cons
   bool empty = false;
   BLR_TRY(check_linear(T, N, K, &empty));
   if (empty) return BLR_OK;
-  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   BLR_TRY(need(dy, "dy", 16));
-  if (dx != nullptr) {
-    BLR_TRY(need(weight, "weight", 16));
-    BLR_TRY(need(dx, "dx", 16));
-    BLR_TRY(launch_gemm<blr::kNN>(blr::GemmArgs{T, K, N, 0, dy, weight, nullptr, dx, add_dx}, 1, st));
+  BLR_TRY(optional(dx, "dx", 16));
+  if (dx != nullptr) BLR_TRY(need(weight, "weight", 16));
+  if (dweight != nullptr) {
+    BLR_TRY(need(dweight, "dweight", 4));
+    BLR_TRY(need(x, "x", 16));
+    BLR_TRY(need(dbias, "dbias", 4));
+    BLR_TRY(need(ws, "ws", 16));
+    if (ws_bytes < blr_linear_workspace(T, N, K)) return fail(BLR_ERR_INVALID_ARG, "workspace too small");
   }
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  if (dx != nullptr)
+    BLR_TRY(launch_gemm<blr::kNN>(blr::GemmArgs{T, K, N, 0, dy, weight, nullptr, dx, add_dx}, 1, st));
   if (dweight == nullptr) return BLR_OK;
-  BLR_TRY(need(x, "x", 16));
-  BLR_TRY(need(dbias, "dbias", 4));
-  BLR_TRY(need(ws, "ws", 16));
-  if (ws_bytes < blr_linear_workspace(T, N, K)) return fail(BLR_ERR_INVALID_ARG, "workspace too small");
   int64_t splits = wgrad_splits(T, N, K);
   const int64_t rows = ((T + splits - 1) / splits + blr::kGemmK - 1) / blr::kGemmK * blr::kGemmK;
   splits = (T + rows - 1) / rows;
