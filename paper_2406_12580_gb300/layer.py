@@ -33,16 +33,19 @@ class BDLRUGatedScan(torch.autograd.Function):
     float32 or bfloat16; lam (D,) and h0 (B, D) or None in float32. Returns
     (y, h_last)."""
 
+    @classmethod
+    def apply(cls, x, gate_logits, lam, z, h0=None, c: float = 1.0):
+        # laid out for the kernels in autograd's sight: create_graph needs the inputs' history
+        return super().apply(x.contiguous(), gate_logits.contiguous(), lam.contiguous().float(),
+                             z.contiguous(), h0, c)
+
     @staticmethod
-    def forward(ctx, x, gate_logits, lam, z, h0=None, c: float = 1.0):
+    def forward(ctx, x, gate_logits, lam, z, h0, c):
         B, L, D = x.shape
         for name, t, n in (("gate_logits", gate_logits, 2 * B * L * D), ("lam", lam, D),
                            ("z", z, B * L * D), ("h0", h0, B * D)):
             if t is not None and t.numel() < n:
                 raise ValueError(f"{name}: fewer values ({t.numel()}) than the scan reads ({n})")
-        x, gate_logits, z = x.contiguous(), gate_logits.contiguous(), z.contiguous()
-        ctx.lam_dtype = lam.dtype
-        lam = lam.contiguous().float()
         desc = Desc(B, L, D, _dtype_code(x), c)
         ws = torch.empty(max(blr_workspace_bytes(desc), 16), dtype=torch.uint8, device=x.device)
         y = torch.empty_like(x)
@@ -54,18 +57,56 @@ class BDLRUGatedScan(torch.autograd.Function):
 
     @staticmethod
     def backward(ctx, dy, dh_last):
-        x, gate_logits, lam, z, h0, ws = ctx.saved_tensors
-        B, L, D = x.shape
+        x = ctx.saved_tensors[0]
         dy = torch.zeros_like(x) if dy is None else dy.contiguous().to(x.dtype)
         dh_last = None if dh_last is None else dh_last.contiguous().float()
-        dx = torch.empty_like(x)
-        dgl = torch.empty_like(gate_logits)
-        dz = torch.empty_like(z)
-        dlam = torch.empty(D, dtype=torch.float32, device=x.device)
-        dh0 = torch.empty(B, D, dtype=torch.float32, device=x.device) if h0 is not None else None
-        blr_scan_bwd_gated(ctx.desc, dy, dh_last, x, gate_logits, lam, h0, z, dx, dgl, dz, dlam,
-                           dh0, ws)
-        return dx, dgl, dlam.to(ctx.lam_dtype), dz, dh0, None
+        grad = _GatedScanGrad.apply if torch.is_grad_enabled() else _gated_scan_bwd
+        return (*grad(dy, dh_last, *ctx.saved_tensors, ctx.desc), None)
+
+
+def _gated_scan_bwd(dy, dh_last, x, gate_logits, lam, z, h0, ws, desc):
+    dx, dgl, dlam, dz = (torch.empty_like(t) for t in (x, gate_logits, lam, z))
+    dh0 = None
+    if h0 is not None:
+        dh0 = torch.empty(x.shape[0], x.shape[2], dtype=torch.float32, device=x.device)
+    blr_scan_bwd_gated(desc, dy, dh_last, x, gate_logits, lam, h0, z, dx, dgl, dz, dlam, dh0, ws)
+    return dx, dgl, dlam, dz, dh0
+
+
+def _gated_scan_torch(c, x, gate_logits, lam, z, h0):
+    """The gated scan's definition (Sec. 3.2) by torch operators, step by step."""
+    r, i = torch.sigmoid(gate_logits.float()).chunk(2, dim=-1)
+    log_a = -c * nn.functional.softplus(lam) * r
+    a, u = torch.exp(log_a), torch.sqrt(-torch.expm1(2 * log_a)) * i * x.float()
+    h = x.new_zeros(x.shape[0], x.shape[2], dtype=torch.float32) if h0 is None else h0
+    hs = []
+    for t in range(x.shape[1]):
+        h = a[:, t] * h + u[:, t]
+        hs.append(h)
+    return (torch.stack(hs, dim=1) * nn.functional.silu(z.float())).to(x.dtype), h
+
+
+def _gated_scan_grad_torch(c, dy, dh_last, *inputs):
+    at = [t if t is None or t.requires_grad else t.detach().requires_grad_() for t in inputs]
+    got = iter(torch.autograd.grad(_gated_scan_torch(c, *at), [t for t in at if t is not None],
+                                   (dy, dh_last), create_graph=True))
+    return tuple(None if t is None else next(got) for t in at)
+
+
+class _GatedScanGrad(torch.autograd.Function):
+    """BDLRUGatedScan's gradients as a function of their own (create_graph): computed
+    by the library's kernels, and differentiated again by the definition's operators."""
+
+    @staticmethod
+    def forward(ctx, dy, dh_last, x, gate_logits, lam, z, h0, ws, desc):
+        ctx.save_for_backward(dy, dh_last, x, gate_logits, lam, z, h0)
+        ctx.c = desc.c
+        return _gated_scan_bwd(dy, dh_last, x, gate_logits, lam, z, h0, ws, desc)
+
+    @staticmethod
+    def backward(ctx, *grads):
+        return (*_differentiable(lambda *t: _gated_scan_grad_torch(ctx.c, *t), ctx.saved_tensors,
+                                 grads), None, None)
 
 
 def _plain_cuda(dtype, *tensors) -> bool:
@@ -108,12 +149,14 @@ def _differentiable(fn, inputs, grads):
     (a layer applied twice), and what reaches it that way is not this call's."""
     graph = torch.is_grad_enabled()
     with torch.enable_grad():
-        at = [t.view_as(t) if graph else t.detach().requires_grad_(t.requires_grad) for t in inputs]
+        at = [t if t is None else t.view_as(t) if graph
+              else t.detach().requires_grad_(t.requires_grad) for t in inputs]
         outs = fn(*at)
         outs = outs if isinstance(outs, tuple) else (outs,)
-        need = [t for t in at if t.requires_grad]
+        outs, grads = zip(*((o, g) for o, g in zip(outs, grads) if o is not None))
+        need = [t for t in at if t is not None and t.requires_grad]
         got = iter(torch.autograd.grad(outs, need, grads, create_graph=graph))
-    return tuple(next(got) if t.requires_grad else None for t in at)
+    return tuple(next(got) if t is not None and t.requires_grad else None for t in at)
 
 
 def _linear_fwd(x, weight, bias):

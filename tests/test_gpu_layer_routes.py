@@ -10,20 +10,25 @@ if not torch.cuda.is_available():
     pytest.skip("no CUDA device", allow_module_level=True)
 
 
-def reference(layer, h):
-    """The layer's output in float64, its modules called one by one, the scan step by step."""
+def float64(layer, h):
+    """The layer and its input in float64 on the CPU, and its output by its modules
+    one by one, the scan step by step."""
     import copy
     m = copy.deepcopy(layer).cpu().double()
-    h, L = h.detach().double().cpu(), h.shape[1]
+    h = h.detach().double().cpu().requires_grad_()
     hx, hz = m.in_proj(h).chunk(2, dim=-1)
-    x = torch.nn.functional.silu(m.conv(hx.transpose(1, 2))[..., :L].transpose(1, 2))
+    x = torch.nn.functional.silu(m.conv(hx.transpose(1, 2))[..., :h.shape[1]].transpose(1, 2))
     r, i = torch.sigmoid(m.gate_proj(x)).chunk(2, dim=-1)
     a = torch.exp(-m.c * torch.nn.functional.softplus(m.lam) * r)
     u, state, ys = torch.sqrt(1 - a * a) * i * x, 0.0, []
-    for t in range(L):
+    for t in range(h.shape[1]):
         state = a[:, t] * state + u[:, t]
         ys.append(state)
-    return m.out_proj(torch.stack(ys, 1) * torch.nn.functional.silu(hz)).detach().numpy()
+    return m, h, m.out_proj(torch.stack(ys, 1) * torch.nn.functional.silu(hz))
+
+
+def close(got, want, tol):
+    assert normwise(got.detach().double().cpu().numpy(), want.detach().numpy()) <= tol
 
 
 @pytest.mark.parametrize("kw", [dict(padding=6, dilation=2), dict(padding=3, padding_mode="circular")])
@@ -36,4 +41,24 @@ def test_other_convolutions(kw):
     with torch.backends.cudnn.flags(enabled=True, allow_tf32=False):
         got = layer(h)
     # float32 throughout: the bound of the layer's kernels (1e-5)
-    assert normwise(got.detach().cpu().numpy(), reference(layer, h)) <= 1e-5
+    close(got, float64(layer, h)[2], 1e-5)
+
+
+def test_gradients_of_gradients():
+    """A gradient penalty of the whole layer, scan included. Float32 evaluations of
+    the formulas over 20 steps whose 1 / (1 - alpha^2) is about 10: 2^-24 * 20 * 10
+    * 10 operations, 1e-4."""
+    from paper_2406_12580_gb300.layer import GatedRecurrentLayer
+    torch.manual_seed(12)
+    layer = GatedRecurrentLayer(16, device="cuda")
+    h = torch.randn(3, 20, 16, device="cuda", requires_grad=True)
+    y = layer(h)
+    assert "LayerF32" in type(y.grad_fn).__name__
+    m, h64, y64 = float64(layer, h)
+    both = []
+    for mod, inp, out in ((layer, h, y), (m, h64, y64)):
+        ins = [inp, *mod.parameters()]
+        first = torch.autograd.grad(out.square().sum(), ins, create_graph=True)
+        both.append(first + torch.autograd.grad(sum(g.square().sum() for g in first), ins))
+    for got, want in zip(*both):
+        close(got, want, 1e-4)

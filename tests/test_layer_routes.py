@@ -77,9 +77,41 @@ def kernels_on_cpu(monkeypatch):
         for to, of in zip((x, z), layer_module._conv_silu_torch(hxz, w, b)):
             to.copy_(of)
 
+    def definition(c, x, gl, lam, z, h0):
+        """The gated scan in float64, written out from Sec. 3.2."""
+        D = x.shape[2]
+        r, i = torch.sigmoid(gl[..., :D]), torch.sigmoid(gl[..., D:])
+        a = torch.exp(-c * r * torch.log1p(torch.exp(lam)))
+        h, hs = (0.0 if h0 is None else h0), []
+        for t in range(x.shape[1]):
+            h = a[:, t] * h + torch.sqrt(1 - a[:, t] ** 2) * i[:, t] * x[:, t]
+            hs.append(h)
+        return torch.stack(hs, 1) * z * torch.sigmoid(z), h
+
+    def scan_fwd(desc, x, gl, lam, h0, z, y, h_last, ws):
+        ins = [None if t is None else t.double() for t in (x, gl, lam, z, h0)]
+        for to, of in zip((y, h_last), definition(desc.c, *ins)):
+            if to is not None:
+                to.copy_(of)
+
+    def scan_bwd(desc, dy, dh_last, x, gl, lam, h0, z, dx, dgl, dz, dlam, dh0, ws):
+        with torch.enable_grad():
+            ins = [None if t is None else t.detach().double().requires_grad_() for t in (x, gl, lam, z, h0)]
+            outs = definition(desc.c, *ins)
+            dh_last = torch.zeros_like(outs[1]) if dh_last is None else dh_last
+            got = torch.autograd.grad(outs, [t for t in ins if t is not None],
+                                      (dy.double(), dh_last.double()))
+        for to, of in zip((dx, dgl, dlam, dz, dh0), got):
+            to.copy_(of)
+
+    monkeypatch.setattr(layer_module, "blr_scan_fwd_gated", scan_fwd)
+    monkeypatch.setattr(layer_module, "blr_scan_bwd_gated", scan_bwd)
+    monkeypatch.setattr(layer_module, "blr_workspace_bytes", lambda d: 64)
     monkeypatch.setattr(layer_module, "_dtype_code", lambda t: 0)
+    kernels = dict(definition=definition)
     monkeypatch.setattr(layer_module, "blr_linear_fwd", linear_fwd)
     monkeypatch.setattr(layer_module, "blr_conv_silu_fwd", conv_fwd)
+    return kernels
 
 
 def _grads(out, inputs, create_graph):
@@ -110,6 +142,45 @@ def test_gradients_by_torch_operators_are_this_calls_own(kernels_on_cpu, graph):
             kernel = got
     for a, r in zip(kernel, got):  # the same operators in the same precision: float64's rounding
         assert (a - r).abs().max() <= 1e-12 * r.abs().max() and a.requires_grad == r.requires_grad
+
+
+@pytest.mark.parametrize("state", [False, True])
+def test_second_gradients_pass_through_the_scan(kernels_on_cpu, state):
+    """A gradient penalty through the gated scan has every term, for inputs of other
+    strides too, and the first gradients under create_graph are the kernels'. Both
+    sides are float32 evaluations of the same formulas over 12 steps whose 1 / (1 -
+    alpha^2) is about 10: 2^-24 * 12 * 10 * 10 operations, 1e-4."""
+    torch.manual_seed(9)
+    rand = lambda *s: torch.randn(*s, requires_grad=True)  # noqa: E731
+    x, gl, lam, z = rand(6, 12, 3), rand(3, 12, 12), rand(6), rand(3, 12, 6)
+    h0 = rand(3, 6) if state else None
+    ins = [t for t in (x, gl, lam, z, h0) if t is not None]
+    seen = []
+    for scan, to in ((layer_module.BDLRUGatedScan.apply, torch.Tensor.float),
+                     (lambda x, gl, lam, z, h0: kernels_on_cpu["definition"](1.0, x, gl, lam, z, h0),
+                      torch.Tensor.double)):
+        args = [None if t is None else to(t) for t in (x.transpose(0, 2), gl, lam, z, h0)]
+        y, h_last = scan(*args)
+        seen.append(_grads((y.square().sum() + h_last.sum()).sum(), ins, True))
+    for a, r in zip(*seen):
+        assert (a - r).abs().max() <= 1e-4 * r.abs().max()
+
+
+def test_second_gradients_of_the_whole_layer(kernels_on_cpu, monkeypatch):
+    torch.manual_seed(10)
+    layer, h = layer_module.GatedRecurrentLayer(8), torch.randn(2, 9, 8, requires_grad=True)
+    p = [dict(layer.named_parameters())[n] for n in
+         ("in_proj.weight", "in_proj.bias", "conv.weight", "conv.bias", "gate_proj.weight",
+          "gate_proj.bias", "lam", "out_proj.weight", "out_proj.bias")]
+    out = layer_module._LayerF32.apply(1.0, h, *p)
+    got = _grads(out.square().sum(), [h, *p], True)
+    p64, h64 = [t.detach().double().requires_grad_() for t in p], h.detach().double().requires_grad_()
+    hxz = nn.functional.linear(h64, p64[0], p64[1])
+    x, z = layer_module._conv_silu_torch(hxz, p64[2], p64[3])
+    y, _ = kernels_on_cpu["definition"](1.0, x, nn.functional.linear(x, p64[4], p64[5]), p64[6], z, None)
+    want = _grads(nn.functional.linear(y, p64[7], p64[8]).square().sum(), [h64, *p64], True)
+    for a, r in zip(got, want):
+        assert (a - r).abs().max() <= 1e-4 * r.abs().max()
 
 
 @pytest.mark.parametrize("n,k,kernel", [(65536, 4, True), (65540, 4, False), (4, 65540, False),
