@@ -42,6 +42,8 @@
  *          softplus(Lambda) > 0 in float32 (|rho| below about 80). At
  *          alpha_t == 1 exactly the gradient through beta_t is infinite
  *          (the derivative of sqrt(1 - alpha^2)); such inputs give inf/nan.
+ *          An infinite state or adjoint stays infinite from its step on, as in
+ *          the definition (bfloat16 scans: an infinite x with iota < 0 gives nan).
  * Errors   The library never exits, traps or prints. Waits between thread
  *          blocks are bounded (about one second); an expired wait is recorded
  *          in the workspace and reported by blr_workspace_status().

@@ -433,7 +433,7 @@ __global__ void __maxnreg__(kTeamMaxRegs)
 #pragma unroll
         for (int w = NW - 1; w >= 0; --w) {
           const float2 e = w < ns ? maps[(m * NW + w) * CHW + lane * VEC + v] : make_float2(0.0f, 0.0f);
-          TU[v] = map_apply(e.x, TU[v], e.y);
+          TU[v] = map_apply_any(e.x, TU[v], e.y);
           TM[v] = m_compose(TM[v], e.x);
         }
       }
@@ -455,7 +455,7 @@ __global__ void __maxnreg__(kTeamMaxRegs)
         if (records && !last) {
 #pragma unroll
           for (int v = 0; v < VEC; ++v)
-            st_record(&inc[rec + v], __float_as_uint(map_apply(TM[v], ws[v], TU[v])));
+            st_record(&inc[rec + v], __float_as_uint(map_apply_any(TM[v], ws[v], TU[v])));
         }
       } else {
         ahead();
@@ -467,7 +467,7 @@ __global__ void __maxnreg__(kTeamMaxRegs)
 #pragma unroll
       for (int v = 0; v < VEC; ++v) {
         carries[m * CHW + lane * VEC + v] = ws[v];
-        carry[v] = map_apply(TM[v], ws[v], TU[v]);
+        carry[v] = map_apply_any(TM[v], ws[v], TU[v]);
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(&carry_ready[m]);
@@ -607,6 +607,13 @@ __global__ void __maxnreg__(kTeamMaxRegs)
         for (int o = ns - 1; o > w; --o) {
           const float2 e0 = mp[o * CHW], e1 = mp[o * CHW + VEC - 1];
           win = map_apply2(make_float2(e0.x, e1.x), win, make_float2(e0.y, e1.y));
+        }
+        if (__any_sync(kFull, !all_finite(win))) {
+          tmem_ld_wait(pr);
+          if constexpr (GATED) tmem_ld8_ready(merge);
+          const float2 in = make_float2(carries[mq * CHW + lane * VEC], carries[mq * CHW + lane * VEC + VEC - 1]);
+          win = team_enter_any<T>(from, mp + (ns - 1) * CHW, ns - 1 - w, -1, in);
+          tmem_ld16_start(from, pr);
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&maps_read[mq]);

@@ -257,7 +257,7 @@ __global__ void __maxnreg__(kTeamMaxRegs)
 #pragma unroll
         for (int w = 0; w < NW; ++w) {
           const float2 e = w < ns ? maps[(m * NW + w) * CHW + lane * VEC + v] : make_float2(0.0f, 0.0f);
-          TU[v] = map_apply(e.x, TU[v], e.y);
+          TU[v] = map_apply_any(e.x, TU[v], e.y);
           TM[v] = m_compose(TM[v], e.x);
         }
       }
@@ -279,7 +279,7 @@ __global__ void __maxnreg__(kTeamMaxRegs)
         if (records && !last) {
 #pragma unroll
           for (int v = 0; v < VEC; ++v)
-            st_record(&inc[rec + v], __float_as_uint(map_apply(TM[v], hs[v], TU[v])));
+            st_record(&inc[rec + v], __float_as_uint(map_apply_any(TM[v], hs[v], TU[v])));
         }
       } else {
         refill();
@@ -291,7 +291,7 @@ __global__ void __maxnreg__(kTeamMaxRegs)
 #pragma unroll
       for (int v = 0; v < VEC; ++v) {
         carries[m * CHW + lane * VEC + v] = hs[v];
-        carry[v] = map_apply(TM[v], hs[v], TU[v]);
+        carry[v] = map_apply_any(TM[v], hs[v], TU[v]);
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(&carry_ready[m]);
@@ -393,6 +393,12 @@ __global__ void __maxnreg__(kTeamMaxRegs)
         for (int o = 0; o < w; ++o) {
           const float2 e0 = mp[o * CHW], e1 = mp[o * CHW + VEC - 1];
           hs = map_apply2(make_float2(e0.x, e1.x), hs, make_float2(e0.y, e1.y));
+        }
+        if (__any_sync(kFull, !all_finite(hs))) {
+          tmem_ld_wait(pr0);
+          const float2 in = make_float2(carries[mq * CHW + lane * VEC], carries[mq * CHW + lane * VEC + VEC - 1]);
+          hs = team_enter_any<T>(tq + mq * COLS, mp, w, 1, in);
+          tmem_ld16_start(tq + mq * COLS, pr0);
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&maps_read[mq]);
