@@ -7,16 +7,21 @@
     H_o      = Linear(H'_y)                        reduce E D -> D
 
 The scan and the merge, forward and backward, run in the library
-(``BDLRUGatedScan``). So do the convolution with its SiLU (``blr_conv_silu_*``,
-float32 and bfloat16) and the float32 projections (``blr_linear_*``) on a CUDA
-device in plain eager execution; elsewhere (autocast, TF32 allowed, traced, under
-a dispatch or function mode or transformed by functorch, forward-mode AD, tensor subclasses, other dtypes,
-devices or widths, hooks on the convolution) they are the torch operators. The
+(``BDLRUGatedScan``). So do, on a CUDA device in plain eager execution, the
+convolution with its SiLU (``blr_conv_silu_*``, float32 and bfloat16) and the
+float32 projections of the sizes at which its kernels are the faster ones
+(``blr_linear_*``, ``_own_product``). Elsewhere (autocast, TF32 allowed, traced,
+under a dispatch or function mode or transformed by functorch, forward-mode AD,
+tensor subclasses, other dtypes, devices or widths, hooks on the modules, a
+convolution of other settings) they are the torch operators. The
 decay parameter Lambda is initialised as in Sec. 3.2: exp(-softplus(Lambda))
 uniform in [0.9, 0.999]. The convolution width is not given in the paper; it
 is a parameter (default 4).
 """
 from __future__ import annotations
+
+import functools
+import threading
 
 import torch
 from torch import nn
@@ -134,13 +139,10 @@ def _plain_cuda(dtype, *tensors) -> bool:
 def _tf32() -> bool:
     """Whether torch may run float32 products in TF32, by either of its settings
     (reading the older one raises once the newer one says something else)."""
-    mm = torch.backends.cuda.matmul
     try:
-        if hasattr(mm, "fp32_precision"):
-            return mm.fp32_precision not in ("none", "ieee")
-        return mm.allow_tf32
-    except RuntimeError:
-        return True
+        return torch.backends.cuda.matmul.fp32_precision not in ("none", "ieee")
+    except AttributeError:
+        return torch.backends.cuda.matmul.allow_tf32
 
 
 def _differentiable(fn, inputs, grads):
@@ -159,17 +161,83 @@ def _differentiable(fn, inputs, grads):
     return tuple(next(got) if t is not None and t.requires_grad else None for t in at)
 
 
-def _linear_fwd(x, weight, bias):
+_OWN_NK = 1 << 19
+_products = threading.local()  # .ready: devices on which this thread may capture torch's products
+
+
+def _own_product(T: int, n: int, k: int) -> bool:
+    """Whether a projection of T rows, n outputs and k inputs runs on the library's
+    kernels: where they are the faster ones on the device, and in eager execution
+    also where they take less there than torch's products take to be launched. The
+    kernels tile the outputs: few rows of a wide projection leave the GPU idle, and
+    its weight gradient is split too finely. Device time of torch's products over
+    theirs, forward and both gradients, for 128, 512, 1600, 6400 and 51200 rows:
+    64 x 32 (n x k) 0.83 1.27 1.89 2.21 4.17, 128 x 64 0.71 1.03 1.41 1.47 3.78,
+    256 x 128 0.54 0.73 0.96 1.63 1.69, 512 x 256 0.39 0.50 0.85 1.23 1.24, 1024 x 256
+    0.27 0.40 0.65 0.99 1.10, 1024 x 512 0.27 0.37 0.65 0.92 0.96, 2048 x 1024 0.21 0.35
+    0.55 0.69 0.76. Launching one's forward and gradients takes torch 85 us, the
+    library 25, while 1 << 30 multiply-adds take 160 us on the device: a whole layer
+    of them no longer than the 545 us its other launches take. A captured graph pays
+    for no launch: there the device decides (a layer of 128 x 2 channels at 200 rows,
+    forward and backward: 205 us captured on the kernels, 115 on the products; eager
+    545 and 860), if a pass before the capture could set the products up: they
+    cannot be set up during one."""
+    return _own_products(T, ((n, k),))[0]
+
+
+def _own_products(T, sizes):
+    """_own_product for several projections of the same rows: [(n, k), ...]."""
+    kinds = _product_kinds(T, sizes)
+    if kinds is _OWN:
+        return _ALL
+    device = torch._C._cuda_getDevice()
+    ready = getattr(_products, "ready", ())
+    if torch.cuda.is_current_stream_capturing():
+        return [k == "own" or k != "torch" and device not in ready for k in kinds]
+    if device not in ready:
+        torch.cuda.current_blas_handle()
+        _products.ready = (*ready, device)
+    return [k == "own" or k == "eager" for k in kinds]
+
+
+_OWN, _ALL = ("own",), (True, True, True)
+
+
+@functools.lru_cache(maxsize=1024)
+def _product_kinds(T, sizes):
+    """For each: own, on the library's kernels; eager, there but in a capture; device,
+    only in a capture that could not take torch's; torch, never. _OWN: all own."""
+    kinds = []
+    for n, k in sizes:
+        nk = n * k
+        if n % 4 != 0 or k % 4 != 0 or n > 65536 or k > 65536:
+            kinds.append("torch")
+        elif nk <= 2048 or nk <= 1 << 18 and T * T >= 100 * nk:
+            kinds.append("own")
+        else:
+            kinds.append("eager" if nk <= _OWN_NK and T * nk <= 1 << 30 else "device")
+    return _OWN if all(k == "own" for k in kinds) else kinds
+
+
+def _linear_fwd(own, x, weight, bias):
+    if not own:
+        return nn.functional.linear(x, weight, bias)
     N, K = weight.shape
     y = x.new_empty(*x.shape[:-1], N)
     blr_linear_fwd(x.numel() // K, N, K, x, weight, bias, y)
     return y
 
 
-def _linear_bwd(dy, x, weight, dx, with_weight, add_dx=False):
+def _linear_bwd(own, dy, x, weight, dx, with_weight, add_dx=False):
     """dx into `dx` (None: not computed); returns (dweight, dbias), or Nones."""
     N, K = weight.shape
     T = x.numel() // K
+    if not own:
+        dy = dy.view(T, N)
+        if dx is not None:
+            to = dx.view(T, K)
+            to.addmm_(dy, weight) if add_dx else torch.mm(dy, weight, out=to)
+        return (torch.mm(dy.t(), x.view(T, K)), dy.sum(0)) if with_weight else (None, None)
     dw = db = ws = None
     if with_weight:
         dw, db = torch.empty_like(weight), weight.new_empty(N)
@@ -185,33 +253,33 @@ class _LinearF32(torch.autograd.Function):
     @staticmethod
     def forward(ctx, x, weight, bias):
         ctx.save_for_backward(x, weight, bias)  # as they came: create_graph needs their history
-        return _linear_fwd(x.contiguous(), weight.contiguous(), bias.contiguous())
+        own = _own_product(x.numel() // x.shape[-1], *weight.shape)
+        return _linear_fwd(own, x.contiguous(), weight.contiguous(), bias.contiguous())
 
     @staticmethod
     def backward(ctx, dy):
         x, weight, bias = ctx.saved_tensors
         if torch.is_grad_enabled() or not _plain_cuda(torch.float32, dy, x, weight):
             return _differentiable(nn.functional.linear, (x, weight, bias), (dy,))
+        need = ctx.needs_input_grad
         x, weight = x.contiguous(), weight.contiguous()
-        dx = torch.empty_like(x) if ctx.needs_input_grad[0] else None
-        dw, db = _linear_bwd(dy.contiguous(), x, weight, dx, any(ctx.needs_input_grad[1:]))
-        return dx, dw if ctx.needs_input_grad[1] else None, db if ctx.needs_input_grad[2] else None
-
-
-def _linear_ok(n: int, k: int) -> bool:
-    """Whether the kernels take a projection of n outputs and k inputs."""
-    return n % 4 == 0 and k % 4 == 0 and n <= 65536 and k <= 65536
+        dx = torch.empty_like(x) if need[0] else None
+        own = _own_product(x.numel() // x.shape[-1], *weight.shape)
+        dw, db = _linear_bwd(own, dy.contiguous(), x, weight, dx, need[1] or need[2])
+        return dx, dw if need[1] else None, db if need[2] else None
 
 
 class _Linear(nn.Linear):
-    """nn.Linear whose float32 product runs in the library (in float32: where
-    TF32 is allowed it stays with torch)."""
+    """nn.Linear whose float32 product may run in the library (in float32: where
+    TF32 is allowed it stays with torch, as ones too wide for it at any rows do)."""
 
     def forward(self, x):
         w, b = self.weight, self.bias
-        if (b is not None and w.dtype == torch.float32 and w.dim() == 2 and _linear_ok(*w.shape)
-                and b.shape == w.shape[:1] and x.dim() > 1 and x.shape[-1] == w.shape[1]
-                and _plain_cuda(torch.float32, x, w, b) and not _tf32()):
+        if (b is not None and w.dtype == torch.float32 and w.dim() == 2 and b.shape == w.shape[:1]
+                and x.dim() > 1 and x.shape[-1] == w.shape[1]
+                and w.shape[0] % 4 == 0 and w.shape[1] % 4 == 0
+                and _plain_cuda(torch.float32, x, w, b) and not _tf32()
+                and (w.numel() <= _OWN_NK or _own_product(x.numel() // w.shape[1], *w.shape))):
             return _LinearF32.apply(x, w, b)
         return super().forward(x)
 
@@ -264,6 +332,10 @@ def _layer_torch(c, h, w_in, b_in, w_conv, b_conv, w_gate, b_gate, lam, w_out, b
     return nn.functional.linear(y, w_out, b_out)
 
 
+def _layer_products(h, *weights):
+    return _own_products(h.numel() // h.shape[-1], tuple([tuple(w.shape) for w in weights]))
+
+
 class _LayerF32(torch.autograd.Function):
     """The whole layer in float32 on the library's kernels: one node in the graph
     instead of five, and the gate projection's gradient of the scan's input added
@@ -271,9 +343,10 @@ class _LayerF32(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, c, h, w_in, b_in, w_conv, b_conv, w_gate, b_gate, lam, w_out, b_out):
-        hxz = _linear_fwd(h.contiguous(), w_in, b_in)
+        own = _layer_products(h, w_in, w_gate, w_out)
+        hxz = _linear_fwd(own[0], h.contiguous(), w_in, b_in)
         x, z = _conv_fwd(hxz, w_conv, b_conv)
-        gl = _linear_fwd(x, w_gate, b_gate)
+        gl = _linear_fwd(own[1], x, w_gate, b_gate)
         B, L, D = x.shape
         desc = Desc(B, L, D, 0, c)
         ws = torch.empty(blr_workspace_bytes(desc), dtype=torch.uint8, device=x.device)
@@ -282,7 +355,7 @@ class _LayerF32(torch.autograd.Function):
         ctx.desc = desc
         ctx.save_for_backward(h, w_in, b_in, w_conv, b_conv, w_gate, b_gate, lam, w_out, b_out,
                               hxz, x, z, gl, y, ws)
-        return _linear_fwd(y, w_out, b_out)
+        return _linear_fwd(own[2], y, w_out, b_out)
 
     @staticmethod
     def backward(ctx, dout):
@@ -295,26 +368,27 @@ class _LayerF32(torch.autograd.Function):
                                            (h, w_in, b_in, w_conv, b_conv, w_gate, b_gate, lam,
                                             w_out, b_out), (dout,)))
         dout, h = dout.contiguous(), h.contiguous()
+        own = _layer_products(h, w_in, w_gate, w_out)
         dy = torch.empty_like(y)
-        dw_out, db_out = _linear_bwd(dout, y, w_out, dy, need[8] or need[9])
+        dw_out, db_out = _linear_bwd(own[2], dout, y, w_out, dy, need[8] or need[9])
         dx, dz, dgl, dlam = (torch.empty_like(t) for t in (x, z, gl, lam))
         blr_scan_bwd_gated(ctx.desc, dy, None, x, gl, lam, None, z, dx, dgl, dz, dlam, None, ws)
-        dw_gate, db_gate = _linear_bwd(dgl, x, w_gate, dx, need[5] or need[6], add_dx=True)
+        dw_gate, db_gate = _linear_bwd(own[1], dgl, x, w_gate, dx, need[5] or need[6], add_dx=True)
         dhxz, dw_conv, db_conv = _conv_bwd(dx, dz, hxz, w_conv, b_conv)
         dh = torch.empty_like(h) if need[0] else None
-        dw_in, db_in = _linear_bwd(dhxz, h, w_in, dh, need[1] or need[2])
+        dw_in, db_in = _linear_bwd(own[0], dhxz, h, w_in, dh, need[1] or need[2])
         grads = (dh, dw_in, db_in, dw_conv, db_conv, dw_gate, db_gate, dlam, dw_out, db_out)
         return (None, *(g if n else None for g, n in zip(grads, need)))
 
 
-_GLOBAL_HOOKS = ("_global_forward_hooks", "_global_forward_pre_hooks", "_global_backward_hooks",
-                 "_global_backward_pre_hooks")
+def _hooks_on_all() -> bool:
+    m = nn.modules.module
+    return bool(m._global_forward_hooks or m._global_forward_pre_hooks or m._global_backward_hooks
+                or m._global_backward_pre_hooks)
 
 
 def _bare(module, kind) -> bool:
-    """Whether calling the module is its forward and nothing else."""
-    if any(getattr(nn.modules.module, n) for n in _GLOBAL_HOOKS):
-        return False
+    """Whether calling the module is its forward and nothing else (but for hooks on all)."""
     return (type(module) is kind and module.bias is not None and not module._forward_hooks
             and not module._forward_pre_hooks and not module._backward_hooks
             and not module._backward_pre_hooks and "forward" not in module.__dict__)
@@ -346,14 +420,16 @@ class GatedRecurrentLayer(nn.Module):
     def _conv_ok(self) -> bool:
         """Whether the convolution is the kernels': depthwise, 4 taps, causal by zeros."""
         c = self.conv
-        return (_bare(c, nn.Conv1d) and c.weight.shape == (self.ed, 1, 4)
-                and c.bias.shape == (self.ed,) and c.groups == self.ed and c.stride == (1,) and c.dilation == (1,) and c.padding == (3,)
-                and c.padding_mode == "zeros" and self.ed <= 1024)
+        return (_bare(c, nn.Conv1d) and not _hooks_on_all() and self.ed <= 1024 and c.groups == self.ed
+                and c.kernel_size == (4,) and c.stride == (1,) and c.dilation == (1,)
+                and c.padding == (3,) and c.padding_mode == "zeros")
 
     def _conv_silu(self, hxz):
         """The scan's inputs from the expansion's output: SiLU(conv(H_x)) and H_z."""
-        conv = self.conv
-        if (self._conv_ok() and hxz.dim() == 3 and hxz.shape[-1] == 2 * self.ed and hxz.dtype in (torch.float32, torch.bfloat16)
+        conv, ed = self.conv, self.ed
+        if (self._conv_ok() and hxz.dtype in (torch.float32, torch.bfloat16)
+                and hxz.dim() == 3 and hxz.shape[-1] == 2 * ed
+                and conv.weight.shape == (ed, 1, 4) and conv.bias.shape == (ed,)
                 and _plain_cuda(hxz.dtype, hxz, conv.weight, conv.bias)):
             return _ConvSiLU.apply(hxz, conv.weight, conv.bias)
         hx, hz = hxz.split(self.ed, dim=-1)
@@ -366,13 +442,13 @@ class GatedRecurrentLayer(nn.Module):
         if not (self._conv_ok() and _bare(i, _Linear) and _bare(g, _Linear) and _bare(o, _Linear)):
             return None
         ed, d, n = self.ed, h.shape[-1], o.bias.shape[0]
-        if h.dim() != 3 or not _linear_ok(ed, d) or not _linear_ok(n, ed):
+        if h.dim() != 3 or d % 4 != 0 or n % 4 != 0:
             return None
         p = (i.weight, i.bias, self.conv.weight, self.conv.bias, g.weight, g.bias, self.lam,
              o.weight, o.bias)
-        # the kernels take the sizes as given: parameters of others go to the operators, which refuse them
-        if [t.shape for t in p] != [(2 * ed, d), (2 * ed,), (ed, 1, 4), (ed,), (2 * ed, ed), (2 * ed,),
-                                    (ed,), (n, ed), (n,)]:
+        # the kernels take the sizes as given: parameters of others are left to the operators to refuse
+        if [t.shape for t in p] != [(2 * ed, d), (2 * ed,), (ed, 1, 4), (ed,), (2 * ed, ed),
+                                    (2 * ed,), (ed,), (n, ed), (n,)]:
             return None
         if (not _plain_cuda(torch.float32, h, *p) or not all(t.is_contiguous() for t in p)
                 or _tf32()):

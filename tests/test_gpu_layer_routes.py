@@ -62,3 +62,40 @@ def test_gradients_of_gradients():
         both.append(first + torch.autograd.grad(sum(g.square().sum() for g in first), ins))
     for got, want in zip(*both):
         close(got, want, 1e-4)
+
+
+@pytest.mark.parametrize("captured", [False, True])
+@pytest.mark.parametrize("B,L", [(2, 20), (35, 20), (33, 31), (60, 31)])
+def test_projections_by_either_product(B, L, captured):
+    """Captured, one, two or all of the layer's projections (128 x 32, 128 x 64, 32 x
+    64) run on the library's kernels and the others on torch's products, by the rows:
+    the output and every gradient. Five float32 stages of 1e-5 each."""
+    from paper_2406_12580_gb300.layer import GatedRecurrentLayer, _own_product
+    torch.manual_seed(13)
+    layer = GatedRecurrentLayer(32, device="cuda")
+    h = torch.randn(B, L, 32, device="cuda", requires_grad=True)
+    dy = torch.randn(B, L, 32, device="cuda")
+
+    def run():
+        y = layer(h)
+        assert "LayerF32" in type(y.grad_fn).__name__
+        own = [_own_product(B * L, n, k) for n, k in ((128, 32), (128, 64), (32, 64))]
+        assert own == ([B * L >= 640, B * L >= 906, True] if captured else [True] * 3)
+        return y, *torch.autograd.grad(y, [h, *layer.parameters()], dy)
+
+    if captured:
+        side = torch.cuda.Stream()
+        side.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(side):
+            layer(h).backward(dy)  # a capture follows an eager pass
+        torch.cuda.current_stream().wait_stream(side)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            got = run()
+        graph.replay()
+    else:
+        got = run()
+    m, h64, y64 = float64(layer, h)
+    want = torch.autograd.grad(y64, [h64, *m.parameters()], dy.double().cpu())
+    for g, w in zip(got, (y64, *want)):
+        close(g, w, 5e-5)

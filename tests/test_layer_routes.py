@@ -74,8 +74,8 @@ def kernels_on_cpu(monkeypatch):
 
     def conv_fwd(B, L, C, io, hxz, w, b, x, z):
         assert hxz.is_contiguous()
-        for to, of in zip((x, z), layer_module._conv_silu_torch(hxz, w, b)):
-            to.copy_(of)
+        for to, of in zip((x, z), layer_module._conv_silu_torch(hxz.view(B, L, 2 * C), w, b)):
+            to.copy_(of.reshape(to.shape))
 
     def definition(c, x, gl, lam, z, h0):
         """The gated scan in float64, written out from Sec. 3.2."""
@@ -89,10 +89,11 @@ def kernels_on_cpu(monkeypatch):
         return torch.stack(hs, 1) * z * torch.sigmoid(z), h
 
     def scan_fwd(desc, x, gl, lam, h0, z, y, h_last, ws):
-        ins = [None if t is None else t.double() for t in (x, gl, lam, z, h0)]
+        ins = [t.double().view(desc.B, desc.L, -1) for t in (x, gl, z)]
+        ins = (ins[0], ins[1], lam.double(), ins[2], None if h0 is None else h0.double())
         for to, of in zip((y, h_last), definition(desc.c, *ins)):
             if to is not None:
-                to.copy_(of)
+                to.copy_(of.reshape(to.shape))
 
     def scan_bwd(desc, dy, dh_last, x, gl, lam, h0, z, dx, dgl, dz, dlam, dh0, ws):
         with torch.enable_grad():
@@ -108,6 +109,7 @@ def kernels_on_cpu(monkeypatch):
     monkeypatch.setattr(layer_module, "blr_scan_bwd_gated", scan_bwd)
     monkeypatch.setattr(layer_module, "blr_workspace_bytes", lambda d: 64)
     monkeypatch.setattr(layer_module, "_dtype_code", lambda t: 0)
+    monkeypatch.setattr(layer_module, "_own_products", lambda T, sizes: (True,) * len(sizes))
     kernels = dict(definition=definition)
     monkeypatch.setattr(layer_module, "blr_linear_fwd", linear_fwd)
     monkeypatch.setattr(layer_module, "blr_conv_silu_fwd", conv_fwd)
@@ -183,12 +185,46 @@ def test_second_gradients_of_the_whole_layer(kernels_on_cpu, monkeypatch):
         assert (a - r).abs().max() <= 1e-4 * r.abs().max()
 
 
+@pytest.fixture
+def device_state(monkeypatch):
+    """The calls by which the rule for a projection asks about the device."""
+    state = dict(capturing=False, handles=0)
+    monkeypatch.setattr(torch._C, "_cuda_getDevice", lambda: 0, raising=False)
+    monkeypatch.setattr(torch.cuda, "is_current_stream_capturing", lambda: state["capturing"])
+    monkeypatch.setattr(torch.cuda, "current_blas_handle",
+                        lambda: state.update(handles=state["handles"] + 1))
+    monkeypatch.setattr(layer_module, "_products", type(layer_module._products)())
+    return state
+
+
+def test_rule_for_a_projection(device_state):
+    """The library's kernels where they are the faster, or launched the faster; in a
+    capture by device time, but torch's products only once they have been set up in
+    the thread, by an eager pass."""
+    own, state = layer_module._own_product, device_state
+    always = ((50, 64, 32), (51200, 256, 128), (10240, 1024, 256))
+    eager = ((50, 256, 128), (200, 1024, 512), (4000, 1024, 256))
+    never = ((200, 2048, 1024), (51200, 1024, 1024), (3000, 1024, 512))
+    state["capturing"] = True
+    assert all(own(*s) for s in always + eager + never)
+    state["capturing"] = False
+    assert all(own(*s) for s in always) and state["handles"] == 0
+    assert all(own(*s) for s in eager) and state["handles"] == 1
+    assert not any(own(*s) for s in never)
+    state["capturing"] = True
+    assert all(own(*s) for s in always) and not any(own(*s) for s in eager + never)
+    assert state["handles"] == 1
+    assert not own(50, 65540, 4) and not own(50, 6, 4)  # the kernels refuse them
+
+
 @pytest.mark.parametrize("n,k,kernel", [(65536, 4, True), (65540, 4, False), (4, 65540, False),
                                         (6, 4, False), (4, 6, False)])
-def test_projections_the_kernels_refuse_stay_with_torch(monkeypatch, n, k, kernel):
+def test_projections_the_kernels_refuse_stay_with_torch(monkeypatch, device_state, n, k, kernel):
     monkeypatch.setattr(layer_module, "_plain_cuda", lambda *a: True)
-    monkeypatch.setattr(layer_module._LinearF32, "apply", staticmethod(lambda x, w, b: "kernel"))
-    assert isinstance(layer_module._Linear(k, n)(torch.randn(2, k)), str) == kernel
+    called = []
+    monkeypatch.setattr(layer_module, "blr_linear_fwd", lambda *a: called.append(a))
+    y = layer_module._Linear(k, n)(torch.randn(2, k))
+    assert y.shape == (2, n) and len(called) == kernel
 
 
 @pytest.mark.parametrize("name,shape", [
