@@ -165,7 +165,7 @@ _OWN_NK = 1 << 19
 _products = threading.local()  # .ready: devices on which this thread may capture torch's products
 
 
-def _own_product(T: int, n: int, k: int) -> bool:
+def _own_product(T: int, n: int, k: int, forward: bool = False) -> bool:
     """Whether a projection of T rows, n outputs and k inputs runs on the library's
     kernels: where they are the faster ones on the device, and in eager execution
     also where they take less there than torch's products take to be launched. The
@@ -175,19 +175,21 @@ def _own_product(T: int, n: int, k: int) -> bool:
     64 x 32 (n x k) 0.83 1.27 1.89 2.21 4.17, 128 x 64 0.71 1.03 1.41 1.47 3.78,
     256 x 128 0.54 0.73 0.96 1.63 1.69, 512 x 256 0.39 0.50 0.85 1.23 1.24, 1024 x 256
     0.27 0.40 0.65 0.99 1.10, 1024 x 512 0.27 0.37 0.65 0.92 0.96, 2048 x 1024 0.21 0.35
-    0.55 0.69 0.76. Launching one's forward and gradients takes torch 85 us, the
+    0.55 0.69 0.76. The forward alone keeps ahead longer, inner sums of up to 512 over
+    enough outputs (3200 x 1024 x 256 1.24, 1600 x 1024 x 256 0.92, 6400 x 2048 x 512
+    1.07, 1600 x 1024 x 512 0.77, 51200 x 1024 x 1024 0.96). Launching one's forward and gradients takes torch 85 us, the
     library 25, while 1 << 30 multiply-adds take 160 us on the device: a whole layer
     of them no longer than the 545 us its other launches take. A captured graph pays
     for no launch: there the device decides (a layer of 128 x 2 channels at 200 rows,
     forward and backward: 205 us captured on the kernels, 115 on the products; eager
     545 and 860), if a pass before the capture could set the products up: they
     cannot be set up during one."""
-    return _own_products(T, ((n, k),))[0]
+    return _own_products(T, ((n, k),), forward)[0]
 
 
-def _own_products(T, sizes):
+def _own_products(T, sizes, forward=False):
     """_own_product for several projections of the same rows: [(n, k), ...]."""
-    kinds = _product_kinds(T, sizes)
+    kinds = _product_kinds(T, sizes, forward)
     if kinds is _OWN:
         return _ALL
     device = torch._C._cuda_getDevice()
@@ -204,7 +206,7 @@ _OWN, _ALL = ("own",), (True, True, True)
 
 
 @functools.lru_cache(maxsize=1024)
-def _product_kinds(T, sizes):
+def _product_kinds(T, sizes, forward):
     """For each: own, on the library's kernels; eager, there but in a capture; device,
     only in a capture that could not take torch's; torch, never. _OWN: all own."""
     kinds = []
@@ -212,7 +214,8 @@ def _product_kinds(T, sizes):
         nk = n * k
         if n % 4 != 0 or k % 4 != 0 or n > 65536 or k > 65536:
             kinds.append("torch")
-        elif nk <= 2048 or nk <= 1 << 18 and T * T >= 100 * nk:
+        elif (nk <= 2048 or nk <= 1 << 18 and T * T >= 100 * nk
+              or forward and k <= 512 and T * n >= 8192 * k):
             kinds.append("own")
         else:
             kinds.append("eager" if nk <= _OWN_NK and T * nk <= 1 << 30 else "device")
@@ -253,7 +256,7 @@ class _LinearF32(torch.autograd.Function):
     @staticmethod
     def forward(ctx, x, weight, bias):
         ctx.save_for_backward(x, weight, bias)  # as they came: create_graph needs their history
-        own = _own_product(x.numel() // x.shape[-1], *weight.shape)
+        own = _own_product(x.numel() // x.shape[-1], *weight.shape, True)
         return _linear_fwd(own, x.contiguous(), weight.contiguous(), bias.contiguous())
 
     @staticmethod
@@ -332,8 +335,8 @@ def _layer_torch(c, h, w_in, b_in, w_conv, b_conv, w_gate, b_gate, lam, w_out, b
     return nn.functional.linear(y, w_out, b_out)
 
 
-def _layer_products(h, *weights):
-    return _own_products(h.numel() // h.shape[-1], tuple([tuple(w.shape) for w in weights]))
+def _layer_products(h, forward, *weights):
+    return _own_products(h.numel() // h.shape[-1], tuple([tuple(w.shape) for w in weights]), forward)
 
 
 class _LayerF32(torch.autograd.Function):
@@ -343,7 +346,7 @@ class _LayerF32(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, c, h, w_in, b_in, w_conv, b_conv, w_gate, b_gate, lam, w_out, b_out):
-        own = _layer_products(h, w_in, w_gate, w_out)
+        own = _layer_products(h, True, w_in, w_gate, w_out)
         hxz = _linear_fwd(own[0], h.contiguous(), w_in, b_in)
         x, z = _conv_fwd(hxz, w_conv, b_conv)
         gl = _linear_fwd(own[1], x, w_gate, b_gate)
@@ -368,7 +371,7 @@ class _LayerF32(torch.autograd.Function):
                                            (h, w_in, b_in, w_conv, b_conv, w_gate, b_gate, lam,
                                             w_out, b_out), (dout,)))
         dout, h = dout.contiguous(), h.contiguous()
-        own = _layer_products(h, w_in, w_gate, w_out)
+        own = _layer_products(h, False, w_in, w_gate, w_out)
         dy = torch.empty_like(y)
         dw_out, db_out = _linear_bwd(own[2], dout, y, w_out, dy, need[8] or need[9])
         dx, dz, dgl, dlam = (torch.empty_like(t) for t in (x, z, gl, lam))

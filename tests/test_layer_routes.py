@@ -109,7 +109,7 @@ def kernels_on_cpu(monkeypatch):
     monkeypatch.setattr(layer_module, "blr_scan_bwd_gated", scan_bwd)
     monkeypatch.setattr(layer_module, "blr_workspace_bytes", lambda d: 64)
     monkeypatch.setattr(layer_module, "_dtype_code", lambda t: 0)
-    monkeypatch.setattr(layer_module, "_own_products", lambda T, sizes: (True,) * len(sizes))
+    monkeypatch.setattr(layer_module, "_own_products", lambda T, sizes, forward: (True,) * len(sizes))
     kernels = dict(definition=definition)
     monkeypatch.setattr(layer_module, "blr_linear_fwd", linear_fwd)
     monkeypatch.setattr(layer_module, "blr_conv_silu_fwd", conv_fwd)
@@ -215,6 +215,8 @@ def test_rule_for_a_projection(device_state):
     assert all(own(*s) for s in always) and not any(own(*s) for s in eager + never)
     assert state["handles"] == 1
     assert not own(50, 65540, 4) and not own(50, 6, 4)  # the kernels refuse them
+    assert own(51200, 2048, 512, True) and not own(51200, 2048, 512, False)
+    assert not own(1600, 1024, 512, True) and not own(51200, 2048, 1024, True)
 
 
 @pytest.mark.parametrize("n,k,kernel", [(65536, 4, True), (65540, 4, False), (4, 65540, False),
