@@ -611,7 +611,8 @@ blr_status scan_bwd_entry(const blr_desc* desc, const void* dh, const float* dh_
   BLR_TRY(check_ws(plan, ws, ws_bytes));
 
   unsigned char* w = static_cast<unsigned char*>(ws);
-  if (plan.seq)  // the forward cleared the counters and partial sums
+  // the forward cleared the counters and partial sums
+  if (plan.seq || (plan.seq_bwd && !varlen))
     return scan_bwd_seq(plan, dh, dh_last, x, gate_logits, lambda, h0, dx, dgate_logits, dlambda,
                         dh0, w, st, z, dz, lengths);
   return scan_bwd_team(plan, dh, dh_last, x, gate_logits, lambda, h0, dx, dgate_logits, dlambda,

@@ -65,6 +65,16 @@ constexpr int64_t kSeqTallRowsMinL = 1024;
 // above. Measured on GB300 (fwd + bwd, us, serial / team kernels): 600 chains x
 // 800 steps 119 / 124, x 3000 399 / 431, 400 x 3000 320 / 297, 512 x 2048 251 / 274.
 constexpr int64_t kSeqMinChainsF32 = 512;
+// The plain and gated backward from fewer on, on the states a team forward kept
+// (they lie the same way): the team backward takes two rounds of whole chains from
+// 305 to 608 of them however many, a serial one grows by the chain (backward, us,
+// serial / team, L = 50, 150, 400, 2000: 352 chains 9.7 / 11.0, 17.4 / 20.9, 31.2 /
+// 29.7, 126 / 119; 400 9.9 / 10.8, 17.0 / 20.5, 31.8 / 38.2, 130 / 134; 456 9.6 / 11.3,
+// 17.7 / 20.9, 32.7 / 39.1, 136 / 154; 511 9.9 / 12.5, 18.0 / 23.2, 33.2 / 42.1, 148 /
+// 171; the forward at 456 7.6 / 7.6, 9.2 / 10.1, 19.6 / 17.6, 81 / 82). Rows with
+// lengths share the teams' work better and stay with them (fwd + bwd 456 x 400
+// 51.2 / 47.8, x 2000 206 / 158).
+constexpr int64_t kSeqMinChainsBwdF32 = 400;
 
 // Team kernels: kTeamWarps compute warps a block, in teams of kTeamWidth;
 // a warp takes kTeamSlice steps of a tile. The plan (and with it the workspace)
@@ -127,6 +137,7 @@ struct Plan {
   int io;           // 0 = float32, 1 = bfloat16
   float c;
   int seq;          // 1: serial kernels, 0: team kernels
+  int seq_bwd;      // 1: the serial backward all the same, without lengths
   int sv;           // channels per lane (a chain is a row segment of 32 * sv channels)
   int rb;           // steps between the forward's kept states
   int sr, srb;      // serial: rows per TMA box, forward and backward (multiples of rb)
@@ -191,6 +202,7 @@ inline void make_plan(int64_t B, int64_t L, int64_t D, int io, float c, bool loc
   p->sv = io == 0 ? 1 : 2;
   p->n_chain = B * ((D + 32 * p->sv - 1) / (32 * p->sv));
   p->seq = io == 0 ? p->n_chain >= kSeqMinChainsF32 : plan_seq_bf16(p->n_chain, L);
+  p->seq_bwd = p->seq || (io == 0 && p->n_chain >= kSeqMinChainsBwdF32);
   p->segmented = p->n_chain < kManyChains && io == 1 && L >= kSegMinL &&
                  (B * L * D >= kSegMinElems || L >= kSegLongL);
   // Long float32 sequences stream the serial forward in 32-row boxes (fewer,

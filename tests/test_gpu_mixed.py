@@ -1,0 +1,28 @@
+"""GPU: float32 scans whose forward runs on the team kernels and whose backward on the
+serial ones (400 to 511 chains), against the oracle: a step, a slice and its edges,
+tiles in the local order and with the look-back, channel tails."""
+import pytest
+
+from gpu_common import TOL, compare, gpu_outputs, gpu_scan, gpu_scan_gated, normwise, oracle_outputs
+from paper_2406_12580_gb300 import inputs as I
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+
+@pytest.mark.parametrize("gated", [False, True])
+@pytest.mark.parametrize("B,L,D", [(400, 1, 32), (511, 16, 8), (200, 17, 64), (400, 129, 24),
+                                   (137, 300, 72), (450, 700, 32)])
+def test_team_forward_serial_backward(B, L, D, gated):
+    cfg = I.ScanConfig("mixed", io=I.F32, seed=B + L, gated=gated, B=B, L=L, D=D, random_h0=True,
+                       random_dh_last=True)
+    inp = I.make_scan_inputs(cfg)
+    buf, want = (gpu_scan_gated if gated else gpu_scan)(inp), oracle_outputs(inp)
+    compare(inp, gpu_outputs(buf), want)
+    (buf.bwd_gated if gated else buf.bwd)()  # again on the same workspace
+    torch.cuda.synchronize()
+    for k, v in gpu_outputs(buf).items():
+        assert normwise(v, want[k]) <= TOL[I.F32], k
