@@ -752,6 +752,13 @@ blr_status blr_steps(int64_t B, int64_t K, int64_t D, blr_dtype io, blr_dtype st
   BLR_TRY(need(x, "x", 16));
   BLR_TRY(need(gate_logits, "gate_logits", 16));
   BLR_TRY(optional(h_seq, "h_seq", 16));
+  using bf = __nv_bfloat16;
+  const int64_t row_blocks = (B * (D / 4) + 255) / 256;
+  if (io == BLR_F32 && K >= blr::kStepsRowK && row_blocks < ((int64_t)1 << 31)) {
+    const blr::StepsArgs a{B, K, D, c, 0, h_prev, x, gate_logits, lambda, h_out, h_seq};
+    return launch_overlapped(state == BLR_F32 ? blr::steps_row_kernel<float> : blr::steps_row_kernel<bf>,
+                             (unsigned)row_blocks, dim3(256), 0, st, a, "launch steps_row_kernel");
+  }
   const int vec = io == BLR_F32 ? 4 : 8;
   const int64_t nvec = D / vec;
   const int bx = (int)(nvec < 64 ? nvec : 64);
@@ -759,12 +766,12 @@ blr_status blr_steps(int64_t B, int64_t K, int64_t D, blr_dtype io, blr_dtype st
   const int64_t n_vgroups = (nvec + bx - 1) / bx;
   // a persistent grid, at most one row group per block row of work
   const int64_t need_rg = (B + by - 1) / by;
-  int64_t n_rg = ((int64_t)sm_count() * blr::kStepsBlocksPerSm + n_vgroups - 1) / n_vgroups;
+  const int per_sm = io == BLR_F32 ? blr::steps_blocks_per_sm<float>() : blr::steps_blocks_per_sm<bf>();
+  int64_t n_rg = ((int64_t)sm_count() * per_sm + n_vgroups - 1) / n_vgroups;
   if (n_rg > need_rg) n_rg = need_rg;
   if (n_rg < 1) n_rg = 1;
   if (n_vgroups * n_rg >= ((int64_t)1 << 31)) return fail(BLR_ERR_UNSUPPORTED, "grid too large");
   blr::StepsArgs a{B, K, D, c, n_vgroups, h_prev, x, gate_logits, lambda, h_out, h_seq};
-  using bf = __nv_bfloat16;
   const unsigned grid = (unsigned)(n_vgroups * n_rg);
   const dim3 block((unsigned)bx, (unsigned)by);
   auto launch = [&](auto kernel) { return launch_overlapped(kernel, grid, block, 0, st, a, "launch steps_kernel"); };

@@ -123,13 +123,16 @@ __global__ void __launch_bounds__(256, kStepBlocksPerSm) step_kernel(const StepA
 // in memory (a bfloat16 state is rounded once, when it is stored).
 //
 // A persistent grid (as the single step's): a thread goes on to its next row
-// without a gap. Its inputs come through kStepsAhead register sets, each
+// without a gap. Its inputs come through steps_ahead register sets, each
 // refilled as soon as its step is done, across the ends of rows, so that loads
 // are always in flight; the next row's state is requested a row ahead. The
 // arithmetic runs on pairs of channels, and k is computed once a block.
 // 65536 x 8 x 64 bfloat16 with all states written: 47.6 us (0.88 of the
 // measured copy rate); one row a thread, its loads in batches of four steps and
 // the arithmetic unpaired took 55.7.
+// float32, whose loads are half as many values each, wants more threads and fewer
+// sets: 3 blocks an SM and 2 sets against 2 and 4, 65536 x 2 x 64 20.2 against 24.3
+// us, x 4 44.3 / 48.6. From kStepsRowK steps on it runs steps_row_kernel.
 
 struct StepsArgs {
   int64_t B, K, D;
@@ -143,8 +146,10 @@ struct StepsArgs {
   void* h_seq;         // (B, K, D), io dtype, or NULL
 };
 
-constexpr int kStepsAhead = 4;
-constexpr int kStepsBlocksPerSm = 2;
+template <typename T>
+__host__ __device__ constexpr int steps_ahead() { return sizeof(T) == 4 ? 2 : 4; }
+template <typename T>
+__host__ __device__ constexpr int steps_blocks_per_sm() { return sizeof(T) == 4 ? 3 : 2; }
 
 // One step of a pair of channels from its raw inputs (a bfloat16 word, halved
 // on the packed pair, or two floats): h <- alpha h + sqrt(1 - alpha^2) i x.
@@ -197,7 +202,7 @@ __device__ __forceinline__ void steps_walk(const StepsArgs& a, const float2 (&kp
                                            int64_t r, int64_t rstride) {
   using IO = Io<T, VEC>;
   using Raw = typename IO::Raw;
-  constexpr int A = kStepsAhead, P = VEC / 2;
+  constexpr int A = steps_ahead<T>(), P = VEC / 2;
   if (r >= a.B) return;
   // where the next inputs are: row lr, step lj
   int64_t lr = r, lj = 0;
@@ -261,7 +266,7 @@ __device__ __forceinline__ void steps_walk(const StepsArgs& a, const float2 (&kp
 }
 
 template <typename T, typename S, int VEC>
-__global__ void __launch_bounds__(256, kStepsBlocksPerSm) steps_kernel(const StepsArgs a) {
+__global__ void __launch_bounds__(256, steps_blocks_per_sm<T>()) steps_kernel(const StepsArgs a) {
   __shared__ float s_k[64 * 8];
   pdl_wait();
   pdl_release();
@@ -289,6 +294,65 @@ __global__ void __launch_bounds__(256, kStepsBlocksPerSm) steps_kernel(const Ste
     steps_walk<T, S, VEC, true>(a, kp, d0, r, rstride);
   else
     steps_walk<T, S, VEC, false>(a, kp, d0, r, rstride);
+}
+
+// float32 with kStepsRowK steps or more: one row a thread, its inputs in batches of
+// kStepsRowBatch steps, whose gates are independent work. With rows this long a
+// thread needs no next one, and with few rows the gates' latency binds, which the
+// walk above takes step by step (us, walk / rows: 65536 x 8 x 64 85.3 / 83.0, 0.99 of
+// the measured copy rate, x 12 126.9 / 123.6, 1000 x 50 x 64 23.1 / 18.0, 100000 x 12 x
+// 16 53.9 / 52.0; but 20000 x 8 x 64 22.5 / 24.7, 65536 x 4 x 64 44.3 / 45.9, x 2
+// 20.2 / 32.1).
+constexpr int64_t kStepsRowK = 8;
+constexpr int kStepsRowBatch = 4;
+
+template <typename S>
+__global__ void __launch_bounds__(256) steps_row_kernel(const StepsArgs a) {
+  using IO = Io<float, 4>;
+  using M = MathPrecise;
+  constexpr int A = kStepsRowBatch;
+  pdl_wait();
+  pdl_release();
+  const int64_t nv = a.D / 4;
+  const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (idx >= a.B * nv) return;
+  const int64_t b = idx / nv, d0 = (idx - b * nv) * 4;
+  float k[4], h[4];
+#pragma unroll
+  for (int v = 0; v < 4; ++v) k[v] = decay_rate(a.c, a.lambda[d0 + v]);
+  load_state<S, 4>(static_cast<const S*>(a.h_prev) + b * a.D + d0, h);
+  const float* x = static_cast<const float*>(a.x) + b * a.K * a.D + d0;
+  const float* gl = static_cast<const float*>(a.gl) + b * a.K * 2 * a.D + d0;
+  float* hs = a.h_seq != nullptr ? static_cast<float*>(a.h_seq) + b * a.K * a.D + d0 : nullptr;
+  for (int64_t j0 = 0; j0 < a.K; j0 += A) {
+    float4 rx[A], rr[A], ri[A];
+#pragma unroll
+    for (int u = 0; u < A; ++u) {
+      const int64_t j = j0 + u;
+      if (j < a.K) {
+        rx[u] = IO::load_raw(x + j * a.D);
+        rr[u] = IO::load_raw(gl + j * 2 * a.D);
+        ri[u] = IO::load_raw(gl + j * 2 * a.D + a.D);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < A; ++u) {
+      const int64_t j = j0 + u;
+      if (j < a.K) {
+        float xv[4], rv[4], iv[4];
+        IO::unpack(rx[u], xv);
+        IO::unpack(rr[u], rv);
+        IO::unpack(ri[u], iv);
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+          const float e = M::expm1_any(k[v] * M::sigmoid(rv[v]));
+          h[v] = fmaf(1.0f + e, h[v], M::sqrt(-e * (2.0f + e)) * M::sigmoid(iv[v]) * xv[v]);
+        }
+        if (hs != nullptr) IO::store(hs + j * a.D, h);
+      }
+    }
+  }
+  store_state<S, 4>(static_cast<S*>(a.h_out) + b * a.D + d0, h);
 }
 
 // ------------------------------------------------------------ bounded-wait test
