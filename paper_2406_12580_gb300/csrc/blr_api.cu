@@ -438,11 +438,7 @@ blr_status launch_team(K kernel, size_t smem, A& args, cudaStream_t st, const ch
   const int64_t units = p.lookback ? p.n_tc * p.n_chain : p.n_chain;
   unsigned grid = 1;
   BLR_TRY(persistent_grid(kernel, threads, smem, (units + blr::kTeams - 1) / blr::kTeams, &grid));
-  // A multiple of the channel groups, if that idles few teams: a team then
-  // stays within one group, and the backward adds its d Lambda sums up once.
-  args.teams = grid * (unsigned)blr::kTeams;
-  const int64_t n_g = p.n_chain / p.B;
-  if (args.teams >= 8 * n_g) args.teams -= args.teams % (unsigned)n_g;
+  args.teams = blr::plan_teams(p, grid * (unsigned)blr::kTeams);
   if (!p.lookback) return launch_overlapped(kernel, grid, dim3((unsigned)threads), smem, st, args, what);
   if (fill)
     BLR_TRY(cuda_check(cudaMemsetAsync(args.ws + p.off_cinc, 0xff, p.rec_set, st),

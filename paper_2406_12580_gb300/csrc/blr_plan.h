@@ -239,4 +239,15 @@ inline void make_plan(int64_t B, int64_t L, int64_t D, int io, float c, bool loc
   p->bytes = o + p->rec_set;
 }
 
+// The teams that work, of `teams` launched: a multiple of the channel groups, if
+// that idles few of them (a team then stays within one group, and the backward adds
+// its d Lambda sums up once) and gives the busiest no further chain to walk.
+inline uint32_t plan_teams(const Plan& p, uint32_t teams) {
+  const int64_t n_g = p.n_chain / p.B;
+  if (teams < 8 * n_g) return teams;
+  const uint32_t whole = teams - teams % (uint32_t)n_g;
+  const bool longer = (p.n_chain + whole - 1) / whole > (p.n_chain + teams - 1) / teams;
+  return !p.lookback && longer ? teams : whole;
+}
+
 }  // namespace blr
