@@ -151,16 +151,16 @@ __host__ __device__ constexpr int steps_ahead() { return sizeof(T) == 4 ? 2 : 4;
 template <typename T>
 __host__ __device__ constexpr int steps_blocks_per_sm() { return sizeof(T) == 4 ? 3 : 2; }
 
-// One step of a pair of channels from its raw inputs (a bfloat16 word, halved
-// on the packed pair, or two floats): h <- alpha h + sqrt(1 - alpha^2) i x.
+// One step of a pair of channels from its raw inputs (a bfloat16 word, its logits
+// halved on the packed pair, or two floats): h <- alpha h + sqrt(1 - alpha^2) i x.
 // kp: k/2 of the channels for bfloat16, k for float32.
 template <bool POLY>
 __device__ __forceinline__ void step_pair(uint32_t x, uint32_t r, uint32_t i, float2 kp, float2& h) {
-  const float2 hx = bf2_scaled(x, kBf2Half);
   const float2 e = expm1_neg2<POLY>(__ffma2_rn(kp, tanh2(bf2_scaled(r, kBf2Half)), kp));
   const float2 m2 = __fmul2_rn(e, __fadd2_rn(e, f2(2.0f)));  // -(1 - alpha^2)
-  const float2 u = __fmul2_rn(make_float2(sqrt_approx(-m2.x), sqrt_approx(-m2.y)),
-                              __ffma2_rn(hx, tanh2(bf2_scaled(i, kBf2Half)), hx));
+  // i and x apart ((x/2) tanh(iota/2) + x/2 is nan at an infinite x)
+  const float2 si = __ffma2_rn(f2(0.5f), tanh2(bf2_scaled(i, kBf2Half)), f2(0.5f));
+  const float2 u = __fmul2_rn(make_float2(sqrt_approx(-m2.x), sqrt_approx(-m2.y)), __fmul2_rn(si, bf2_unpack(x)));
   h = __ffma2_rn(__fadd2_rn(f2(1.0f), e), h, u);
 }
 template <bool POLY>

@@ -67,3 +67,32 @@ def test_infinite_adjoints(B, L, D, gated, io):
     # the gates' gradients: infinite in the same places (a sign is that of a difference)
     assert np.array_equal(np.isfinite(got["dgl"]), np.isfinite(want["dgl"]))
     assert np.array_equal(np.isfinite(got["dlam"]), np.isfinite(want["dlam"]))
+
+
+@pytest.mark.parametrize("io", [0, 1])
+@pytest.mark.parametrize("K", [1, 3, 9])
+def test_infinite_steps(K, io):
+    """blr_steps and blr_step on infinite inputs and states, gates open and nearly closed."""
+    from paper_2406_12580_gb300 import blr_step, blr_steps
+    B, D = 5, 24
+    g = torch.Generator(device="cuda").manual_seed(K)
+    rand = lambda *s: torch.randn(*s, device="cuda", generator=g)  # noqa: E731
+    dtype = (torch.float32, torch.bfloat16)[io]
+    h, x, gl, lam = rand(B, D), rand(B, K, D), rand(B, K, 2 * D), rand(D) - 3.0
+    x[0, 0, 0], x[1, K - 1, 1], x[2, 0, 2], h[3, 3], h[4, 4] = np.inf, -np.inf, np.inf, np.inf, -np.inf
+    gl[0, 0, D], gl[1, K - 1, D + 1], gl[2, 0, D + 2] = -2.0, -1.0, 3.0
+    x, gl = x.to(dtype), gl.to(dtype)
+    ref, want = h.double(), []
+    r, i = torch.sigmoid(gl.double()).chunk(2, dim=-1)
+    log_a = -torch.nn.functional.softplus(lam.double()) * r
+    for k in range(K):
+        ref = torch.exp(log_a[:, k]) * ref + torch.sqrt(-torch.expm1(2 * log_a[:, k])) * i[:, k] * x[:, k].double()
+        want.append(ref)
+    out, seq = torch.empty_like(h), torch.empty_like(x)
+    blr_steps(B, K, D, io, 0, 1.0, h, x, gl, lam, out, seq)
+    tol = TOL[I.BF16 if io else I.F32]
+    same(out.double().cpu().numpy(), ref.cpu().numpy(), tol, "h")
+    same(seq.double().cpu().numpy(), torch.stack(want, 1).cpu().numpy(), tol, "h_seq")
+    if K == 1:
+        blr_step(B, D, io, 1.0, h, x[:, 0].contiguous(), gl[:, 0].contiguous(), lam, out)
+        same(out.double().cpu().numpy(), ref.cpu().numpy(), tol, "step")
