@@ -116,14 +116,19 @@ inline bool plan_narrow(int64_t wide, int64_t narrow, int64_t most = kSeqMaxNarr
 inline bool plan_narrow_bwd(int64_t wide, int64_t narrow, int64_t L) {
   return plan_narrow(wide, narrow, L <= kSeqNarrowBwdL ? kSeqMaxNarrowBwd : kSeqMaxNarrow);
 }
-// With the merge, whose work a lane of one channel spreads over more warps, the
-// forward is narrow again for many short chains, and for longer ones where a
-// sixth or more of the wide lanes lie past D (fwd + bwd, us, wide / narrow forward:
-// 2048 x 50 x 64 47.5 / 45.0, x 100 76.4 / 74.7, 3000 x 50 73.0 / 72.2, 8000 x 50
-// 142.8 / 141.3, 700 x 200 x 160 137.6 / 122.9, 3000 x 50 x 160 144.2 / 140.2; but
-// 3000 x 160 x 64 171 / 177, 1500 x 200 99 / 101, 2100 x 800 x 160 1337 / 1347).
+// With the merge the wide forward's rings fit 13 blocks an SM. Where there are more
+// chains than that, some wait for a place, and the narrow form, two blocks of half
+// the size, is faster again for short ones (fwd + bwd, us, wide / narrow forward, L =
+// 50: 913 x 64 27.6 / 27.7, 1400 36.0 / 36.0, 1600 37.6 / 37.4, 1824 39.9 / 41.2, 1950
+// 41.5 / 44.1, 2000 46.8 / 44.8, 2048 47.1 / 44.8, 2600 62.9 / 61.7, 3500 77.1 / 76.0,
+// 8000 142.8 / 141.3; x 100 1950 70.1 / 73.4, 2048 76.4 / 73.8; but 3000 x 160 171 /
+// 177, 1500 x 200 99 / 101). For longer ones it is where a sixth or more of the wide
+// lanes lie past D (700 x 200 x 160 137.6 / 122.9, 3000 x 50 x 160 144.2 / 140.2; but
+// 2100 x 800 x 160 1337 / 1347).
+constexpr int64_t kSeqWideMergeMost = 13 * 152;
 inline bool plan_narrow_merge(int64_t wide, int64_t narrow, int64_t L) {
-  return wide >= kSeqMaxNarrow && (L <= 100 || (L <= 256 && 3 * narrow <= 5 * wide));
+  return (wide > kSeqWideMergeMost && L <= 100) ||
+         (wide >= kSeqMaxNarrow && L <= 256 && 3 * narrow <= 5 * wide);
 }
 
 // The look-back reads this many predecessors a round trip; kFarWindow where the

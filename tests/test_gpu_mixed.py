@@ -1,4 +1,4 @@
-"""GPU: float32 scans whose forward runs on the team kernels and whose backward on the
+"""GPU: scans whose forward and backward run in different forms. float32 ones whose forward runs on the team kernels and whose backward on the
 serial ones (400 to 511 chains), against the oracle: a step, a slice and its edges,
 tiles in the local order and with the look-back, channel tails."""
 import pytest
@@ -26,3 +26,11 @@ def test_team_forward_serial_backward(B, L, D, gated):
     torch.cuda.synchronize()
     for k, v in gpu_outputs(buf).items():
         assert normwise(v, want[k]) <= TOL[I.F32], k
+
+
+@pytest.mark.parametrize("B,L", [(1976, 23), (1977, 23), (1977, 100), (1977, 101)])
+def test_bf16_merge_by_chains(B, L):
+    """bfloat16 with the merge at the line between the wide and the narrow forward."""
+    cfg = I.ScanConfig("merge", io=I.BF16, seed=B + L, gated=True, B=B, L=L, D=64, random_h0=True)
+    inp = I.make_scan_inputs(cfg)
+    compare(inp, gpu_outputs(gpu_scan_gated(inp)), oracle_outputs(inp))
