@@ -45,7 +45,7 @@ class BDLRUGatedScan(torch.autograd.Function):
                              z.contiguous(), h0, c)
 
     @staticmethod
-    def forward(ctx, x, gate_logits, lam, z, h0, c):
+    def forward(ctx, x, gate_logits, lam, z, h0=None, c: float = 1.0):
         B, L, D = x.shape
         for name, t, n in (("gate_logits", gate_logits, 2 * B * L * D), ("lam", lam, D),
                            ("z", z, B * L * D), ("h0", h0, B * D)):
@@ -62,11 +62,12 @@ class BDLRUGatedScan(torch.autograd.Function):
 
     @staticmethod
     def backward(ctx, dy, dh_last):
-        x = ctx.saved_tensors[0]
+        saved = ctx.saved_tensors
+        x = saved[0]
         dy = torch.zeros_like(x) if dy is None else dy.contiguous().to(x.dtype)
         dh_last = None if dh_last is None else dh_last.contiguous().float()
         grad = _GatedScanGrad.apply if torch.is_grad_enabled() else _gated_scan_bwd
-        return (*grad(dy, dh_last, *ctx.saved_tensors, ctx.desc), None)
+        return (*grad(dy, dh_last, *saved, ctx.desc), None)
 
 
 def _gated_scan_bwd(dy, dh_last, x, gate_logits, lam, z, h0, ws, desc):

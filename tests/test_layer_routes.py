@@ -260,3 +260,15 @@ def test_parameters_of_other_sizes_never_reach_the_kernels(monkeypatch, name, sh
         lin = getattr(layer, module)
         with pytest.raises(RuntimeError):
             lin(torch.randn(3, 16 if module != "in_proj" else 8))
+
+
+def test_saved_tensors_are_unpacked_once(kernels_on_cpu):
+    """Hooks that bring a saved tensor back (from another memory, say) run once a backward."""
+    rand = lambda *s: torch.randn(*s, requires_grad=True)  # noqa: E731
+    packed, unpacked = [], []
+    with torch.autograd.graph.saved_tensors_hooks(lambda t: packed.append(t.shape) or t,
+                                                  lambda t: unpacked.append(t.shape) or t):
+        y, _ = layer_module.BDLRUGatedScan.apply(rand(2, 3, 8), rand(2, 3, 16), rand(8), rand(2, 3, 8),
+                                                 rand(2, 8))
+    y.backward(torch.ones_like(y))
+    assert len(packed) == len(unpacked) == 6
