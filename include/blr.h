@@ -115,16 +115,18 @@ BLR_API size_t blr_workspace_bytes(const blr_desc* desc);
  *                         lengths: the backward of a plain or gated forward
  *                         refuses the workspace of a _varlen forward here, and
  *                         the reverse.
- *   BLR_FAMILY_TILED      otherwise.
+ *   BLR_FAMILY_TILED      otherwise. (Here and in SERIAL that misuse is not
+ *                         noticed: the backward's outputs are then undefined.)
  *   BLR_FAMILY_NONE       an invalid or empty problem (nothing is launched).
- * From 512 float32 or 780 bfloat16 chains on (bfloat16 also from 304 where L is
- * at most 5/4 of their number) the serial kernels run: one warp walks each chain
- * (bfloat16: each half of it, where there are few) through the whole sequence.
- * Elsewhere the team kernels: teams
- * of 8 warps scan tiles of up to 128 steps of a chain, 16 steps a warp, whole
+ * The kernels: from 512 float32 or 780 bfloat16 chains on (bfloat16 also from 304
+ * where L is at most 5/4 of their number; a float32 backward without lengths from
+ * 400) the serial ones, in which one warp walks each chain (bfloat16: each half of
+ * it, where there are few) through the whole sequence. Elsewhere the team kernels:
+ * teams of 8 warps scan tiles of up to 128 steps of a chain, 16 steps a warp, whole
  * chains at a time where there are enough of them, else tiles of all chains in
- * time order, chained by a decoupled look-back (the operator of Sec. 3.3) after
- * one cudaMemsetAsync that empties its records. Every call is one kernel.
+ * time order, chained by a decoupled look-back (the operator of Sec. 3.3); a
+ * forward then empties its records by one cudaMemsetAsync first. Every call is one
+ * kernel.
  */
 #define BLR_FAMILY_NONE 0
 #define BLR_FAMILY_TILED 1
@@ -224,8 +226,9 @@ BLR_API blr_status blr_scan_bwd_varlen(const blr_desc* desc, const int32_t* leng
  * z           (B, L, D)  io dtype, the second branch's input (H_z)
  * y           (B, L, D)  io dtype, output; may be NULL (then only h_last and
  *                        the carries, as blr_scan_fwd with h == NULL)
- * Other arguments, the workspace and the errors as blr_scan_fwd; z must be
- * 16-byte aligned and no output may overlap an input.
+ * y is rounded once, from the float32 state. Other arguments, the workspace and
+ * the errors as blr_scan_fwd; z must be 16-byte aligned and no output may overlap
+ * an input.
  */
 BLR_API blr_status blr_scan_fwd_gated(const blr_desc* desc, const void* x, const void* gate_logits,
                                       const float* lambda, const float* h0, const void* z, void* y,
@@ -236,7 +239,9 @@ BLR_API blr_status blr_scan_fwd_gated(const blr_desc* desc, const void* x, const
  *   sum_{b,t,d} dy * y + sum_{b,d} dh_last * h_last:
  * the scan's backward (outputs as blr_scan_bwd) for dh = dy * SiLU(z), and
  *   dz = dy * h * SiLU'(z),   SiLU'(z) = sigmoid(z) (1 + z (1 - sigmoid(z))),
- * with h recomputed, not read.
+ * with h recomputed, not read, and dz rounded once from the float32 h. bfloat16
+ * problems of the shape class TILED round dh to bfloat16 before the scan (2^-9 of
+ * each dh in dx, dgate_logits, dlambda and dh0); the others keep it in float32.
  * dy          (B, L, D)  io dtype, upstream gradient of y
  * z           (B, L, D)  io dtype, the forward's z
  * dz          (B, L, D)  io dtype, output
