@@ -89,13 +89,6 @@ struct Io<__nv_bfloat16, 4> {  // 8 bytes
   static __device__ __forceinline__ void store(T* p, const float (&v)[4]) {
     __stcs(reinterpret_cast<uint2*>(p), make_uint2(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3])));
   }
-  // v = t / 2, halved on the packed pairs (an exponent decrement).
-  static __device__ __forceinline__ void unpack_half(const Raw& t, float (&v)[4]) {
-    uint32_t a, b;
-    asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(a) : "r"(t.x), "r"(0x3f003f00u));
-    asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(b) : "r"(t.y), "r"(0x3f003f00u));
-    v[0] = bf16_lo(a); v[1] = bf16_hi(a); v[2] = bf16_lo(b); v[3] = bf16_hi(b);
-  }
 };
 
 template <>
@@ -104,25 +97,8 @@ struct Io<float, 1> {  // 4 bytes
   using Raw = float;
   static constexpr int VEC = 1;
   static __device__ __forceinline__ void unpack(const Raw& t, float (&v)[1]) { v[0] = t; }
-  static __device__ __forceinline__ void store(T* p, const float (&v)[1]) { __stcs(p, v[0]); }
   static __device__ __forceinline__ void store_smem(unsigned char* p, const float (&v)[VEC]) {
     *reinterpret_cast<float*>(p) = v[0];
-  }
-};
-
-template <>
-struct Io<float, 2> {  // 8 bytes
-  using T = float;
-  using Raw = float2;
-  static constexpr int VEC = 2;
-  static __device__ __forceinline__ void unpack(const Raw& t, float (&v)[2]) {
-    v[0] = t.x; v[1] = t.y;
-  }
-  static __device__ __forceinline__ void store(T* p, const float (&v)[2]) {
-    __stcs(reinterpret_cast<float2*>(p), make_float2(v[0], v[1]));
-  }
-  static __device__ __forceinline__ void store_smem(unsigned char* p, const float (&v)[VEC]) {
-    *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
   }
 };
 
@@ -133,9 +109,6 @@ struct Io<__nv_bfloat16, 2> {  // 4 bytes
   static constexpr int VEC = 2;
   static __device__ __forceinline__ void unpack(const Raw& t, float (&v)[2]) {
     v[0] = __uint_as_float(t << 16); v[1] = __uint_as_float(t & 0xffff0000u);
-  }
-  static __device__ __forceinline__ void store(T* p, const float (&v)[2]) {
-    __stcs(reinterpret_cast<unsigned int*>(p), pack_bf16x2(v[0], v[1]));
   }
   static __device__ __forceinline__ void store_smem(unsigned char* p, const float (&v)[VEC]) {
     *reinterpret_cast<uint32_t*>(p) = pack_bf16x2(v[0], v[1]);
@@ -232,23 +205,13 @@ __device__ __forceinline__ float rcp_approx(float x) {
   return y;
 }
 
-// sqrt(q) and 1 / sqrt(q) for q >= 0 (0 and 0 at q = 0).
-__device__ __forceinline__ void sqrt_pair(float q, float& n, float& inv_n) {
-  const float rs = rsqrt_approx(q);
-  const bool pos = q > 0.0f;
-  n = pos ? q * rs : 0.0f;
-  inv_n = pos ? rs : 0.0f;
-}
-
 struct MathPrecise {
   static __device__ __forceinline__ float sigmoid(float z) {
     return rcp_approx(1.0f + ex2_approx(-1.4426950408889634f * z));
   }
-  // e^l - 1 for -0.25 < l <= 0: the degree-6 series (truncation below
-  // l^6/7! < 5e-8 relative). Decays usually live there: |l| <= softplus(Lambda)
-  // <= 0.11 for base decays in [0.9, 1).
-  static __device__ __forceinline__ float expm1_poly(float l) { return expm1_taylor<6>(l); }
-  // Any l <= 0: beyond the series' range e^l < 0.78 and e^l - 1 loses
+  // e^l - 1 for l <= 0: above -0.25 the degree-6 series (truncation below
+  // l^6/7! < 5e-8 relative), where decays usually live: |l| <= softplus(Lambda)
+  // <= 0.11 for base decays in [0.9, 1). Beyond, e^l < 0.78 and e^l - 1 loses
   // nothing to cancellation.
   static __device__ __forceinline__ float expm1_any(float l) {
     if (l > -0.25f) return expm1_taylor<6>(l);
@@ -256,15 +219,6 @@ struct MathPrecise {
   }
   // sqrt(q) for q >= 0 (one sqrt.approx; 0 at q = 0, denormals flushed)
   static __device__ __forceinline__ float sqrt(float q) { return sqrt_approx(q); }
-  // beta = sqrt(q) i, u = beta x and c2 = alpha u / q (= alpha i x / n).
-  static __device__ __forceinline__ void norm_terms(float q, float i, float x, float alpha,
-                                                    float& beta, float& u, float& c2) {
-    float n, inv_n;
-    sqrt_pair(q, n, inv_n);
-    beta = n * i;
-    u = beta * x;
-    c2 = alpha * u * (inv_n * inv_n);
-  }
 };
 
 struct MathFast {
@@ -273,20 +227,11 @@ struct MathFast {
   }
   // Degree-4 series for -0.25 < l <= 0 (truncation below l^4/5! < 3.3e-5
   // relative), ex2.approx beyond.
-  static __device__ __forceinline__ float expm1_poly(float l) { return expm1_taylor<4>(l); }
   static __device__ __forceinline__ float expm1_any(float l) {
     if (l > -0.25f) return expm1_taylor<4>(l);
     return ex2_approx(l * 1.4426950408889634f) - 1.0f;
   }
   static __device__ __forceinline__ float sqrt(float q) { return sqrt_approx(q); }
-  static __device__ __forceinline__ void norm_terms(float q, float i, float x, float alpha,
-                                                    float& beta, float& u, float& c2) {
-    float n, inv_n;
-    sqrt_pair(q, n, inv_n);
-    beta = n * i;
-    u = beta * x;
-    c2 = alpha * u * (inv_n * inv_n);
-  }
 };
 
 // ------------------------------------------------- per-element gate terms
@@ -294,7 +239,7 @@ struct MathFast {
 // The serial kernels evaluate the gates of one element with as few
 // instructions as the precision policy allows. With l = k r = log(alpha) and
 // E = e^l - 1 (so alpha = 1 + E and 1 - alpha^2 = -E (2 + E)):
-//   decay_log(rho): l. MathFast folds sigmoid(rho) = (1 + tanh(rho/2)) / 2 into
+//   decay_log(rho), decay_log_half(rho / 2): l. MathFast folds sigmoid(rho) = (1 + tanh(rho/2)) / 2 into
 //     l = kh tanh(rho/2) + kh with kh = k/2 (one multiply-add after tanh).
 //   expm1<POLY>(l): the policy's Taylor series when every l of the channel lies
 //     in (-kExpm1Series, 0] (POLY), else the series or ex2 - 1 beyond it.
@@ -334,9 +279,6 @@ struct GatesFast : MathFast {
   }
   static __device__ __forceinline__ float gated_x_half(float hiota, float hx) {
     return fmaf(hx, tanh_approx(hiota), hx);
-  }
-  static __device__ __forceinline__ float decay_log(float rho, float, float kh) {
-    return fmaf(kh, tanh_approx(0.5f * rho), kh);
   }
   // With hz = z/2 and th = tanh(hz): SiLU = hz (1 + th), sigmoid = (1 + th)/2
   // and z (1 - sigmoid) = hz (1 - th).
@@ -454,10 +396,10 @@ __device__ __forceinline__ void st_record(uint32_t* p, uint32_t v) {
 __device__ __forceinline__ void st_record(unsigned long long* p, unsigned long long v) {
   asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
-// An aggregate (A, U): A in the low word. The tiled kernels store A in [0, 1],
-// the chained forward A - 1 in (-1, 0]: a finite float, never the empty pattern.
-__device__ __forceinline__ unsigned long long pack_agg(float A, float U) {
-  return (unsigned long long)__float_as_uint(A) | ((unsigned long long)__float_as_uint(U) << 32);
+// An aggregate (A - 1, U): A - 1, a float in [-1, 0] or a computed NaN, never the
+// empty pattern, in the low word.
+__device__ __forceinline__ unsigned long long pack_agg(float m, float U) {
+  return (unsigned long long)__float_as_uint(m) | ((unsigned long long)__float_as_uint(U) << 32);
 }
 __device__ __forceinline__ bool agg_empty(unsigned long long v) { return (uint32_t)v == kEmpty; }
 
@@ -510,8 +452,8 @@ __device__ __noinline__ bool wait_word(const uint32_t* flag, uint32_t* err, uint
 // ------------------------------------------------------------- TMA and mbarrier
 //
 // Tiles of the inputs are moved into shared memory by the tensor memory
-// accelerator (cp.async.bulk.tensor, 3-D boxes of 32 channels x tile steps x
-// one batch row) and counted on an mbarrier per pipeline stage.
+// accelerator (cp.async.bulk.tensor, 3-D boxes of a chain's channels x some steps
+// x one batch row) and counted on an mbarrier per pipeline stage.
 
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
@@ -533,19 +475,8 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
 
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-      " selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(smem_addr(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
-// The same test, letting the hardware suspend the thread for up to
-// `hint_ns` while the phase is incomplete (instead of returning at once).
+// Whether the phase of `parity` is complete; the hardware may suspend the thread
+// for up to `hint_ns` while it is not.
 __device__ __forceinline__ bool mbar_try_wait_sleep(uint64_t* bar, uint32_t parity, uint32_t hint_ns) {
   uint32_t ok;
   asm volatile(
@@ -619,8 +550,8 @@ __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wa
 
 // ------------------------------------------------------------ tensor memory
 //
-// The chained forward parks each tile's per-step states in the SM's tensor
-// memory (TMEM, 128 lanes x 512 columns of 32 bits) between its two passes.
+// The team kernels park each slice's per-step states in the SM's tensor memory
+// (TMEM, 128 lanes x 512 columns of 32 bits) between their two passes.
 // A warp reaches only the 32 lanes of its quarter (warp index % 4) and moves
 // 16 consecutive columns of its own lane per thread with one instruction.
 // Addresses: lane in bits 31..16, column in bits 15..0.

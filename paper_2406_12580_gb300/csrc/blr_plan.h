@@ -35,12 +35,10 @@ constexpr uint64_t kWaitTimeoutNs = 1000000000ull;  // 1 s
 constexpr uint32_t kMaxWaitIters = 1u << 23;
 
 struct FwdHeader {     // restarted by every forward
-  uint32_t spare;
-  uint32_t pad0;
   uint32_t err;        // error bits (forward and backward timeouts, workspace misuse)
   uint32_t tag;        // hash of the problem, written by the forward
   uint32_t complete;   // 1 once a forward has run
-  uint32_t pad[3];
+  uint32_t pad[5];
 };
 
 struct BwdHeader {
@@ -102,11 +100,12 @@ inline bool plan_seq_bf16(int64_t wide, int64_t L) {
 // Forward and backward choose by themselves: the states kept between them lie
 // the same way. Both are narrow up to three narrow warps a scheduler (608 of
 // them), the backward of short sequences up to four. Up to there the busiest
-// scheduler has less to walk; beyond, the wide form has the fewer instructions (fwd + bwd, us, wide / narrow: 650 wide chains x 200 steps 57.8 /
-// 52.5, with the merge 74.8 / 61.8; 850 x 200 58.8 / 53.4; forward alone 950 x 200
-// 20.1 / 21.6, x 800 67.9 / 80.3; backward narrow after a wide forward 950 x 50
-// 26.4 / 24.7, 1216 x 50 28.7 / 26.6, with the merge 33.7 / 30.9, 1000 x 200 with
-// lengths 56.0 / 57.1, 950 x 800 202.6 / 205.3, 1500 x 200 80.0 / 92.7). And wherever a third or more of the wide
+// scheduler has less to walk; beyond, the wide form has the fewer instructions
+// (fwd + bwd, us, wide / narrow: 650 wide chains x 200 steps 57.8 / 52.5, with the
+// merge 74.8 / 61.8; 850 x 200 58.8 / 53.4; forward alone 950 x 200 20.1 / 21.6, x 800
+// 67.9 / 80.3; backward narrow after a wide forward 950 x 50 26.4 / 24.7, 1216 x 50
+// 28.7 / 26.6, with the merge 33.7 / 30.9, 1000 x 200 with lengths 56.0 / 57.1, 950 x
+// 800 202.6 / 205.3, 1500 x 200 80.0 / 92.7). And wherever a third or more of the wide
 // lanes lie past D (1000 x 200 x 32 62.4 / 43.9, 4000 x 50 x 32 with the merge
 // 76 / 48, 1500 x 100 x 96 81.3 / 70.6, 3000 x 50 x 96 82.2 / 80.7).
 constexpr int64_t kSeqMaxNarrow = 3 * 608, kSeqMaxNarrowBwd = 4 * 608, kSeqNarrowBwdL = 128;

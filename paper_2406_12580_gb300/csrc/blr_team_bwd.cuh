@@ -9,7 +9,7 @@
 // map w -> A w + W of the w entering its right end, A the product of the run's
 // alphas. The life of a tile in its team:
 //   scanner   announces the tile (its coordinates and decay constants) two
-//             tiles ahead and prefetches its inputs into L2;
+//             tiles ahead;
 //   pass A    every warp evaluates the alphas of its slice and folds the
 //             reverse recurrence from a zero adjoint, last step first (gl_t,
 //             and sm_t = the product of the alphas after step t within the
@@ -175,7 +175,7 @@ __device__ __forceinline__ void team_rfold_f32(const unsigned char* lb, float2 k
 // stage (the TMA store clips rows past the sequence); rows from `rows` on are
 // not summed. Adds the d Lambda terms dl_t r_t to dlr. Gated: dz rows to `dz`,
 // moved on. FAST: the whole slice
-// inside the sequence and every l in the series' range. bfloat16: kq = k/4.
+// inside the sequence and every l in the series' range.
 template <bool FAST, bool GATED, uint32_t BOX>
 __device__ __forceinline__ void team_rows_bf16(unsigned char* lb, const uint32_t (&pr)[16], float2 win,
                                                float2 kh, int rows, float2& hp, float2& dlr,
