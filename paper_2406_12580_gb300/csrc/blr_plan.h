@@ -35,10 +35,11 @@ constexpr uint64_t kWaitTimeoutNs = 1000000000ull;  // 1 s
 constexpr uint32_t kMaxWaitIters = 1u << 23;
 
 struct FwdHeader {     // restarted by every forward
+  uint32_t pad0[2];    // (with err first, the gated bfloat16 team backward spills 28 B instead of 8)
   uint32_t err;        // error bits (forward and backward timeouts, workspace misuse)
   uint32_t tag;        // hash of the problem, written by the forward
   uint32_t complete;   // 1 once a forward has run
-  uint32_t pad[5];
+  uint32_t pad[3];
 };
 
 struct BwdHeader {
