@@ -19,7 +19,7 @@ SHAPES = [(3, 100, 72), (310, 300, 24), (3, 1500, 136), (1, 6000, 8), (520, 60, 
 
 def put(inp, name, at, v):
     getattr(inp, name)[at] = v
-    if inp.cfg.io == I.BF16:  # v: infinite or 1
+    if inp.cfg.io == I.BF16:  # v: not finite, or 1
         inp.bits[name][at] = np.float32(v).view(np.uint32) >> 16
 
 
@@ -67,6 +67,23 @@ def test_infinite_adjoints(B, L, D, gated, io):
     # the gates' gradients: infinite in the same places (a sign is that of a difference)
     assert np.array_equal(np.isfinite(got["dgl"]), np.isfinite(want["dgl"]))
     assert np.array_equal(np.isfinite(got["dlam"]), np.isfinite(want["dlam"]))
+
+
+@pytest.mark.parametrize("io", [I.F32, I.BF16])
+@pytest.mark.parametrize("gated", [False, True])
+@pytest.mark.parametrize("B,L,D", SHAPES)
+def test_nans_stay_in_their_channels(B, L, D, gated, io):
+    """A NaN in x, a logit or dh reaches what depends on it and nothing else."""
+    cfg = I.ScanConfig("nan", io=io, seed=53, gated=gated, B=B, L=L, D=D, random_h0=True)
+    inp = I.make_scan_inputs(cfg)
+    put(inp, "x", (0, L // 2, 0), np.nan)
+    put(inp, "gl", (B - 1, L // 3, 1), np.nan)
+    put(inp, "dh", (B // 2, 2 * L // 3, 2), np.nan)
+    got = gpu_outputs(gpu_scan_gated(inp) if gated else gpu_scan(inp))
+    want = oracle_outputs(inp)
+    for k in ("h", "h_last", "dx", "dgl", "dlam", "dh0") + (("dz",) if gated else ()):
+        assert np.isnan(want[k]).any() or k == "dh0"
+        same(got[k], want[k], TOL[io], k)
 
 
 @pytest.mark.parametrize("io", [0, 1])

@@ -99,3 +99,25 @@ def test_projections_by_either_product(B, L, captured):
     want = torch.autograd.grad(y64, [h64, *m.parameters()], dy.double().cpu())
     for g, w in zip(got, (y64, *want)):
         close(g, w, 5e-5)
+
+
+def test_nans_stay_in_their_rows():
+    """A NaN in one sequence reaches its later steps, and gradients of the weights, but
+    no other sequence (the layer's kernels, at tails of their tiles)."""
+    from paper_2406_12580_gb300.layer import GatedRecurrentLayer
+    torch.manual_seed(14)
+    layer = GatedRecurrentLayer(12, device="cuda")
+    h = torch.randn(5, 37, 12, device="cuda")
+    h[2, 20, 3] = float("nan")
+    h.requires_grad_()
+    dy = torch.randn(5, 37, 12, device="cuda")
+    y = layer(h)
+    assert "LayerF32" in type(y.grad_fn).__name__
+    dh, dw = torch.autograd.grad(y, [h, layer.in_proj.weight], dy)
+    m, h64, y64 = float64(layer, h)
+    dh64, dw64 = torch.autograd.grad(y64, [h64, m.in_proj.weight], dy.double().cpu())
+    for got, want in ((y, y64), (dh, dh64), (dw, dw64)):
+        nan = torch.isnan(want)
+        assert nan.any() and torch.equal(torch.isnan(got).cpu(), nan)
+        if not nan.all():
+            close(got.detach()[~nan.cuda()], want[~nan], 5e-5)
