@@ -299,8 +299,8 @@ __global__ void __launch_bounds__(256, steps_blocks_per_sm<T>()) steps_kernel(co
 // float32 with kStepsRowK steps or more: one row a thread, its inputs in batches of
 // kStepsRowBatch steps, whose gates are independent work. With rows this long a
 // thread needs no next one, and with few rows the gates' latency binds, which the
-// walk above takes step by step (us, walk / rows: 65536 x 8 x 64 85.3 / 83.0, 0.99 of
-// the measured copy rate, x 12 126.9 / 123.6, 1000 x 50 x 64 23.1 / 18.0, 100000 x 12 x
+// walk above takes step by step (us, walk / rows: 65536 x 8 x 64 85.3 / 83.0, the
+// measured copy rate, x 12 126.9 / 123.6, 1000 x 50 x 64 23.1 / 18.0, 100000 x 12 x
 // 16 53.9 / 52.0; but 20000 x 8 x 64 22.5 / 24.7, 65536 x 4 x 64 44.3 / 45.9, x 2
 // 20.2 / 32.1).
 constexpr int64_t kStepsRowK = 8;
