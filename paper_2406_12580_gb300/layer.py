@@ -336,10 +336,6 @@ def _layer_torch(c, h, w_in, b_in, w_conv, b_conv, w_gate, b_gate, lam, w_out, b
     return nn.functional.linear(y, w_out, b_out)
 
 
-def _layer_products(h, forward, *weights):
-    return _own_products(h.numel() // h.shape[-1], tuple([tuple(w.shape) for w in weights]), forward)
-
-
 class _LayerF32(torch.autograd.Function):
     """The whole layer in float32 on the library's kernels: one node in the graph
     instead of five, and the gate projection's gradient of the scan's input added
@@ -347,11 +343,13 @@ class _LayerF32(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, c, h, w_in, b_in, w_conv, b_conv, w_gate, b_gate, lam, w_out, b_out):
-        own = _layer_products(h, True, w_in, w_gate, w_out)
+        B, L, d = h.shape
+        n, D = w_out.shape
+        ctx.products = products = (B * L, ((2 * D, d), (2 * D, D), (n, D)))
+        own = _own_products(*products, True)
         hxz = _linear_fwd(own[0], h.contiguous(), w_in, b_in)
         x, z = _conv_fwd(hxz, w_conv, b_conv)
         gl = _linear_fwd(own[1], x, w_gate, b_gate)
-        B, L, D = x.shape
         desc = Desc(B, L, D, 0, c)
         ws = torch.empty(blr_workspace_bytes(desc), dtype=torch.uint8, device=x.device)
         y = torch.empty_like(x)
@@ -372,7 +370,7 @@ class _LayerF32(torch.autograd.Function):
                                            (h, w_in, b_in, w_conv, b_conv, w_gate, b_gate, lam,
                                             w_out, b_out), (dout,)))
         dout, h = dout.contiguous(), h.contiguous()
-        own = _layer_products(h, False, w_in, w_gate, w_out)
+        own = _own_products(*ctx.products)
         dy = torch.empty_like(y)
         dw_out, db_out = _linear_bwd(own[2], dout, y, w_out, dy, need[8] or need[9])
         dx, dz, dgl, dlam = (torch.empty_like(t) for t in (x, z, gl, lam))
