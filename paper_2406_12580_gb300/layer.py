@@ -38,12 +38,6 @@ class BDLRUGatedScan(torch.autograd.Function):
     float32 or bfloat16; lam (D,) and h0 (B, D) or None in float32. Returns
     (y, h_last)."""
 
-    @classmethod
-    def apply(cls, x, gate_logits, lam, z, h0=None, c: float = 1.0):
-        # laid out for the kernels in autograd's sight: create_graph needs the inputs' history
-        return super().apply(x.contiguous(), gate_logits.contiguous(), lam.contiguous().float(),
-                             z.contiguous(), h0, c)
-
     @staticmethod
     def forward(ctx, x, gate_logits, lam, z, h0=None, c: float = 1.0):
         B, L, D = x.shape
@@ -53,21 +47,25 @@ class BDLRUGatedScan(torch.autograd.Function):
                 raise ValueError(f"{name}: fewer values ({t.numel()}) than the scan reads ({n})")
         desc = Desc(B, L, D, _dtype_code(x), c)
         ws = torch.empty(max(blr_workspace_bytes(desc), 16), dtype=torch.uint8, device=x.device)
-        y = torch.empty_like(x)
-        h_last = torch.empty(B, D, dtype=torch.float32, device=x.device)
-        blr_scan_fwd_gated(desc, x, gate_logits, lam, h0, z, y, h_last, ws)
+        # as they came: create_graph needs their history
         ctx.save_for_backward(x, gate_logits, lam, z, h0, ws)
         ctx.desc = desc
+        x = x.contiguous()
+        y = torch.empty_like(x)
+        h_last = torch.empty(B, D, dtype=torch.float32, device=x.device)
+        blr_scan_fwd_gated(desc, x, gate_logits.contiguous(), lam.contiguous().float(), h0,
+                           z.contiguous(), y, h_last, ws)
         return y, h_last
 
     @staticmethod
     def backward(ctx, dy, dh_last):
-        saved = ctx.saved_tensors
-        x = saved[0]
+        x, gate_logits, lam, z, h0, ws = ctx.saved_tensors
         dy = torch.zeros_like(x) if dy is None else dy.contiguous().to(x.dtype)
         dh_last = None if dh_last is None else dh_last.contiguous().float()
         grad = _GatedScanGrad.apply if torch.is_grad_enabled() else _gated_scan_bwd
-        return (*grad(dy, dh_last, *saved, ctx.desc), None)
+        dx, dgl, dlam, dz, dh0 = grad(dy, dh_last, x.contiguous(), gate_logits.contiguous(),
+                                      lam.contiguous().float(), z.contiguous(), h0, ws, ctx.desc)
+        return dx, dgl, dlam.to(lam.dtype), dz, dh0, None
 
 
 def _gated_scan_bwd(dy, dh_last, x, gate_logits, lam, z, h0, ws, desc):
@@ -178,13 +176,13 @@ def _own_product(T: int, n: int, k: int, forward: bool = False) -> bool:
     0.27 0.40 0.65 0.99 1.10, 1024 x 512 0.27 0.37 0.65 0.92 0.96, 2048 x 1024 0.21 0.35
     0.55 0.69 0.76. The forward alone keeps ahead longer, inner sums of up to 512 over
     enough outputs (3200 x 1024 x 256 1.24, 1600 x 1024 x 256 0.92, 6400 x 2048 x 512
-    1.07, 1600 x 1024 x 512 0.77, 51200 x 1024 x 1024 0.96). Launching one's forward and gradients takes torch 85 us, the
-    library 25, while 1 << 30 multiply-adds take 160 us on the device: a whole layer
-    of them no longer than the 545 us its other launches take. A captured graph pays
-    for no launch: there the device decides (a layer of 128 x 2 channels at 200 rows,
-    forward and backward: 205 us captured on the kernels, 115 on the products; eager
-    545 and 860), if a pass before the capture could set the products up: they
-    cannot be set up during one."""
+    1.07, 1600 x 1024 x 512 0.77, 51200 x 1024 x 1024 0.96). Launching one's forward and
+    gradients takes torch 85 us, the library 25, while 1 << 30 multiply-adds take 160 us
+    on the device: a whole layer of them no longer than the 545 us its other launches
+    take. A captured graph pays for no launch: there the device decides (a layer of
+    128 x 2 channels at 200 rows, forward and backward: 205 us captured on the kernels,
+    115 on the products; eager 545 and 860), if a pass before the capture could set the
+    products up: they cannot be set up during one."""
     return _own_products(T, ((n, k),), forward)[0]
 
 

@@ -121,3 +121,18 @@ def test_nans_stay_in_their_rows():
         assert nan.any() and torch.equal(torch.isnan(got).cpu(), nan)
         if not nan.all():
             close(got.detach()[~nan.cuda()], want[~nan], 5e-5)
+
+
+def test_compiled_layer():
+    """torch.compile breaks its graph at the scan and goes on: the eager layer's output
+    and gradients, from torch's operators around the scan (1e-5 as any of them)."""
+    from paper_2406_12580_gb300.layer import GatedRecurrentLayer
+    torch.manual_seed(15)
+    layer = GatedRecurrentLayer(16, device="cuda")
+    h = torch.randn(3, 40, 16, device="cuda", requires_grad=True)
+    both = []
+    for call in (layer, torch.compile(layer, backend="eager")):
+        y = call(h)
+        both.append((y, *torch.autograd.grad(y.square().sum(), [h, *layer.parameters()])))
+    for got, want in zip(*reversed(both)):
+        close(got, want.cpu(), 1e-5)
