@@ -64,13 +64,17 @@ def test_gradients_of_gradients():
         close(got, want, 1e-4)
 
 
-@pytest.mark.parametrize("captured", [False, True])
+@pytest.mark.parametrize("how", ["eager", "captured", "captured at once"])
 @pytest.mark.parametrize("B,L", [(2, 20), (35, 20), (33, 31), (60, 31)])
-def test_projections_by_either_product(B, L, captured):
-    """Captured, one, two or all of the layer's projections (128 x 32, 128 x 64, 32 x
-    64) run on the library's kernels and the others on torch's products, by the rows:
-    the output and every gradient. Five float32 stages of 1e-5 each."""
+def test_projections_by_either_product(monkeypatch, B, L, how):
+    """Captured after an eager pass, one, two or all of the layer's projections (128 x 32, 128 x 64, 32 x
+    64) run on the library's kernels and the others on torch's products, by the rows;
+    else all on the kernels: the output and every gradient. Five float32 stages of 1e-5 each."""
+    import threading
+
+    from paper_2406_12580_gb300 import layer as layer_module
     from paper_2406_12580_gb300.layer import GatedRecurrentLayer, _own_product
+    monkeypatch.setattr(layer_module, "_products", threading.local())
     torch.manual_seed(13)
     layer = GatedRecurrentLayer(32, device="cuda")
     h = torch.randn(B, L, 32, device="cuda", requires_grad=True)
@@ -80,15 +84,16 @@ def test_projections_by_either_product(B, L, captured):
         y = layer(h)
         assert "LayerF32" in type(y.grad_fn).__name__
         own = [_own_product(B * L, n, k) for n, k in ((128, 32), (128, 64), (32, 64))]
-        assert own == ([B * L >= 640, B * L >= 906, True] if captured else [True] * 3)
+        assert own == ([B * L >= 640, B * L >= 906, True] if how == "captured" else [True] * 3)
         return y, *torch.autograd.grad(y, [h, *layer.parameters()], dy)
 
-    if captured:
+    if how == "captured":
         side = torch.cuda.Stream()
         side.wait_stream(torch.cuda.current_stream())
         with torch.cuda.stream(side):
             layer(h).backward(dy)  # a capture follows an eager pass
         torch.cuda.current_stream().wait_stream(side)
+    if how != "eager":
         graph = torch.cuda.CUDAGraph()
         with torch.cuda.graph(graph):
             got = run()
