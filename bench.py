@@ -144,17 +144,17 @@ def kernel_sources_sha() -> str:
 def scan_kernels(cfg):
     """(forward kernels, backward kernels, our kernels per forward call, per
     backward call) the library runs on this shape: the serial kernels from 512
-    float32 (backward: 400) or 780 bfloat16 chains on (bfloat16 also from 304 where L
-    is at most 5/4 of their number), else the team kernels. (In their look-back order
-    a forward also clears its records with one cudaMemsetAsync, which is not counted
-    as a kernel of ours.)"""
+    float32 or 780 bfloat16 chains on (bfloat16 also from 304 where L is at most 5/4
+    of their number; float32 backwards of long rows from somewhat fewer, which no
+    workload has), else the team kernels. (In their look-back order a forward also
+    clears its records with one cudaMemsetAsync, which is not counted as a kernel of
+    ours.)"""
     f32 = cfg.io == "f32"
     width = 32 if f32 else 64
     chains = cfg.B * ((cfg.D + width - 1) // width)
     seq = chains >= (512 if f32 else 780) or (not f32 and chains >= 304 and 4 * cfg.L <= 5 * chains)
-    seq_bwd = seq or (f32 and chains >= 400)
-    return ("seq_fwd_kernel" if seq else "team_fwd_kernel",
-            "seq_bwd_kernel" if seq_bwd else "team_bwd_kernel", 1, 1)
+    family = "seq" if seq else "team"
+    return f"{family}_fwd_kernel", f"{family}_bwd_kernel", 1, 1
 
 
 def config_dict(cfg, world: int, l2: str) -> dict:

@@ -119,8 +119,8 @@ BLR_API size_t blr_workspace_bytes(const blr_desc* desc);
  *                         noticed: the backward's outputs are then undefined.)
  *   BLR_FAMILY_NONE       an invalid or empty problem (nothing is launched).
  * The kernels: from 512 float32 or 780 bfloat16 chains on (bfloat16 also from 304
- * where L is at most 5/4 of their number; a float32 backward without lengths from
- * 400) the serial ones, in which one warp walks each chain (bfloat16: each half of
+ * where L is at most 5/4 of their number; float32 backwards without lengths from
+ * 416 to 488, by L and D, where the rows are long) the serial ones, in which one warp walks each chain (bfloat16: each half of
  * it, where there are few) through the whole sequence. Elsewhere the team kernels:
  * teams of 8 warps scan tiles of up to 128 steps of a chain, 16 steps a warp, whole
  * chains at a time where there are enough of them, else tiles of all chains in

@@ -608,7 +608,7 @@ blr_status scan_bwd_entry(const blr_desc* desc, const void* dh, const float* dh_
 
   unsigned char* w = static_cast<unsigned char*>(ws);
   // the forward cleared the counters and partial sums
-  if (plan.seq || (plan.seq_bwd && !varlen))
+  if (varlen ? plan.seq : plan.seq_bwd[gated])
     return scan_bwd_seq(plan, dh, dh_last, x, gate_logits, lambda, h0, dx, dgate_logits, dlambda,
                         dh0, w, st, z, dz, lengths);
   return scan_bwd_team(plan, dh, dh_last, x, gate_logits, lambda, h0, dx, dgate_logits, dlambda,

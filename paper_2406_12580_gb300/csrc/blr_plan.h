@@ -64,16 +64,24 @@ constexpr int64_t kSeqTallRowsMinL = 1024;
 // above. Measured on GB300 (fwd + bwd, us, serial / team kernels): 600 chains x
 // 800 steps 119 / 124, x 3000 399 / 431, 400 x 3000 320 / 297, 512 x 2048 251 / 274.
 constexpr int64_t kSeqMinChainsF32 = 512;
-// The plain and gated backward from fewer on, on the states a team forward kept
-// (they lie the same way): the team backward takes two rounds of whole chains from
-// 305 to 608 of them however many, a serial one grows by the chain (backward, us,
-// serial / team, L = 50, 150, 400, 2000: 352 chains 9.7 / 11.0, 17.4 / 20.9, 31.2 /
-// 29.7, 126 / 119; 400 9.9 / 10.8, 17.0 / 20.5, 31.8 / 38.2, 130 / 134; 456 9.6 / 11.3,
-// 17.7 / 20.9, 32.7 / 39.1, 136 / 154; 511 9.9 / 12.5, 18.0 / 23.2, 33.2 / 42.1, 148 /
-// 171; the forward at 456 7.6 / 7.6, 9.2 / 10.1, 19.6 / 17.6, 81 / 82). Rows with
-// lengths share the teams' work better and stay with them (fwd + bwd 456 x 400
-// 51.2 / 47.8, x 2000 206 / 158).
-constexpr int64_t kSeqMinChainsBwdF32 = 400;
+// Its backward without lengths from somewhat fewer on, where the rows are long, on
+// the states a team forward kept (they lie the same way): the team backward takes
+// two rounds of whole chains from 305 to 608 of them however many, a serial one
+// grows by the chain. Rows whose last chain is not full, and wide ones, whose d Lambda
+// the serial kernel's last warp adds up by itself, stay with the teams (backward, us
+// over us, serial / team: D = 32, L = 800 430 chains 0.95, 460 0.90, 511 0.90, L =
+// 2000 0.94, 0.91, 0.87; D = 64 1.03, 0.96, 0.94 and 1.00, 0.95, 0.92; D = 128 1.04,
+// 1.00, 0.96 and 1.01, 0.96, 0.94; D = 256 1.15, 1.07, 1.06; D = 16 1.10, 1.03, 0.88 and
+// 1.25, 1.18, 1.10; L = 373 D = 32 1.07, 1.02, 1.02, D = 128 1.17, 1.09, 1.12. With the
+// merge D = 32, L = 800 416 chains 0.88, 488 0.81, D = 64 0.93, 0.85, D = 128 0.94, 0.87;
+// 488 chains, L = 400, 512, 700 D = 32 0.91, 0.86, 0.85, D = 64 0.95, 0.93, 0.90, D = 128
+// 0.99, 0.96, 0.94, at L = 420 1.03). Rows with lengths share the teams' work better
+// and stay with them (fwd + bwd 456 x 400 51.2 / 47.8 us, x 2000 206 / 158).
+inline bool plan_seq_bwd_f32(int64_t chains, int64_t L, int64_t D, bool gated) {
+  if (D % 32 != 0 || D > 128) return false;
+  if (gated) return (chains >= 416 && L >= 800) || (chains >= 488 && L >= (D <= 64 ? 385 : 512));
+  return chains >= 456 && L >= 800;
+}
 
 // Team kernels: kTeamWarps compute warps a block, in teams of kTeamWidth;
 // a warp takes kTeamSlice steps of a tile. The plan (and with it the workspace)
@@ -142,7 +150,7 @@ struct Plan {
   int io;           // 0 = float32, 1 = bfloat16
   float c;
   int seq;          // 1: serial kernels, 0: team kernels
-  int seq_bwd;      // 1: the serial backward all the same, without lengths
+  int seq_bwd[2];   // without lengths, plain and gated: 1: the serial backward all the same
   int sv;           // channels per lane (a chain is a row segment of 32 * sv channels)
   int rb;           // steps between the forward's kept states
   int sr, srb;      // serial: rows per TMA box, forward and backward (multiples of rb)
@@ -207,7 +215,8 @@ inline void make_plan(int64_t B, int64_t L, int64_t D, int io, float c, bool loc
   p->sv = io == 0 ? 1 : 2;
   p->n_chain = B * ((D + 32 * p->sv - 1) / (32 * p->sv));
   p->seq = io == 0 ? p->n_chain >= kSeqMinChainsF32 : plan_seq_bf16(p->n_chain, L);
-  p->seq_bwd = p->seq || (io == 0 && p->n_chain >= kSeqMinChainsBwdF32);
+  for (int g = 0; g < 2; ++g)
+    p->seq_bwd[g] = p->seq || (io == 0 && plan_seq_bwd_f32(p->n_chain, L, D, g != 0));
   p->segmented = p->n_chain < kManyChains && io == 1 && L >= kSegMinL &&
                  (B * L * D >= kSegMinElems || L >= kSegLongL);
   // Long float32 sequences stream the serial forward in 32-row boxes (fewer,

@@ -1,6 +1,7 @@
-"""GPU: scans whose forward and backward run in different forms. float32 ones whose forward runs on the team kernels and whose backward on the
-serial ones (400 to 511 chains), against the oracle: a step, a slice and its edges,
-tiles in the local order and with the look-back, channel tails."""
+"""GPU: scans whose forward and backward run in different forms, against the oracle:
+float32 ones whose forward runs on the team kernels and whose backward on the serial
+ones, on both sides of the lines between (tiles in the local order and with the
+look-back, whole and ragged last ones), and gated bfloat16 ones at the narrow form's."""
 import pytest
 
 from gpu_common import TOL, compare, gpu_outputs, gpu_scan, gpu_scan_gated, normwise, oracle_outputs
@@ -14,8 +15,9 @@ if not torch.cuda.is_available():
 
 
 @pytest.mark.parametrize("gated", [False, True])
-@pytest.mark.parametrize("B,L,D", [(400, 1, 32), (511, 16, 8), (200, 17, 64), (400, 129, 24),
-                                   (137, 300, 72), (450, 700, 32)])
+@pytest.mark.parametrize("B,L,D", [(455, 800, 32), (456, 799, 32), (456, 800, 32), (228, 801, 64),
+                                   (122, 1024, 128), (416, 800, 32), (488, 385, 32), (244, 400, 64),
+                                   (244, 384, 64), (460, 810, 24), (58, 800, 256)])
 def test_team_forward_serial_backward(B, L, D, gated):
     cfg = I.ScanConfig("mixed", io=I.F32, seed=B + L, gated=gated, B=B, L=L, D=D, random_h0=True,
                        random_dh_last=True)
