@@ -71,8 +71,8 @@ constexpr int64_t kSeqMinChainsF32 = 512;
 // the serial kernel's last warp adds up by itself, stay with the teams (backward, us
 // over us, serial / team: D = 32, L = 800 430 chains 0.95, 460 0.90, 511 0.90, L =
 // 2000 0.94, 0.91, 0.87; D = 64 1.03, 0.96, 0.94 and 1.00, 0.95, 0.92; D = 128 1.04,
-// 1.00, 0.96 and 1.01, 0.96, 0.94; D = 256 1.15, 1.07, 1.06; D = 16 1.10, 1.03, 0.88 and
-// 1.25, 1.18, 1.10; L = 373 D = 32 1.07, 1.02, 1.02, D = 128 1.17, 1.09, 1.12. With the
+// 1.00, 0.96 and 1.01, 0.96, 0.94; D = 256 1.15, 1.07, 1.06; D = 16 1.12, 1.03, 0.88 and
+// 1.25, 1.17, 1.08; L = 373 D = 32 1.07, 1.02, 1.02, D = 128 1.17, 1.09, 1.12. With the
 // merge D = 32, L = 800 416 chains 0.88, 488 0.81, D = 64 0.93, 0.85, D = 128 0.94, 0.87;
 // 488 chains, L = 400, 512, 700 D = 32 0.91, 0.86, 0.85, D = 64 0.95, 0.93, 0.90, D = 128
 // 0.99, 0.96, 0.94, at L = 420 1.03). Rows with lengths share the teams' work better
